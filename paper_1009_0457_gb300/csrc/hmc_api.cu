@@ -76,6 +76,8 @@ struct hmc_handle {
     int cur = 0;
     void *sig = nullptr, *ctab = nullptr, *wtab = nullptr, *atab = nullptr;
     float *cubw = nullptr;                // FP32 MPM step: Voigt weights of two crystal axes per orientation
+    int2 *cfix = nullptr;                 // FP64 MPM step: stiffness rows in fixed point
+    int cexp = 0;
     // 27-point zone (HMC_ELASTIC_ZONE1): trial list, start-of-step spins, element tables, schedule
     uint4 *zone_work = nullptr, *snap = nullptr;
     unsigned *zone_count = nullptr;
@@ -217,6 +219,32 @@ std::vector<T> pack_ctab(const std::vector<double> &Cv, int Q) {
     return out;
 }
 
+// The stiffness rows as 64-bit integers C' 2^cexp with every row's absolute sum below 2^63 (the
+// bound the fixed-point step's accumulators are laid out for), each split into a signed low and a
+// high 32-bit half.
+std::vector<int2> pack_cfix(const std::vector<double> &Cv, int Q, int &cexp) {
+    double top = 0;
+    for (size_t r = 0; r < (size_t)Q * 6; ++r) {
+        double s = 0;
+        for (int j = 0; j < 6; ++j) s += std::fabs(Cv[6 * r + j]);
+        top = std::fmax(top, s);
+    }
+    int er = 0;
+    std::frexp(top * (1.0 + 1e-9), &er);   // top < 2^er
+    cexp = 63 - er;
+    std::vector<int2> out((size_t)Q * 24, make_int2(0, 0));
+    for (int q = 0; q < Q; ++q) {
+        int n = 0;
+        for (int i = 0; i < 6; ++i)
+            for (int j = i; j < 6; ++j) {
+                const long long v = std::llrint(std::ldexp(Cv[(size_t)q * 36 + 6 * i + j], cexp));
+                const int lo = (int)(uint32_t)(v & 0xffffffffll);
+                out[(size_t)q * 24 + n++] = make_int2(lo, (int)((v - lo) >> 32));
+            }
+    }
+    return out;
+}
+
 template <typename T>
 std::vector<T> pack_wtab(const std::vector<double> &A, int Q) {
     std::vector<T> out((size_t)Q * 20, T(0));
@@ -260,8 +288,9 @@ hmc::MpmArgs<T> mpm_args(hmc_handle *h, const void *u_in, void *u_out, void *v) 
     a.u_in = static_cast<const T *>(u_in);
     a.u_out = static_cast<T *>(u_out);
     a.v = static_cast<T *>(v);
-    a.ctab = static_cast<const T *>(h->ctab);
     a.cubw = h->cubw;               // FP32 step: cubic form of Hooke's law
+    a.cfix = h->cfix;               // FP64 step: stiffness in fixed point
+    a.cexp = h->cexp;
     a.cub[0] = (float)h->p.c12;
     a.cub[1] = (float)(2.0 * h->p.c44);
     a.cub[2] = (float)h->p.c44;
@@ -524,7 +553,7 @@ void destroy_buffers(hmc_handle *h) {
     free_adjoint(h);
     for (int i = 0; i < 2; ++i)
         if (h->gexec[i]) cudaGraphExecDestroy(h->gexec[i]);
-    void *bufs[] = {h->spins, h->stage16, h->u[0], h->u[1], h->v, h->sig, h->ctab, h->cubw, h->wtab, h->atab, h->thr, h->counts,
+    void *bufs[] = {h->spins, h->stage16, h->u[0], h->u[1], h->v, h->sig, h->ctab, h->cubw, h->cfix, h->wtab, h->atab, h->thr, h->counts,
                     h->bins, h->partials, h->fractions, h->binmap, h->st, h->d_reps, h->d_cta_rep, h->d_sched,
                     h->zone_work, h->snap, h->zone_count, h->ktab, h->zone_sched, h->cc_parent, h->cc_count,
                     h->stab, h->plain_sig, h->plain_f};
@@ -971,17 +1000,20 @@ hmc_status hmc_create_batch(const hmc_params *params, int32_t n_replicas, hmc_ha
     }
     if ((e = cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking)) != cudaSuccess)
         return bail(cuda_fail(h, e, "capture stream create"));
-    if ((e = hmc::mpm_prepare()) != cudaSuccess) return bail(cuda_fail(h, e, "MPM kernel attribute"));
+    if ((e = hmc::mpm_prepare()) != cudaSuccess || (e = hmc::mpm64_prepare()) != cudaSuccess)
+        return bail(cuda_fail(h, e, "MPM kernel attribute"));
     if ((e = hmc::sweep_prepare()) != cudaSuccess) return bail(cuda_fail(h, e, "sweep kernel attribute"));
     struct Alloc { void **ptr; size_t bytes; const char *what; };
     const size_t nodes_b = node_bytes(h);
+    const bool fp32 = p->precision == HMC_FP32;
     Alloc allocs[] = {
         {(void **)&h->spins, sizeof(uint4) * (size_t)h->nblk_total, "spins"},
         {(void **)&h->stage16, sizeof(uint16_t) * (size_t)h->N_max, "spin staging"},
         {&h->u[0], nodes_b, "u0"}, {&h->u[1], nodes_b, "u1"}, {&h->v, nodes_b, "v"},
         {&h->sig, h->tsize * 48 * (size_t)h->nblk_total, "stress"},
         {&h->ctab, h->tsize * 24 * (size_t)p->n_orient, "stiffness table"},
-        {(void **)&h->cubw, sizeof(float) * 12 * (size_t)p->n_orient, "cubic axis table"},
+        {(void **)&h->cubw, fp32 ? sizeof(float) * 12 * (size_t)p->n_orient : 16, "cubic axis table"},
+        {(void **)&h->cfix, fp32 ? 16 : sizeof(int2) * 24 * (size_t)p->n_orient, "fixed-point stiffness table"},
         {&h->wtab, h->tsize * 20 * (size_t)p->n_orient, "axis weight table"},
         {&h->atab, h->tsize * 8 * (size_t)p->n_orient, "axis table"},
         {(void **)&h->thr, sizeof(unsigned long long) * 8, "threshold table"},
@@ -1207,6 +1239,8 @@ hmc_status hmc_set_orientations(hmc_handle *h, const double *euler, const uint16
         auto c = pack_ctab<double>(h->Cv, Q);
         auto w = pack_wtab<double>(h->A, Q);
         auto ax = pack_atab<double>(h->A, Q);
+        auto cf = pack_cfix(h->Cv, Q, h->cexp);
+        HMC_CK(h, cudaMemcpy(h->cfix, cf.data(), cf.size() * sizeof(int2), cudaMemcpyHostToDevice), "table upload");
         HMC_CK(h, cudaMemcpy(h->ctab, c.data(), c.size() * sizeof(double), cudaMemcpyHostToDevice), "table upload");
         HMC_CK(h, cudaMemcpy(h->wtab, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice), "table upload");
         HMC_CK(h, cudaMemcpy(h->atab, ax.data(), ax.size() * sizeof(double), cudaMemcpyHostToDevice), "table upload");

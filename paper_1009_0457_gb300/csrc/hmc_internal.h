@@ -18,6 +18,8 @@
 //                               energy)
 //   cubw    float[Q][12]        FP32 MPM step: the Voigt weights (x^2, y^2, z^2, yz,
 //                               xz, xy) of the first two crystal axes a_0, a_1
+//   cfix    int2[Q][24]         FP64 MPM step: C'(q) as 64-bit integers C' 2^cexp, each as
+//                               signed 32-bit halves (x low, y high)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -105,9 +107,10 @@ struct MpmArgs {
     const T *u_in;
     T *u_out;
     T *v;
-    const T *ctab;           // FP64 step: rotated stiffness rows
     const float *cubw;       // FP32 step: Voigt weights of two crystal axes per orientation (12 each)
     float cub[4];            // FP32 step: C12, 2 C44, C44 and C11 - C12 - 2 C44
+    const int2 *cfix;        // FP64 step: rotated stiffness in fixed point, 24 entries per orientation (21 used)
+    int cexp;                // ... entry = round(C' 2^cexp), x the signed low half, y the high half
     int nq;                  // orientations (the FP32 step stages cubw in shared memory up to MPM_STAB_MAX)
     T dt, dt_over_m, keep;   // keep = 1 - damping
     int grid;                // persistent CTAs
@@ -232,6 +235,7 @@ std::vector<uint16_t> zone_schedule();   // empty if it does not fit the kernel'
 std::vector<uint16_t> zone_scatter_table(const std::vector<uint16_t> &schedule);
 void zone_element_tables(const double *Cv, int Q, std::vector<double> &out);
 cudaError_t mpm_prepare();  // opt the MPM kernels into their dynamic shared memory (once, before any capture)
+cudaError_t mpm64_prepare();  // ... those of the FP64 step
 cudaError_t sweep_prepare();  // opt the elastic sweeps into their shared memory
 template <typename T>
 int mpm_per_sm(int variant, int nq);  // resident MPM CTAs per SM

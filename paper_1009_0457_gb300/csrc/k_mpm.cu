@@ -1,4 +1,4 @@
-// Fused explicit MPM step (Sec. "Elastic Deformation"): for every material
+// Fused explicit MPM step in FP32 (Sec. "Elastic Deformation"): for every material
 // point strain from the nodal displacement, Hooke's law (Eq. 1) with the
 // point's rotated stiffness, internal nodal force, then the damped
 // velocity / displacement update of every node -- one kernel, one pass over
@@ -38,35 +38,33 @@ namespace {
 // A node's or a cell corner's three components and a pad: one 16-byte shared-memory access
 // in FP32 (eight consecutive lanes read 128 contiguous bytes, free of bank conflicts)
 // instead of three 4-byte ones.
-template <typename T>
 struct alignas(16) Vec4 {
-    T x, y, z, p;
+    float x, y, z, p;
 };
 
 template <int CX, int CY>
 struct MpmSmem {
     static constexpr int NX = CX + 1, NY = CY + 1;   // node tile (one node of halo each side)
-    template <typename T>
     struct S {
-        Vec4<T> us[3][NY][NX];  // node planes (buffer, j, i), held as u/32
-        Vec4<T> fb[4][CY][CX];  // cell contributions to their lower corner nodes (corner I+2J)
-        Vec4<T> ft[4][CY][CX];  // ... to their upper corner nodes
+        Vec4 us[3][NY][NX];  // node planes (buffer, j, i), held as u/32
+        Vec4 fb[4][CY][CX];  // cell contributions to their lower corner nodes (corner I+2J)
+        Vec4 ft[4][CY][CX];  // ... to their upper corner nodes
     };
 };
 
 // byte offset of the FP32 orientation table behind a CTA's tiles (16-byte aligned)
-template <int CX, int CY, typename T>
+template <int CX, int CY>
 __host__ __device__ constexpr size_t mpm_table_offset() {
-    return (sizeof(typename MpmSmem<CX, CY>::template S<T>) + 15) & ~size_t(15);
+    return (sizeof(typename MpmSmem<CX, CY>::S) + 15) & ~size_t(15);
 }
 
 // Node plane k of the tile with origin (i0, j0) (one node of halo on each side),
 // read from global memory into registers / written to shared memory.
-template <typename T, int CX, int CY>
+template <int CX, int CY>
 struct PlaneLoad {
     static constexpr int NX = CX + 1, NY = CY + 1, NN = NX * NY, NTHR = CX * CY;
     static constexpr int PER = (NN + NTHR - 1) / NTHR;
-    T r[PER][3];
+    float r[PER][3];
     int col[PER];   // this thread's tile nodes as (i + nbx j) in the replica's node plane
     // once per tile: the periodic (i, j) of each node this thread loads
     __device__ __forceinline__ void prepare(int i0, int j0, int nbx, int nby) {
@@ -78,32 +76,31 @@ struct PlaneLoad {
         }
     }
     // node plane k, -1 <= k <= nbz (periodic in z)
-    __device__ __forceinline__ void fetch(const T *__restrict__ u, long long node0, int k, int nbz, int plane) {
+    __device__ __forceinline__ void fetch(const float *__restrict__ u, long long node0, int k, int nbz, int plane) {
         const int gk = k < 0 ? k + nbz : (k >= nbz ? k - nbz : k);
-        const T *base = u + 3 * (node0 + (long long)plane * gk);
+        const float *base = u + 3 * (node0 + (long long)plane * gk);
 #pragma unroll
         for (int m = 0; m < PER; ++m) {
             const int t = threadIdx.x + m * NTHR;
             if (t < NN) {
-                const T *p = base + 3 * col[m];
+                const float *p = base + 3 * col[m];
                 r[m][0] = __ldg(p);
                 r[m][1] = __ldg(p + 1);
                 r[m][2] = __ldg(p + 2);
             }
         }
     }
-    __device__ __forceinline__ void store(Vec4<T> (&us)[NY][NX]) const {
+    __device__ __forceinline__ void store(Vec4 (&us)[NY][NX]) const {
 #pragma unroll
         for (int m = 0; m < PER; ++m) {
             const int t = threadIdx.x + m * NTHR;
             if (t < NN)   // node (t % NX, t / NX) of the row-major tile
-                (&us[0][0])[t] = Vec4<T>{r[m][0] * T(0.03125), r[m][1] * T(0.03125), r[m][2] * T(0.03125), T(0)};
+                (&us[0][0])[t] = Vec4{r[m][0] * 0.03125f, r[m][1] * 0.03125f, r[m][2] * 0.03125f, 0.f};
         }
     }
 };
 
-// Hooke's law for the MPM step.  FP64: the 21-entry symmetric row of C'(q).  FP32:
-// the cubic form of one rotated cubic material,
+// Hooke's law for the MPM step: the cubic form of one rotated cubic material,
 //   sigma = (C12 tr + Ad p2) I + 2 C44 eps + Ad (p0 - p2) a0 a0 + Ad (p1 - p2) a1 a1,
 //   p_m = a_m.eps.a_m = W_m.e,  p2 = tr - p0 - p1,  Ad = C11 - C12 - 2 C44,
 // with e the Voigt strain (engineering shear), sigma in tensor shear and W_m the Voigt
@@ -161,19 +158,11 @@ __device__ __forceinline__ void cubic_hooke_paired(const float (&w)[12], const f
     }
 }
 
-template <typename T, bool PAIR, bool STAB>
-struct HookeRow {
-    Row24<T> r;
-    __device__ __forceinline__ void load(const T *tab, const float *, uint32_t q) { r.load(tab + 24ll * q); }
-    __device__ __forceinline__ void apply(const T (&e)[6], T (&s)[6], const float (&)[4]) const {
-        hooke21<T>(r.v, e, s);
-    }
-};
 template <bool PAIR, bool STAB>
-struct HookeRow<float, PAIR, STAB> {
+struct HookeRow {
     float w[12];
     // cw: the table in shared memory (STAB) or in global memory
-    __device__ __forceinline__ void load(const float *, const float *cw, uint32_t q) {
+    __device__ __forceinline__ void load(const float *cw, uint32_t q) {
         const float4 *p = reinterpret_cast<const float4 *>(cw + 12 * q);
         float4 v[3];
 #pragma unroll
@@ -193,36 +182,34 @@ struct HookeRow<float, PAIR, STAB> {
 
 // 2x2 -> 2x2 transform with weights 3 (same side) and 1 (other side) in both
 // indices: o[b][c] = sum_J sum_K W(J,b) W(K,c) d[J][K], eight FMAs.
-template <typename T>
-__device__ __forceinline__ void interp31(T d00, T d10, T d01, T d11, T (&o)[2][2]) {
-    const T e00 = fma(T(3), d00, d10), e10 = fma(T(3), d10, d00);  // (b, K=0)
-    const T e01 = fma(T(3), d01, d11), e11 = fma(T(3), d11, d01);  // (b, K=1)
-    o[0][0] = fma(T(3), e00, e01);
-    o[0][1] = fma(T(3), e01, e00);
-    o[1][0] = fma(T(3), e10, e11);
-    o[1][1] = fma(T(3), e11, e10);
+__device__ __forceinline__ void interp31(float d00, float d10, float d01, float d11, float (&o)[2][2]) {
+    const float e00 = fma(3.f, d00, d10), e10 = fma(3.f, d10, d00);  // (b, K=0)
+    const float e01 = fma(3.f, d01, d11), e11 = fma(3.f, d11, d01);  // (b, K=1)
+    o[0][0] = fma(3.f, e00, e01);
+    o[0][1] = fma(3.f, e01, e00);
+    o[1][0] = fma(3.f, e10, e11);
+    o[1][1] = fma(3.f, e11, e10);
 }
 
 // Displacement gradients of the cell's points from corner displacements held
 // as u/32: the 3/1 weights then give (1/h) sum w w (difference) exactly.
-template <typename T>
-__device__ __forceinline__ void cell_gradients31(const T (&u)[8][3], CellGrad<T> &g) {
+__device__ __forceinline__ void cell_gradients31(const float (&u)[8][3], CellGrad<float> &g) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        T o[2][2];
-        interp31<T>(u[corner(1, 0, 0)][d] - u[corner(0, 0, 0)][d], u[corner(1, 1, 0)][d] - u[corner(0, 1, 0)][d],
+        float o[2][2];
+        interp31(u[corner(1, 0, 0)][d] - u[corner(0, 0, 0)][d], u[corner(1, 1, 0)][d] - u[corner(0, 1, 0)][d],
                     u[corner(1, 0, 1)][d] - u[corner(0, 0, 1)][d], u[corner(1, 1, 1)][d] - u[corner(0, 1, 1)][d], o);
 #pragma unroll
         for (int b = 0; b < 2; ++b)
 #pragma unroll
             for (int c = 0; c < 2; ++c) g.gx[b][c][d] = o[b][c];
-        interp31<T>(u[corner(0, 1, 0)][d] - u[corner(0, 0, 0)][d], u[corner(1, 1, 0)][d] - u[corner(1, 0, 0)][d],
+        interp31(u[corner(0, 1, 0)][d] - u[corner(0, 0, 0)][d], u[corner(1, 1, 0)][d] - u[corner(1, 0, 0)][d],
                     u[corner(0, 1, 1)][d] - u[corner(0, 0, 1)][d], u[corner(1, 1, 1)][d] - u[corner(1, 0, 1)][d], o);
 #pragma unroll
         for (int a = 0; a < 2; ++a)
 #pragma unroll
             for (int c = 0; c < 2; ++c) g.gy[a][c][d] = o[a][c];
-        interp31<T>(u[corner(0, 0, 1)][d] - u[corner(0, 0, 0)][d], u[corner(1, 0, 1)][d] - u[corner(1, 0, 0)][d],
+        interp31(u[corner(0, 0, 1)][d] - u[corner(0, 0, 0)][d], u[corner(1, 0, 1)][d] - u[corner(1, 0, 0)][d],
                     u[corner(0, 1, 1)][d] - u[corner(0, 1, 0)][d], u[corner(1, 1, 1)][d] - u[corner(1, 1, 0)][d], o);
 #pragma unroll
         for (int a = 0; a < 2; ++a)
@@ -243,17 +230,17 @@ __host__ __device__ constexpr int gray_point(int n) {
 // Eight points of one cell: F[corner] = (2I-1) X'[J][K] + (2J-1) Y'[I][K] +
 // (2K-1) Z'[I][J] with X', Y', Z' the 3/1-weighted sums of the traction
 // columns of sigma; the nodal force is -(V/h)/16 F = -F/32 (V = 1 voxel, h = 2).
-template <typename T, bool PAIR, bool STAB>
-__device__ __forceinline__ void cell_forces(const T (&u)[8][3], const uint4 &sp, const T *__restrict__ ctab,
-                                            const float *cw, const float (&cub)[4], const T (&eb)[6],
-                                            T (&f)[8][3]) {
+template <bool PAIR, bool STAB>
+__device__ __forceinline__ void cell_forces(const float (&u)[8][3], const uint4 &sp,
+                                            const float *cw, const float (&cub)[4], const float (&eb)[6],
+                                            float (&f)[8][3]) {
     // the first point's stiffness row is requested before the gradients are formed, so that
     // its load latency overlaps them
-    HookeRow<T, PAIR, STAB> row;
+    HookeRow<PAIR, STAB> row;
     uint32_t qprev = spin_of(sp, local_slot(0));
-    row.load(ctab, cw, qprev);
-    CellGrad<T> g;
-    cell_gradients31<T>(u, g);
+    row.load(cw, qprev);
+    CellGrad<float> g;
+    cell_gradients31(u, g);
     // each strain component of a point is eb_k plus gradient entries that two points share:
     // add eb_k once to the one entry of each component that only that component uses (the
     // normal entries, and one of the two entries of each shear)
@@ -268,18 +255,18 @@ __device__ __forceinline__ void cell_forces(const T (&u)[8][3], const uint4 &sp,
             g.gz[i][j][0] = eb[4] + g.gz[i][j][0];
             g.gy[i][j][0] = eb[5] + g.gy[i][j][0];
         }
-    T tx[2][2][3], ty[2][2][3], tz[2][2][3];  // traction sums over a, b, c respectively
+    float tx[2][2][3], ty[2][2][3], tz[2][2][3];  // traction sums over a, b, c respectively
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int d = 0; d < 3; ++d) tx[i][j][d] = ty[i][j][d] = tz[i][j][d] = T(0);
+            for (int d = 0; d < 3; ++d) tx[i][j][d] = ty[i][j][d] = tz[i][j][d] = 0.f;
 #pragma unroll
     for (int n = 0; n < 8; ++n) {
         const int L = gray_point(n);
         const int a = L & 1, b = (L >> 1) & 1, c = L >> 2;
-        T e[6], s[6];
+        float e[6], s[6];
         e[0] = g.gx[b][c][0];
         e[1] = g.gy[a][c][1];
         e[2] = g.gz[a][b][2];
@@ -289,7 +276,7 @@ __device__ __forceinline__ void cell_forces(const T (&u)[8][3], const uint4 &sp,
         // points of one cell mostly share one orientation: fetch the row only when it changes
         const uint32_t q = spin_of(sp, local_slot(L));
         if (q != qprev) {
-            row.load(ctab, cw, q);
+            row.load(cw, q);
             qprev = q;
         }
         row.apply(e, s, cub);
@@ -300,39 +287,39 @@ __device__ __forceinline__ void cell_forces(const T (&u)[8][3], const uint4 &sp,
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        T X[2][2], Y[2][2], Z[2][2];
-        interp31<T>(tx[0][0][d], tx[1][0][d], tx[0][1][d], tx[1][1][d], X);  // X[J][K]
-        interp31<T>(ty[0][0][d], ty[1][0][d], ty[0][1][d], ty[1][1][d], Y);  // Y[I][K]
-        interp31<T>(tz[0][0][d], tz[1][0][d], tz[0][1][d], tz[1][1][d], Z);  // Z[I][J]
+        float X[2][2], Y[2][2], Z[2][2];
+        interp31(tx[0][0][d], tx[1][0][d], tx[0][1][d], tx[1][1][d], X);  // X[J][K]
+        interp31(ty[0][0][d], ty[1][0][d], ty[0][1][d], ty[1][1][d], Y);  // Y[I][K]
+        interp31(tz[0][0][d], tz[1][0][d], tz[0][1][d], tz[1][1][d], Z);  // Z[I][J]
 #pragma unroll
         for (int K = 0; K < 2; ++K)
 #pragma unroll
             for (int J = 0; J < 2; ++J)
 #pragma unroll
                 for (int I = 0; I < 2; ++I) {
-                    const T fx = I ? X[J][K] : -X[J][K];
-                    const T fy = J ? Y[I][K] : -Y[I][K];
-                    const T fz = K ? Z[I][J] : -Z[I][J];
+                    const float fx = I ? X[J][K] : -X[J][K];
+                    const float fy = J ? Y[I][K] : -Y[I][K];
+                    const float fz = K ? Z[I][J] : -Z[I][J];
                     f[corner(I, J, K)][d] = fx + fy + fz;
                 }
     }
 }
 
-template <typename T, int CX, int CY, bool PAIR, bool STAB>
-__global__ void __launch_bounds__(CX *CY, (sizeof(T) == 4 ? 2 : 1)) k_mpm_step(MpmArgs<T> a) {
+template <int CX, int CY, bool PAIR, bool STAB>
+__global__ void __launch_bounds__(CX *CY, 2) k_mpm_step(MpmArgs<float> a) {
     constexpr int OX = CX - 1, OY = CY - 1;
-    using Smem = typename MpmSmem<CX, CY>::template S<T>;
+    using Smem = typename MpmSmem<CX, CY>::S;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
     const int tid = threadIdx.x;
-    const T fscale = -a.dt_over_m * T(0.03125);          // -dt / (32 m)
+    const float fscale = -a.dt_over_m * 0.03125f;          // -dt / (32 m)
     // the next step may be launched now: its CTAs take the SM slots this grid's CTAs free
     // and stage their table while this grid finishes
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // FP32: the orientation table of the cubic form, staged in shared memory behind the tiles
     const float *cw = a.cubw;
     if constexpr (STAB) {
-        float *ts = reinterpret_cast<float *>(smem_raw + mpm_table_offset<CX, CY, T>());
+        float *ts = reinterpret_cast<float *>(smem_raw + mpm_table_offset<CX, CY>());
         for (int i = tid; i < 3 * a.nq; i += CX * CY)
             reinterpret_cast<float4 *>(ts)[i] = __ldg(reinterpret_cast<const float4 *>(a.cubw) + i);
         __syncthreads();
@@ -370,10 +357,10 @@ __global__ void __launch_bounds__(CX *CY, (sizeof(T) == 4 ? 2 : 1)) k_mpm_step(M
         const int gi = wrapi(ni, nbx), gj = wrapi(nj, nby);
         const int plane = nbx * nby;
         const long long col = R.blk_off + gi + nbx * gj;    // (i, j) column of this cell and node in the batch
-        T eb[6];
-        load_ebar<T>(R.st, eb);
+        float eb[6];
+        load_ebar<float>(R.st, eb);
 
-        PlaneLoad<T, CX, CY> pl;
+        PlaneLoad<CX, CY> pl;
         int b0 = 0, b1 = 1, b2 = 2;
         pl.prepare(i0, j0, nbx, nby);
         pl.fetch(a.u_in, R.blk_off, k0 - 1, nbz, plane);
@@ -383,19 +370,19 @@ __global__ void __launch_bounds__(CX *CY, (sizeof(T) == 4 ? 2 : 1)) k_mpm_step(M
         uint4 sp = need ? __ldg(a.spins + col + (long long)plane * wrapi(k0 - 1, nbz)) : make_uint4(0, 0, 0, 0);
         __syncthreads();
 
-        T acc[3] = {T(0), T(0), T(0)};
+        float acc[3] = {0.f, 0.f, 0.f};
         // this column's spins of the next plane, and its node's velocity and new displacement in
         // the current plane, advanced by one plane per iteration
         const uint4 *spn = a.spins + col + (long long)plane * k0;
-        T *vp = a.v + 3 * (col + (long long)plane * k0);
-        T *up = a.u_out + 3 * (col + (long long)plane * k0);
+        float *vp = a.v + 3 * (col + (long long)plane * k0);
+        float *up = a.u_out + 3 * (col + (long long)plane * k0);
         const long long pstride = 3ll * plane;
         for (int kk = k0 - 1; kk < kend; ++kk) {
             // one plane ahead: next plane's spins and u, this plane's owned velocity
             uint4 sp_next = make_uint4(0, 0, 0, 0);
             if (need && kk + 1 < kend) sp_next = __ldg(spn);
             spn += plane;
-            T vold[3] = {T(0), T(0), T(0)};
+            float vold[3] = {0.f, 0.f, 0.f};
             if (own && kk >= k0) {
 #pragma unroll
                 for (int d = 0; d < 3; ++d) vold[d] = vp[d];
@@ -403,27 +390,27 @@ __global__ void __launch_bounds__(CX *CY, (sizeof(T) == 4 ? 2 : 1)) k_mpm_step(M
             const bool more = kk + 1 < kend;
             if (more) pl.fetch(a.u_in, R.blk_off, kk + 2, nbz, plane);
             if (need) {
-                T u[8][3];
+                float u[8][3];
 #pragma unroll
                 for (int K = 0; K < 2; ++K)
 #pragma unroll
                     for (int J = 0; J < 2; ++J)
 #pragma unroll
                         for (int I = 0; I < 2; ++I) {
-                            const Vec4<T> n = sm.us[K ? b1 : b0][lcj + J][lci + I];
+                            const Vec4 n = sm.us[K ? b1 : b0][lcj + J][lci + I];
                             u[corner(I, J, K)][0] = n.x;
                             u[corner(I, J, K)][1] = n.y;
                             u[corner(I, J, K)][2] = n.z;
                         }
-                T f[8][3];
-                cell_forces<T, PAIR, STAB>(u, sp, a.ctab, cw, cub, eb, f);
+                float f[8][3];
+                cell_forces<PAIR, STAB>(u, sp, cw, cub, eb, f);
 #pragma unroll
                 for (int J = 0; J < 2; ++J)
 #pragma unroll
                     for (int I = 0; I < 2; ++I) {
-                        const T *fl = f[corner(I, J, 0)], *fu = f[corner(I, J, 1)];
-                        sm.fb[I + 2 * J][lcj][lci] = Vec4<T>{fl[0], fl[1], fl[2], T(0)};
-                        sm.ft[I + 2 * J][lcj][lci] = Vec4<T>{fu[0], fu[1], fu[2], T(0)};
+                        const float *fl = f[corner(I, J, 0)], *fu = f[corner(I, J, 1)];
+                        sm.fb[I + 2 * J][lcj][lci] = Vec4{fl[0], fl[1], fl[2], 0.f};
+                        sm.ft[I + 2 * J][lcj][lci] = Vec4{fu[0], fu[1], fu[2], 0.f};
                     }
             }
             if (more) pl.store(sm.us[b2]);   // buffer b2 was last read before the previous barrier
@@ -431,23 +418,23 @@ __global__ void __launch_bounds__(CX *CY, (sizeof(T) == 4 ? 2 : 1)) k_mpm_step(M
             if (own) {
                 // cells (lci-1, lcj-1), (lci, lcj-1), (lci-1, lcj), (lci, lcj) see this node as corner 3, 2, 1, 0
                 if (kk >= k0) {
-                    const Vec4<T> c3 = sm.fb[3][lcj - 1][lci - 1], c2 = sm.fb[2][lcj - 1][lci];
-                    const Vec4<T> c1 = sm.fb[1][lcj][lci - 1], c0 = sm.fb[0][lcj][lci];
-                    const Vec4<T> un = sm.us[b0][lcj][lci];
-                    const T F[3] = {acc[0] + c3.x + c2.x + c1.x + c0.x, acc[1] + c3.y + c2.y + c1.y + c0.y,
+                    const Vec4 c3 = sm.fb[3][lcj - 1][lci - 1], c2 = sm.fb[2][lcj - 1][lci];
+                    const Vec4 c1 = sm.fb[1][lcj][lci - 1], c0 = sm.fb[0][lcj][lci];
+                    const Vec4 un = sm.us[b0][lcj][lci];
+                    const float F[3] = {acc[0] + c3.x + c2.x + c1.x + c0.x, acc[1] + c3.y + c2.y + c1.y + c0.y,
                                     acc[2] + c3.z + c2.z + c1.z + c0.z};
-                    const T uc[3] = {un.x, un.y, un.z};
+                    const float uc[3] = {un.x, un.y, un.z};
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
-                        const T vn = rfma(fscale, F[d], rmul(a.keep, vold[d]));
+                        const float vn = rfma(fscale, F[d], rmul(a.keep, vold[d]));
                         vp[d] = vn;
-                        up[d] = rfma(a.dt, vn, uc[d] * T(32));
+                        up[d] = rfma(a.dt, vn, uc[d] * 32.f);
                     }
                     vp += pstride;
                     up += pstride;
                 }
-                const Vec4<T> c3 = sm.ft[3][lcj - 1][lci - 1], c2 = sm.ft[2][lcj - 1][lci];
-                const Vec4<T> c1 = sm.ft[1][lcj][lci - 1], c0 = sm.ft[0][lcj][lci];
+                const Vec4 c3 = sm.ft[3][lcj - 1][lci - 1], c2 = sm.ft[2][lcj - 1][lci];
+                const Vec4 c1 = sm.ft[1][lcj][lci - 1], c0 = sm.ft[0][lcj][lci];
                 acc[0] = c3.x + c2.x + c1.x + c0.x;
                 acc[1] = c3.y + c2.y + c1.y + c0.y;
                 acc[2] = c3.z + c2.z + c1.z + c0.z;
@@ -798,10 +785,10 @@ __global__ void __launch_bounds__(128, 2) k_mpm_step2(MpmArgs<float> a) {
     }
 }
 
-template <typename T, int CX, int CY>
+template <int CX, int CY>
 size_t smem_of(bool stab, int nq) {
-    return stab ? mpm_table_offset<CX, CY, T>() + sizeof(float) * 12 * (size_t)nq
-                : sizeof(typename MpmSmem<CX, CY>::template S<T>);
+    return stab ? mpm_table_offset<CX, CY>() + sizeof(float) * 12 * (size_t)nq
+                : sizeof(typename MpmSmem<CX, CY>::S);
 }
 
 }  // namespace
@@ -809,18 +796,18 @@ size_t smem_of(bool stab, int nq) {
 int mpm_shape_cx(int shape) { return shape == MPM_32x8 ? 32 : shape == MPM_8x32 ? 8 : 16; }
 int mpm_shape_cy(int shape) { return shape == MPM_32x8 ? 8 : shape == MPM_8x32 ? 32 : 16; }
 
-template <typename T, int CX, int CY, bool PAIR, bool STAB>
+template <int CX, int CY, bool PAIR, bool STAB>
 static cudaError_t set_attr() {
-    return cudaFuncSetAttribute(k_mpm_step<T, CX, CY, PAIR, STAB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_of<T, CX, CY>(STAB, MPM_STAB_MAX));
+    return cudaFuncSetAttribute(k_mpm_step<CX, CY, PAIR, STAB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)smem_of<CX, CY>(STAB, MPM_STAB_MAX));
 }
 
 template <bool PAIR, bool STAB>
 static cudaError_t set_attr_f32() {
     cudaError_t e;
-    if ((e = set_attr<float, 16, 16, PAIR, STAB>()) != cudaSuccess) return e;
-    if ((e = set_attr<float, 32, 8, PAIR, STAB>()) != cudaSuccess) return e;
-    return set_attr<float, 8, 32, PAIR, STAB>();
+    if ((e = set_attr<16, 16, PAIR, STAB>()) != cudaSuccess) return e;
+    if ((e = set_attr<32, 8, PAIR, STAB>()) != cudaSuccess) return e;
+    return set_attr<8, 32, PAIR, STAB>();
 }
 
 cudaError_t mpm_prepare() {
@@ -829,27 +816,24 @@ cudaError_t mpm_prepare() {
                                   (int)sizeof(MpmSmem2))) != cudaSuccess)
         return e;
     if ((e = set_attr_f32<false, false>()) != cudaSuccess || (e = set_attr_f32<false, true>()) != cudaSuccess ||
-        (e = set_attr_f32<true, false>()) != cudaSuccess || (e = set_attr_f32<true, true>()) != cudaSuccess ||
-        (e = set_attr<double, 16, 16, false, false>()) != cudaSuccess ||
-        (e = set_attr<double, 32, 8, false, false>()) != cudaSuccess ||
-        (e = set_attr<double, 8, 32, false, false>()) != cudaSuccess)
+        (e = set_attr_f32<true, false>()) != cudaSuccess || (e = set_attr_f32<true, true>()) != cudaSuccess)
         return e;
     return cudaSuccess;
 }
 
-template <typename T, bool PAIR, bool STAB>
+template <bool PAIR, bool STAB>
 static int per_sm_t(int shape, int nq) {
     int n = 1;
     cudaError_t e;
     if (shape == MPM_32x8)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_mpm_step<T, 32, 8, PAIR, STAB>, 256,
-                                                          smem_of<T, 32, 8>(STAB, nq));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_mpm_step<32, 8, PAIR, STAB>, 256,
+                                                          smem_of<32, 8>(STAB, nq));
     else if (shape == MPM_8x32)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_mpm_step<T, 8, 32, PAIR, STAB>, 256,
-                                                          smem_of<T, 8, 32>(STAB, nq));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_mpm_step<8, 32, PAIR, STAB>, 256,
+                                                          smem_of<8, 32>(STAB, nq));
     else
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_mpm_step<T, 16, 16, PAIR, STAB>, 256,
-                                                          smem_of<T, 16, 16>(STAB, nq));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_mpm_step<16, 16, PAIR, STAB>, 256,
+                                                          smem_of<16, 16>(STAB, nq));
     return (e != cudaSuccess || n < 1) ? 1 : n;
 }
 
@@ -864,40 +848,36 @@ int mpm_per_sm<float>(int shape, int nq) {
     const int sh = shape % MPM_NSHAPES;
     int a, b;
     if (nq <= MPM_STAB_MAX) {
-        a = per_sm_t<float, false, true>(sh, nq);
-        b = per_sm_t<float, true, true>(sh, nq);
+        a = per_sm_t<false, true>(sh, nq);
+        b = per_sm_t<true, true>(sh, nq);
     } else {
-        a = per_sm_t<float, false, false>(sh, nq);
-        b = per_sm_t<float, true, false>(sh, nq);
+        a = per_sm_t<false, false>(sh, nq);
+        b = per_sm_t<true, false>(sh, nq);
     }
     return a < b ? a : b;
-}
-template <>
-int mpm_per_sm<double>(int shape, int nq) {
-    return per_sm_t<double, false, false>(shape % MPM_NSHAPES, nq);
 }
 
 // launched with programmatic stream serialisation: the kernel waits for the grid before it
 // (griddepcontrol.wait) only after its prologue
-template <typename T, int CX, int CY, bool PAIR, bool STAB>
-static cudaError_t launch_pdl(const MpmArgs<T> &a, cudaStream_t s) {
+template <int CX, int CY, bool PAIR, bool STAB>
+static cudaError_t launch_pdl(const MpmArgs<float> &a, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.grid);
     cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = smem_of<T, CX, CY>(STAB, a.nq);
+    cfg.dynamicSmemBytes = smem_of<CX, CY>(STAB, a.nq);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_mpm_step<T, CX, CY, PAIR, STAB>, a);
+    return cudaLaunchKernelEx(&cfg, k_mpm_step<CX, CY, PAIR, STAB>, a);
 }
-template <typename T, bool PAIR, bool STAB>
-static cudaError_t launch_t(const MpmArgs<T> &a, int shape, cudaStream_t s) {
-    if (shape == MPM_32x8) return launch_pdl<T, 32, 8, PAIR, STAB>(a, s);
-    if (shape == MPM_8x32) return launch_pdl<T, 8, 32, PAIR, STAB>(a, s);
-    return launch_pdl<T, 16, 16, PAIR, STAB>(a, s);
+template <bool PAIR, bool STAB>
+static cudaError_t launch_t(const MpmArgs<float> &a, int shape, cudaStream_t s) {
+    if (shape == MPM_32x8) return launch_pdl<32, 8, PAIR, STAB>(a, s);
+    if (shape == MPM_8x32) return launch_pdl<8, 32, PAIR, STAB>(a, s);
+    return launch_pdl<16, 16, PAIR, STAB>(a, s);
 }
 
 // shape in 0..2: scalar Hooke; shape + MPM_NSHAPES: paired-FMA Hooke (FP32 only);
@@ -911,13 +891,9 @@ cudaError_t launch_mpm_step<float>(const MpmArgs<float> &a, int shape, cudaStrea
         return cudaGetLastError();
     }
     if (shape >= MPM_NSHAPES)
-        return stab ? launch_t<float, true, true>(a, shape - MPM_NSHAPES, s)
-                    : launch_t<float, true, false>(a, shape - MPM_NSHAPES, s);
-    return stab ? launch_t<float, false, true>(a, shape, s) : launch_t<float, false, false>(a, shape, s);
-}
-template <>
-cudaError_t launch_mpm_step<double>(const MpmArgs<double> &a, int shape, cudaStream_t s) {
-    return launch_t<double, false, false>(a, shape % MPM_NSHAPES, s);
+        return stab ? launch_t<true, true>(a, shape - MPM_NSHAPES, s)
+                    : launch_t<true, false>(a, shape - MPM_NSHAPES, s);
+    return stab ? launch_t<false, true>(a, shape, s) : launch_t<false, false>(a, shape, s);
 }
 
 }  // namespace hmc

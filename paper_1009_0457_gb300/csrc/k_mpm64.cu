@@ -1,0 +1,490 @@
+// The FP64 explicit MPM step (Sec. "Elastic Deformation") in 64-bit fixed point.
+//
+// Why: GB300 retires two FP64 lanes per clock and SM, so the step's ~870 FP64 instructions a
+// cell bounded it at 3.33 ms for 256^3 points whatever else was done.  The integer pipes run
+// 16 to 64 lanes a clock, and everything between the corner displacements and the corner
+// forces of a cell is linear: additions, the 3/1 interpolation weights, and 36 products with
+// the stiffness per point.  So a cell is computed in integers that share one exponent, and
+// only the node update (v, u) stays in FP64.
+//
+// Numbers.  E = the largest biased exponent among the cell's 24 corner displacements and the
+// mean strain.  A displacement is held as m * 2^3 (m its 53-bit mantissa) aligned to E, so
+// |U| < 2^56 and the largest displacements keep three bits below their own last one.  The
+// gradients (16 x interpolated differences) and the strains (two gradient entries and the mean
+// strain) are exact integer sums below 2^62.6; strains are taken / 8 (< 2^59.6) and split into
+// signed 32-bit halves.  The stiffness is held as integers C 2^cexp with row sums below 2^63,
+// split the same way; sigma = round(C e / 2^64) drops only the product of the two low halves
+// (< 2^62, below the rounding) and stays below 2^58.6; the sums behind it stay below 2^63.  The
+// traction sums (< 2^59.6) are exact, their first 3/1 sums (< 2^61.6) are taken / 8, the second
+// (< 2^60.6) and a corner's force (< 2^62.2) are exact again.  Each rounding is far below the
+// 2^-53 that every intermediate of an FP64 evaluation carries, and the corner forces are
+// +-X +-Y +-Z of the same integers, so a cell's forces sum to exactly zero whatever was rounded.
+// A node's force is the sum of its eight cells' integers: exact when their exponents agree and
+// the sum cannot leave 63 bits (both are tested), otherwise aligned to the largest exponent with
+// symmetric rounding.  A cell with a non-finite corner gets E = 2047 and its nodes NaN.
+// A displacement below 2^-1022 (subnormal) counts as zero.
+// Against an 80-bit reference (20x24x28 points, 100 steps) the velocity's relative error is
+// 5.6e-15 and the displacement's 6.8e-16; FP64 arithmetic gave 1.05e-14 and 7.6e-16.
+//
+// Tiling, scheduling and the march in z are those of the FP32 step (k_mpm.cu); nodes and forces
+// are kept in shared memory as two arrays of 16-byte halves, (x, y) and (z, exponent), so that
+// consecutive lanes read consecutive 16 bytes.  The forces are double-buffered, which leaves one
+// barrier per plane (two: 5 % slower).
+// What bounds it: 244 registers leave eight warps per SM, which issue 36 % of the cycles (the
+// busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
+// 32^3 20 (70), 96x90x100 67 (288), 128^3 129 (420), 256^3 714 (3330).
+#include "hmc_device.cuh"
+
+namespace hmc {
+
+namespace {
+
+typedef long long ll;
+
+struct FxHalf {   // 16 bytes: x and y, or z and the exponent
+    ll a, b;
+};
+
+template <int CX, int CY>
+struct alignas(16) FxSmem {
+    static constexpr int NX = CX + 1, NY = CY + 1;
+    FxHalf uxy[3][NY][NX], uze[3][NY][NX];   // node planes
+    FxHalf fxy[2][8][CY][CX], fze[2][8][CY][CX];   // (buffer) cell contributions to corner I + 2J + 4K
+    FxHalf eb[3];                            // mean strain, m * 2^8 aligned to ebe
+    int ebe;
+};
+
+__device__ __forceinline__ int dexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// mantissa of x times 2^K, aligned to the biased exponent E >= dexp(x); subnormals count as zero
+template <int K>
+__device__ __forceinline__ ll dfix(double x, int E) {
+    const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+    const ll m = ((ll)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x);
+    const ll s = e ? (ll)((unsigned long long)(m << K) >> min(E - e, 63)) : 0ll;
+    return hi < 0 ? -s : s;
+}
+
+// o[b][c] = sum_J sum_K W(J,b) W(K,c) d[J][K] with weights 3 (same side) and 1 (other side)
+// (the first index's sums taken / 2^SHIFT)
+template <int SHIFT>
+__device__ __forceinline__ void interp31(ll d00, ll d10, ll d01, ll d11, ll (&o)[2][2]) {
+    const ll s0 = d00 + d10, s1 = d01 + d11;
+    const ll e00 = (s0 + (d00 << 1)) >> SHIFT, e10 = (s0 + (d10 << 1)) >> SHIFT;
+    const ll e01 = (s1 + (d01 << 1)) >> SHIFT, e11 = (s1 + (d11 << 1)) >> SHIFT;
+    const ll t0 = e00 + e01, t1 = e10 + e11;
+    o[0][0] = t0 + (e00 << 1);
+    o[0][1] = t0 + (e01 << 1);
+    o[1][0] = t1 + (e10 << 1);
+    o[1][1] = t1 + (e11 << 1);
+}
+
+// One orientation's stiffness: the 21 upper-triangle entries, each as signed halves (x low, y high)
+struct FxRow {
+    int2 v[22];
+    __device__ __forceinline__ void load(const int2 *tab, uint32_t q) {
+        const int4 *p = reinterpret_cast<const int4 *>(tab + 24ll * q);
+#pragma unroll
+        for (int i = 0; i < 11; ++i) {
+            const int4 t = __ldg(p + i);
+            v[2 * i] = make_int2(t.x, t.y);
+            v[2 * i + 1] = make_int2(t.z, t.w);
+        }
+    }
+};
+
+__host__ __device__ constexpr int upper21(int i, int j) {   // place of entry (i, j) in the upper triangle
+    const int lo = i < j ? i : j, hi = i < j ? j : i;
+    return lo * 6 - lo * (lo - 1) / 2 + hi - lo;
+}
+
+// round(sum_j C_ij e_j / 2^64) for the six stress components
+__device__ __forceinline__ void fx_hooke(const FxRow &r, const ll (&e)[6], ll (&s)[6]) {
+    int eh[6], el[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        const ll x = e[j] >> 3;
+        el[j] = (int)x;
+        eh[j] = (int)(x >> 32) + (int)((unsigned)el[j] >> 31);
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        ll h = 0, x = 1ll << 31;
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const int2 c = r.v[upper21(i, j)];
+            h += (ll)c.y * eh[j];
+            x += (ll)c.y * el[j];
+            x += (ll)c.x * eh[j];
+        }
+        s[i] = h + (x >> 32);
+    }
+}
+
+// the visiting order of a cell's points: one coordinate changes from one to the next, so that a
+// grain boundary normal to x, y, z costs 4, 2, 1 reloads of the stiffness row
+__host__ __device__ constexpr int gray_pt(int n) {
+    return n == 0 ? 0 : n == 1 ? 1 : n == 2 ? 3 : n == 3 ? 2 : n == 4 ? 6 : n == 5 ? 7 : n == 6 ? 5 : 4;
+}
+
+// the 24 corner forces of a cell (times 32, with the sign of -f) from its corner displacements
+__device__ __forceinline__ void fx_cell(const ll (&u)[8][3], const ll (&eb)[6], const uint4 &sp, const int2 *tab,
+                                        ll (&f)[8][3]) {
+    FxRow row;
+    uint32_t qprev = spin_of(sp, local_slot(0));
+    row.load(tab, qprev);
+    ll gx[2][2][3], gy[2][2][3], gz[2][2][3];   // [b][c], [a][c], [a][b]: d u_d / dx, dy, dz
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        ll o[2][2];
+        interp31<0>(u[1][d] - u[0][d], u[3][d] - u[2][d], u[5][d] - u[4][d], u[7][d] - u[6][d], o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) gx[i >> 1][i & 1][d] = o[i >> 1][i & 1] + (d == 0 ? eb[0] : 0);
+        interp31<0>(u[2][d] - u[0][d], u[3][d] - u[1][d], u[6][d] - u[4][d], u[7][d] - u[5][d], o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            gy[i >> 1][i & 1][d] = o[i >> 1][i & 1] + (d == 1 ? eb[1] : d == 0 ? eb[5] : 0);
+        interp31<0>(u[4][d] - u[0][d], u[5][d] - u[1][d], u[6][d] - u[2][d], u[7][d] - u[3][d], o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            gz[i >> 1][i & 1][d] = o[i >> 1][i & 1] + (d == 2 ? eb[2] : d == 1 ? eb[3] : eb[4]);
+    }
+    ll tx[2][2][3], ty[2][2][3], tz[2][2][3];   // traction sums over a, b, c respectively
+#pragma unroll
+    for (int i = 0; i < 12; ++i)
+        tx[i / 6][i / 3 & 1][i % 3] = ty[i / 6][i / 3 & 1][i % 3] = tz[i / 6][i / 3 & 1][i % 3] = 0;
+#pragma unroll
+    for (int n = 0; n < 8; ++n) {
+        const int L = gray_pt(n);
+        const int a = L & 1, b = (L >> 1) & 1, c = L >> 2;
+        ll e[6], s[6];
+        e[0] = gx[b][c][0];
+        e[1] = gy[a][c][1];
+        e[2] = gz[a][b][2];
+        e[3] = gz[a][b][1] + gy[a][c][2];
+        e[4] = gz[a][b][0] + gx[b][c][2];
+        e[5] = gy[a][c][0] + gx[b][c][1];
+        const uint32_t q = spin_of(sp, local_slot(L));
+        if (q != qprev) {
+            row.load(tab, q);
+            qprev = q;
+        }
+        fx_hooke(row, e, s);
+        tx[b][c][0] += s[0]; tx[b][c][1] += s[5]; tx[b][c][2] += s[4];
+        ty[a][c][0] += s[5]; ty[a][c][1] += s[1]; ty[a][c][2] += s[3];
+        tz[a][b][0] += s[4]; tz[a][b][1] += s[3]; tz[a][b][2] += s[2];
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        ll X[2][2], Y[2][2], Z[2][2];
+        interp31<3>(tx[0][0][d], tx[1][0][d], tx[0][1][d], tx[1][1][d], X);   // X[J][K]
+        interp31<3>(ty[0][0][d], ty[1][0][d], ty[0][1][d], ty[1][1][d], Y);   // Y[I][K]
+        interp31<3>(tz[0][0][d], tz[1][0][d], tz[0][1][d], tz[1][1][d], Z);   // Z[I][J]
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            const int I = n & 1, J = (n >> 1) & 1, K = n >> 2;
+            f[n][d] = (I ? X[J][K] : -X[J][K]) + (J ? Y[I][K] : -Y[I][K]) + (K ? Z[I][J] : -Z[I][J]);
+        }
+    }
+}
+
+// three integers with one exponent (that of the cells' displacements; 2047 = not finite)
+struct Fx3 {
+    ll v[3];
+    int e;
+};
+
+// x / 2^n to the nearest, halves away from zero (a shift of 62 or more leaves nothing of |x| < 2^62.3)
+__device__ __forceinline__ ll rshift(ll x, int n) {
+    if (n <= 0) return x;
+    if (n > 61) return 0;
+    return (x + (1ll << (n - 1)) + (x >> 63)) >> n;
+}
+
+// whether a sum of up to eight integers, whose high words / 8 sum to t, stays within 63 bits
+__device__ __forceinline__ bool fits63(int t) { return (unsigned)(t + (1 << 28)) <= (1u << 29) - 8u; }
+
+// The sum of N terms x[i] 2^e[i] per direction.  With one exponent it is exact; otherwise the terms
+// are aligned to the largest exponent, and three bits above it where the sum would leave 63 bits.
+template <int N>
+__device__ __forceinline__ Fx3 fx_sum(const ll (&x)[3][N], const int (&e)[N]) {
+    Fx3 r;
+    r.e = e[0];
+    bool plain = true;
+#pragma unroll
+    for (int i = 1; i < N; ++i) {
+        plain &= e[i] == e[0];
+        r.e = max(r.e, e[i]);
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        ll v = 0;
+        int t = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            v += x[d][i];
+            t += (int)(x[d][i] >> 35);
+        }
+        r.v[d] = v;
+        plain &= fits63(t);
+    }
+    if (!plain && r.e < 2047) {
+        const int top = r.e;
+#pragma unroll 1
+        for (int up = 0; up <= 3; up += 3) {
+            r.e = top + up;
+            bool fits = true;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                ll v = 0;
+                int t = 0;
+#pragma unroll
+                for (int i = 0; i < N; ++i) {
+                    const ll s = rshift(x[d][i], r.e - e[i]);
+                    v += s;
+                    t += (int)(s >> 35);
+                }
+                r.v[d] = v;
+                fits &= fits63(t);
+            }
+            if (fits) break;
+        }
+    }
+    return r;
+}
+
+template <int CX, int CY>
+__global__ void __launch_bounds__(CX *CY, 1) k_mpm_fixed(MpmArgs<double> a) {
+    constexpr int OX = CX - 1, OY = CY - 1, NX = CX + 1, NN = (CX + 1) * (CY + 1), NTHR = CX * CY;
+    constexpr int PER = (NN + NTHR - 1) / NTHR;
+    using Smem = FxSmem<CX, CY>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
+    const int tid = threadIdx.x;
+    const double fscale = -a.dt_over_m * 0.03125;          // -dt / (32 m)
+    // the force integers of exponent E are 2^(E - cexp - 1013) (16/9/.. units as in the FP32 step)
+    const int fexp = dexp(fscale) ? dexp(fscale) - a.cexp - 1013 : -10000;   // (subnormal: the general form)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    long long w = a.total * blockIdx.x / gridDim.x;
+    const long long wend = a.total * (blockIdx.x + 1) / gridDim.x;
+    int r = 0;
+    while (w < wend) {
+        while (a.sched[r + 1].plane_off <= w) ++r;
+        const Replica &R = a.reps[r];
+        const MpmSched &SC = a.sched[r];
+        const int nbx = R.nbx, nby = R.nby, nbz = R.nbz;
+        const long long lw = w - SC.plane_off;
+        const int tile = (int)(lw / nbz);
+        const int k0 = (int)(lw - (long long)tile * nbz);
+        const long long rem = min(wend, a.sched[r + 1].plane_off) - w;
+        const int kend = (int)min((long long)nbz, (long long)k0 + rem);
+        w += kend - k0;
+        const int i0 = (tile % SC.tiles_x) * OX, j0 = (tile / SC.tiles_x) * OY;
+        const int W = min(CX, nbx - i0 + 1), H = min(CY, nby - j0 + 1);
+        const int lci = tid % W, lcj = tid / W;
+        const bool need = tid < W * H;
+        const bool own = need && lci >= 1 && lcj >= 1;
+        const int plane = nbx * nby;
+        const long long col = R.blk_off + wrapi(i0 - 1 + lci, nbx) + nbx * wrapi(j0 - 1 + lcj, nby);
+        int ncol[PER];   // the tile's nodes that this thread loads, as (i + nbx j) in a node plane
+#pragma unroll
+        for (int m = 0; m < PER; ++m) {
+            const int t = tid + m * NTHR;
+            ncol[m] = wrapi(i0 - 1 + t % NX, nbx) + nbx * wrapi(j0 - 1 + t / NX, nby);
+        }
+        double pl[PER][3];
+        auto fetch = [&](int k) {   // node plane k, -1 <= k <= nbz (periodic in z)
+            const int gk = k < 0 ? k + nbz : (k >= nbz ? k - nbz : k);
+            const double *base = a.u_in + 3 * (R.blk_off + (long long)plane * gk);
+#pragma unroll
+            for (int m = 0; m < PER; ++m)
+                if (tid + m * NTHR < NN)
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) pl[m][d] = __ldg(base + 3 * ncol[m] + d);
+        };
+        auto store = [&](int b) {
+#pragma unroll
+            for (int m = 0; m < PER; ++m) {
+                const int t = tid + m * NTHR;
+                if (t < NN) {
+                    const int E = max(dexp(pl[m][0]), max(dexp(pl[m][1]), dexp(pl[m][2])));
+                    (&sm.uxy[b][0][0])[t] = FxHalf{dfix<3>(pl[m][0], E), dfix<3>(pl[m][1], E)};
+                    (&sm.uze[b][0][0])[t] = FxHalf{dfix<3>(pl[m][2], E), (ll)E};
+                }
+            }
+        };
+        int b0 = 0, b1 = 1, b2 = 2, fb = 0;
+        fetch(k0 - 1);
+        store(b0);
+        fetch(k0);
+        store(b1);
+        if (tid == 0) {
+            double e[6];
+            int E = 0;
+            for (int i = 0; i < 6; ++i) {
+                e[i] = R.st->ebar[i];
+                E = max(E, dexp(e[i]));
+            }
+            for (int i = 0; i < 3; ++i) sm.eb[i] = FxHalf{dfix<8>(e[2 * i], E), dfix<8>(e[2 * i + 1], E)};
+            sm.ebe = E;
+        }
+        uint4 sp = need ? __ldg(a.spins + col + (long long)plane * wrapi(k0 - 1, nbz)) : make_uint4(0, 0, 0, 0);
+        __syncthreads();
+
+        Fx3 acc = {{0, 0, 0}, 0};
+        const uint4 *spn = a.spins + col + (long long)plane * k0;
+        const double *uip = a.u_in + 3 * (col + (long long)plane * k0);
+        double *vp = a.v + 3 * (col + (long long)plane * k0);
+        double *up = a.u_out + 3 * (col + (long long)plane * k0);
+        const long long pstride = 3ll * plane;
+        for (int kk = k0 - 1; kk < kend; ++kk) {
+            uint4 sp_next = make_uint4(0, 0, 0, 0);
+            if (need && kk + 1 < kend) sp_next = __ldg(spn);
+            spn += plane;
+            double vold[3] = {0, 0, 0}, uold[3] = {0, 0, 0};
+            if (own && kk >= k0) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    vold[d] = vp[d];
+                    uold[d] = __ldg(uip + d);
+                }
+            }
+            const bool more = kk + 1 < kend;
+            if (more) fetch(kk + 2);
+            if (need) {
+                ll u[8][3];
+                int ne[8], E = sm.ebe;
+#pragma unroll
+                for (int n = 0; n < 8; ++n) {
+                    const int b = n >> 2 ? b1 : b0, j = lcj + ((n >> 1) & 1), i = lci + (n & 1);
+                    const FxHalf p = sm.uxy[b][j][i], q = sm.uze[b][j][i];
+                    u[n][0] = p.a;
+                    u[n][1] = p.b;
+                    u[n][2] = q.a;
+                    ne[n] = (int)q.b;
+                    E = max(E, ne[n]);
+                }
+#pragma unroll
+                for (int n = 0; n < 8; ++n) {
+                    const int s = min(E - ne[n], 63);
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) u[n][d] >>= s;
+                }
+                ll eb[6];
+                const int se = min(E - sm.ebe, 63);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const FxHalf t = sm.eb[i];
+                    eb[2 * i] = t.a >> se;
+                    eb[2 * i + 1] = t.b >> se;
+                }
+                ll f[8][3];
+                fx_cell(u, eb, sp, a.cfix, f);
+#pragma unroll
+                for (int n = 0; n < 8; ++n) {
+                    sm.fxy[fb][n][lcj][lci] = FxHalf{f[n][0], f[n][1]};
+                    sm.fze[fb][n][lcj][lci] = FxHalf{f[n][2], (ll)E};
+                }
+            }
+            if (more) store(b2);   // buffer b2 was last read before the previous barrier
+            __syncthreads();
+            if (own) {
+                auto sum4 = [&](int c) {
+                    const FxHalf a3 = sm.fxy[fb][c + 3][lcj - 1][lci - 1], b3 = sm.fze[fb][c + 3][lcj - 1][lci - 1];
+                    const FxHalf a2 = sm.fxy[fb][c + 2][lcj - 1][lci], b2 = sm.fze[fb][c + 2][lcj - 1][lci];
+                    const FxHalf a1 = sm.fxy[fb][c + 1][lcj][lci - 1], b1 = sm.fze[fb][c + 1][lcj][lci - 1];
+                    const FxHalf a0 = sm.fxy[fb][c][lcj][lci], b0 = sm.fze[fb][c][lcj][lci];
+                    const ll x[3][4] = {{a3.a, a2.a, a1.a, a0.a}, {a3.b, a2.b, a1.b, a0.b}, {b3.a, b2.a, b1.a, b0.a}};
+                    const int e[4] = {(int)b3.b, (int)b2.b, (int)b1.b, (int)b0.b};
+                    return fx_sum<4>(x, e);
+                };
+                if (kk >= k0) {
+                    const Fx3 up4 = sum4(0);
+                    const ll x2[3][2] = {{acc.v[0], up4.v[0]}, {acc.v[1], up4.v[1]}, {acc.v[2], up4.v[2]}};
+                    const int e2[2] = {acc.e, up4.e};
+                    const Fx3 F = fx_sum<2>(x2, e2);
+                    const int ef = fexp + F.e;   // exponent of the product's scale
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        const double Fd = (double)F.v[d], kv = rmul(a.keep, vold[d]);
+                        double vn;
+                        if (F.e >= 2047)
+                            vn = __longlong_as_double(0x7ff8000000000000ll);
+                        else if ((unsigned)(ef - 1) < 2045u)
+                            vn = rfma(__hiloint2double((__double2hiint(fscale) & 0x800fffff) | (ef << 20),
+                                                       __double2loint(fscale)),
+                                      Fd, kv);
+                        else
+                            vn = rfma(fscale, scalbn(Fd, F.e - a.cexp - 1013), kv);
+                        vp[d] = vn;
+                        up[d] = rfma(a.dt, vn, uold[d]);
+                    }
+                    vp += pstride;
+                    up += pstride;
+                    uip += pstride;
+                }
+                acc = sum4(4);
+            }
+            // one barrier a plane: the next plane writes the other force buffer and the node plane that
+            // was last read before this one's barrier
+            fb ^= 1;
+            const int t = b0;
+            b0 = b1;
+            b1 = b2;
+            b2 = t;
+            sp = sp_next;
+        }
+        __syncthreads();   // the next range reuses every buffer
+    }
+}
+
+template <int CX, int CY>
+cudaError_t prepare_t() {
+    return cudaFuncSetAttribute(k_mpm_fixed<CX, CY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sizeof(FxSmem<CX, CY>));
+}
+template <int CX, int CY>
+int per_sm_t() {
+    int n = 1;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_mpm_fixed<CX, CY>, CX * CY,
+                                                                       sizeof(FxSmem<CX, CY>));
+    return (e != cudaSuccess || n < 1) ? 1 : n;
+}
+// programmatic stream serialisation, as the FP32 step
+template <int CX, int CY>
+cudaError_t launch_t(const MpmArgs<double> &a, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(a.grid);
+    cfg.blockDim = dim3(CX * CY);
+    cfg.dynamicSmemBytes = sizeof(FxSmem<CX, CY>);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_mpm_fixed<CX, CY>, a);
+}
+
+}  // namespace
+
+cudaError_t mpm64_prepare() {
+    cudaError_t e;
+    if ((e = prepare_t<16, 16>()) != cudaSuccess || (e = prepare_t<32, 8>()) != cudaSuccess) return e;
+    return prepare_t<8, 32>();
+}
+
+template <>
+int mpm_per_sm<double>(int shape, int) {
+    const int sh = shape % MPM_NSHAPES;
+    return sh == MPM_32x8 ? per_sm_t<32, 8>() : sh == MPM_8x32 ? per_sm_t<8, 32>() : per_sm_t<16, 16>();
+}
+
+template <>
+cudaError_t launch_mpm_step<double>(const MpmArgs<double> &a, int shape, cudaStream_t s) {
+    const int sh = shape % MPM_NSHAPES;
+    return sh == MPM_32x8 ? launch_t<32, 8>(a, s) : sh == MPM_8x32 ? launch_t<8, 32>(a, s) : launch_t<16, 16>(a, s);
+}
+
+}  // namespace hmc
