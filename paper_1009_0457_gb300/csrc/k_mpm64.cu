@@ -29,7 +29,7 @@
 // Tiling, scheduling and the march in z are those of the FP32 step (k_mpm.cu); nodes and forces
 // are kept in shared memory as two arrays of 16-byte halves, (x, y) and (z, exponent), so that
 // consecutive lanes read consecutive 16 bytes.  The forces are double-buffered, which leaves one
-// barrier per plane (two: 5 % slower).
+// barrier per plane.
 // What bounds it: 244 registers leave eight warps per SM, which issue 36 % of the cycles (the
 // busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
 // 32^3 20 (70), 96x90x100 67 (288), 128^3 129 (420), 256^3 714 (3330).

@@ -20,6 +20,8 @@
 // address is looked up once per device and kept for the life of the process,
 // which assumes the device's primary context and no cudaDeviceReset after the
 // first call.
+#include <cooperative_groups.h>
+
 #include <cmath>
 #include <mutex>
 #include <string>
@@ -34,7 +36,8 @@ void set_unbound_error(const std::string &msg);  // message for hmc_last_error(N
 namespace {
 
 constexpr int NOALLOC_MAX_CTAS = 8192;
-constexpr int NOALLOC_THREADS = 256;
+constexpr int NOALLOC_THREADS = 256;   // cells of a CTA (and its threads, over CELLS)
+constexpr int NOALLOC_SPREAD = 304;    // CTAs (two per SM) from which a thread takes four cells
 
 static __device__ __align__(256) double g_noalloc_partials[NOALLOC_MAX_CTAS * 8];
 
@@ -58,20 +61,63 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x) {
     hi = s;
 }
 
+// Compensated running sum (Kahan 1965): four additions a term against TwoSum's seven.
+__device__ __forceinline__ void kahan_add(float &s, float &c, float x) {
+    const float y = __fsub_rn(x, c), t = __fadd_rn(s, y);
+    c = __fsub_rn(__fsub_rn(t, s), y);
+    s = t;
+}
+
+// a point's full 6x6 stiffness, 16-byte loads where the table allows them
+template <bool VEC>
+__device__ __forceinline__ void load_c36(const float *p, float (&c)[36]) {
+    if constexpr (VEC) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const float4 t = __ldg(reinterpret_cast<const float4 *>(p) + i);
+            c[4 * i] = t.x;
+            c[4 * i + 1] = t.y;
+            c[4 * i + 2] = t.z;
+            c[4 * i + 3] = t.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 36; ++i) c[i] = __ldg(p + i);
+    }
+}
+
 // One thread per 2x2x2 cell: strain of its eight points from the trilinear
 // nodal field, Hooke's law with the point's rotated stiffness, natural-order
 // stress out, and per-CTA FP64 partial sums of sigma and 1/2 sigma.eps.
-__global__ void __launch_bounds__(NOALLOC_THREADS) k_stress_noalloc(NoallocArgs a) {
-    __shared__ double red[NOALLOC_THREADS / 32][7];
+//
+// The 24 bytes a point writes are most of the traffic (403 of 461 MB at 256^3).
+// Written by the thread that formed them they were 4-byte stores 48 bytes apart;
+// a lane's two x-neighbours are 48 contiguous bytes instead, which a warp passes
+// through shared memory (16-byte units 3 lane + j: free of bank conflicts) and
+// stores in order of address, 16 bytes a lane.  The stiffness row is kept in
+// registers while consecutive points share an orientation.  VEC: every pointer
+// allows the wide accesses (4 bytes for the spins, 16 for ctab and sigma); the
+// other form takes 4-byte loads and stores in the same order.
+//
+// CELLS: blocks of a CTA's 256 that a thread takes in turn.  Four on large grids: the
+// warp's TwoSum reduction (about 350 of 1900 instructions when every cell paid it) is then paid
+// once for four cells.  One on grids of fewer CTAs than NOALLOC_SPREAD, where the chain of four cells would
+// be longer than the whole pass.
+template <bool VEC, int CELLS>
+__global__ void __launch_bounds__(NOALLOC_THREADS / CELLS, 2 * CELLS) k_stress_noalloc(NoallocArgs a) {
+    constexpr int THREADS = NOALLOC_THREADS / CELLS;
+    __shared__ double red[THREADS / 32][7];
+    __shared__ float4 stage[THREADS / 32][96];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     float hi[7], lo[7];
 #pragma unroll
     for (int i = 0; i < 7; ++i) hi[i] = lo[i] = 0.f;
-    const long long blk = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (blk < a.nblk) {
-        const int bx = (int)(blk % a.nbx);
-        const long long r = blk / a.nbx;
-        const int by = (int)(r % a.nby), bz = (int)(r / a.nby);
-        float u[8][3];
+    // a cell's first point (the caller's arrays), corner displacements and spins (two x neighbours a word)
+    auto load_cell = [&](unsigned blk, unsigned &p0, float (&u)[8][3], unsigned (&sp)[4]) {
+        const unsigned rr = blk / (unsigned)a.nbx;
+        const int bx = (int)(blk - rr * (unsigned)a.nbx), by = (int)(rr % (unsigned)a.nby), bz = (int)(rr / (unsigned)a.nby);
+        p0 = 2u * bx + (unsigned)a.nx * (2u * by + (unsigned)a.ny * 2u * bz);
 #pragma unroll
         for (int K = 0; K < 2; ++K)
 #pragma unroll
@@ -81,35 +127,92 @@ __global__ void __launch_bounds__(NOALLOC_THREADS) k_stress_noalloc(NoallocArgs 
                     const int gi = bx + I == a.nbx ? 0 : bx + I;
                     const int gj = by + J == a.nby ? 0 : by + J;
                     const int gk = bz + K == a.nbz ? 0 : bz + K;
-                    const long long n = 3ll * (gi + (long long)a.nbx * (gj + (long long)a.nby * gk));
+                    const unsigned n = 3u * (gi + (unsigned)a.nbx * (gj + (unsigned)a.nby * gk));
 #pragma unroll
                     for (int d = 0; d < 3; ++d) u[hmc::corner(I, J, K)][d] = __ldg(a.u + n + d);
                 }
+#pragma unroll
+        for (int row = 0; row < 4; ++row) {
+            const unsigned p = p0 + (unsigned)a.nx * ((row & 1) + (unsigned)a.ny * (row >> 1));
+            if constexpr (VEC)
+                sp[row] = __ldg(reinterpret_cast<const unsigned *>(a.spins + p));
+            else
+                sp[row] = __ldg(a.spins + p) | (unsigned)__ldg(a.spins + p + 1) << 16;
+        }
+    };
+#pragma unroll 1
+    for (int cell = 0; cell < CELLS; ++cell) {
+        const unsigned blk = blockIdx.x * NOALLOC_THREADS + cell * THREADS + threadIdx.x;   // < 2^21 + 256
+        const bool live = blk < (unsigned)a.nblk;
+        if (!__any_sync(0xffffffffu, live)) break;
+        unsigned p0 = 0, sp[4] = {0, 0, 0, 0};
         hmc::CellGrad<float> g;
-        hmc::cell_gradients<float>(u, g);
+        if (live) {
+            float u[8][3];
+            load_cell(blk, p0, u, sp);
+            hmc::cell_gradients<float>(u, g);
+        }
+        // place of the cell's first point in sigma in 16-byte units (6 floats a point, even points)
+        const unsigned base4 = live ? p0 / 2u * 3u : 0xffffffffu;
+        float c[36];
+        unsigned qprev = 0xffffffffu;
+        // rows and the two points of each in a Gray-code order of the eight points, so that a boundary
+        // through the cell reloads the stiffness row least often
 #pragma unroll
-        for (int L = 0; L < 8; ++L) {
-            const int lx = L & 1, ly = (L >> 1) & 1, lz = L >> 2;
-            const long long x = 2 * bx + lx, y = 2 * by + ly, z = 2 * bz + lz;
-            const long long p = x + a.nx * (y + (long long)a.ny * z);
-            float e[6], s[6];
-            hmc::point_strain<float>(g, a.eb, lx, ly, lz, e);
-            const float *c = a.ctab + 36ll * __ldg(a.spins + p);
-            float w = 0.f;
+        for (int n = 0; n < 4; ++n) {
+            const int row = n == 2 ? 3 : n == 3 ? 2 : n, ly = row & 1, lz = row >> 1;
+            __syncwarp();
+            if (live) {
+                float out[12];
 #pragma unroll
-            for (int i = 0; i < 6; ++i) {
-                float acc = 0.f;
+                for (int m = 0; m < 2; ++m) {
+                    const int lx = m ^ (n & 1);
+                    float e[6];
+                    hmc::point_strain<float>(g, a.eb, lx, ly, lz, e);
+                    const unsigned q = lx ? sp[row] >> 16 : sp[row] & 0xffffu;
+                    if (q != qprev) {
+                        load_c36<VEC>(a.ctab + 36ll * q, c);
+                        qprev = q;
+                    }
+                    float w = 0.f;
 #pragma unroll
-                for (int j = 0; j < 6; ++j) acc += __ldg(c + 6 * i + j) * e[j];
-                s[i] = acc;
-                w += acc * e[i];
-                two_sum_add(hi[i], lo[i], acc);
+                    for (int i = 0; i < 6; ++i) {
+                        float acc = 0.f;
+#pragma unroll
+                        for (int j = 0; j < 6; ++j) acc += c[6 * i + j] * e[j];
+                        out[6 * lx + i] = acc;
+                        w += acc * e[i];
+                        kahan_add(hi[i], lo[i], acc);
+                    }
+                    kahan_add(hi[6], lo[6], 0.5f * w);
+                }
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    stage[warp][3 * lane + j] = make_float4(out[4 * j], out[4 * j + 1], out[4 * j + 2], out[4 * j + 3]);
             }
-            two_sum_add(hi[6], lo[6], 0.5f * w);
+            __syncwarp();
+            const unsigned row4 = (unsigned)a.nx * (ly + (unsigned)a.ny * lz) / 2u * 3u;
+            if constexpr (VEC) {
 #pragma unroll
-            for (int i = 0; i < 6; ++i) a.sigma[6 * p + i] = s[i];
+                for (int k = 0; k < 3; ++k) {
+                    const unsigned t = 32u * k + lane;
+                    const unsigned to = __shfl_sync(0xffffffffu, base4, t / 3);
+                    if (to != 0xffffffffu)
+                        __stcs(reinterpret_cast<float4 *>(a.sigma) + (size_t)(to + row4 + t % 3), stage[warp][t]);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 12; ++k) {
+                    const unsigned t = 32u * k + lane;
+                    const unsigned to = __shfl_sync(0xffffffffu, base4, t / 12);
+                    if (to != 0xffffffffu)
+                        a.sigma[4 * (size_t)(to + row4) + t % 12] = reinterpret_cast<const float *>(stage[warp])[t];
+                }
+            }
         }
     }
+#pragma unroll
+    for (int i = 0; i < 7; ++i) lo[i] = -lo[i];   // Kahan's c is what the sum still owes
 #pragma unroll
     for (int off = 16; off; off >>= 1)
 #pragma unroll
@@ -119,35 +222,44 @@ __global__ void __launch_bounds__(NOALLOC_THREADS) k_stress_noalloc(NoallocArgs 
             two_sum_add(hi[i], lo[i], oh);
             lo[i] += ol;
         }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lane == 0)
         for (int i = 0; i < 7; ++i) red[warp][i] = (double)hi[i] + (double)lo[i];
     __syncthreads();
     if (threadIdx.x < 7) {
         double s = 0.0;
-        for (int w = 0; w < NOALLOC_THREADS / 32; ++w) s += red[w][threadIdx.x];
+        for (int w = 0; w < THREADS / 32; ++w) s += red[w][threadIdx.x];
         a.partials[8ll * blockIdx.x + threadIdx.x] = s;  // every slot this call reads is written here
     }
 }
 
-// Fixed-order FP64 sum of the partials of all CTAs.
-__global__ void __launch_bounds__(256) k_noalloc_finish(NoallocArgs a, int nparts) {
-    __shared__ double red[256][7];
-    double s[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int p = threadIdx.x; p < nparts; p += 256)
-        for (int i = 0; i < 7; ++i) s[i] += a.partials[8ll * p + i];
-    for (int i = 0; i < 7; ++i) red[threadIdx.x][i] = s[i];
-    __syncthreads();
-    for (int w = 128; w; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int i = 0; i < 7; ++i) red[threadIdx.x][i] += red[threadIdx.x + w][i];
-        __syncthreads();
+// Fixed-order FP64 sum of the partials of all CTAs by one cluster of FINISH_CTAS CTAs: CTA k
+// takes the slots k, k + FINISH_CTAS, ... with one warp per quantity, and CTA 0 adds the CTAs'
+// sums.  (One CTA alone was bound by the FP64 rate of its SM: 31 us for the 8192 x 7 values of
+// 256^3.)  Launched with programmatic serialisation, so that its launch overlaps the pass.
+constexpr int FINISH_CTAS = 8;
+__global__ void __cluster_dims__(FINISH_CTAS, 1, 1) __launch_bounds__(224) k_noalloc_finish(NoallocArgs a, int nparts) {
+    __shared__ double sum[7];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    double s = 0.0;
+    for (int p = blockIdx.x + FINISH_CTAS * lane; p < nparts; p += FINISH_CTAS * 32) s += a.partials[8ll * p + i];
+#pragma unroll
+    for (int off = 16; off; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    if (lane == 0) sum[i] = s;
+    cl.sync();
+    if (blockIdx.x == 0 && threadIdx.x < 7) {
+        double t = 0.0;
+        for (int k = 0; k < FINISH_CTAS; ++k) t += *cl.map_shared_rank(&sum[threadIdx.x], k);
+        if (threadIdx.x < 6)
+            a.mean[threadIdx.x] = t / (double)a.n_sites;
+        else
+            *a.energy = t;
     }
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < 6; ++i) a.mean[i] = red[0][i] / (double)a.n_sites;
-        *a.energy = red[0][6];
-    }
+    cl.sync();   // the others' shared memory stays until it has been read
 }
+
 
 // Device address of the scratch array, looked up once per device.
 std::mutex g_setup_mutex;
@@ -215,9 +327,32 @@ extern "C" hmc_status hmc_stress_noalloc(const uint16_t *d_spins, const float *d
     a.nblk = nblk;
     a.n_sites = 8 * nblk;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    k_stress_noalloc<<<(unsigned)nparts, NOALLOC_THREADS, 0, s>>>(a);
-    k_noalloc_finish<<<1, 256, 0, s>>>(a, (int)nparts);
+    auto addr = [](const void *p) { return reinterpret_cast<uintptr_t>(p); };
+    const bool vec = (addr(d_ctab) | addr(d_sigma)) % 16 == 0 && addr(d_spins) % 4 == 0;
+    const unsigned grid = (unsigned)nparts;
+    if (nparts < NOALLOC_SPREAD) {
+        if (vec)
+            k_stress_noalloc<true, 1><<<grid, NOALLOC_THREADS, 0, s>>>(a);
+        else
+            k_stress_noalloc<false, 1><<<grid, NOALLOC_THREADS, 0, s>>>(a);
+    } else if (vec) {
+        k_stress_noalloc<true, 4><<<grid, NOALLOC_THREADS / 4, 0, s>>>(a);
+    } else {
+        k_stress_noalloc<false, 4><<<grid, NOALLOC_THREADS / 4, 0, s>>>(a);
+    }
     e = cudaGetLastError();
+    if (e == cudaSuccess) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(FINISH_CTAS);
+        cfg.blockDim = dim3(224);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, k_noalloc_finish, a, (int)nparts);
+    }
     if (e != cudaSuccess) {
         hmc::set_unbound_error(std::string("hmc_stress_noalloc: launch: ") + cudaGetErrorString(e));
         return HMC_ERR_CUDA;
