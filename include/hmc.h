@@ -170,12 +170,13 @@ hmc_status hmc_create_batch(const hmc_params *params, int32_t n_replicas, hmc_ha
 hmc_status hmc_select_replica(hmc_handle *h, int32_t r);
 
 /* Launch configuration chosen by the autotuner at the first MPM step (or the
- * default before it): MPM variant v (patch shape v % 3 -- 0: 16x16 cells,
- * 1: 32x8, 2: 8x32 -- with, for v >= 3 (FP32 only), the Hooke product as
- * paired FP32 FMAs) and the number of persistent MPM CTAs.  The autotuner
- * times every candidate on scratch copies of the nodal state; all patch
- * shapes of one Hooke variant give bit-identical results.  Environment
- * variable HMC_AUTOTUNE=0 keeps variant 0; HMC_MPM_SHAPE=<v> forces one. */
+ * default before it): MPM variant v and the number of CTAs of a step.  March
+ * up z over patches that own 0: 15x15, 1: 31x7, 2: 7x31 nodes, 3: as many as
+ * make the fewest patches of even size, 4: as many as make the fewest cells;
+ * one pass over blocks of at most 5: 256, 6: 96 cells.  The autotuner times
+ * the candidates on scratch copies of the nodal state; all variants give
+ * bit-identical results.  Environment variable HMC_AUTOTUNE=0 keeps variant
+ * 0; HMC_MPM_SHAPE=<v> forces one. */
 hmc_status hmc_get_tuning(hmc_handle *h, int32_t *mpm_shape, int32_t *mpm_grid);
 
 /* The sweep choices of the autotuner, made at the same time (a library service with

@@ -35,7 +35,7 @@ int slot_local_h(int s) { static const int t[8] = {0, 3, 5, 6, 1, 2, 4, 7}; retu
 // Autotuner results, per batch signature, for the life of the process.
 std::mutex g_tune_mutex;
 struct TuneResult {
-    int mpm_shape, mpm_grid, sweep_cta;
+    int mpm_variant, mpm_limit, sweep_cta;
     bool store;
 };
 std::map<std::string, TuneResult> g_tune_cache;
@@ -96,10 +96,10 @@ struct hmc_handle {
     hmc::Replica *d_reps = nullptr;       // R descriptors
     hmc::Replica rep0{};                  // host copy of descriptor 0 (kernel argument of one-replica sweeps)
     int *d_cta_rep = nullptr;             // replica of every sweep / stress CTA
-    hmc::MpmSched *d_sched = nullptr;     // R + 1 MPM schedules for the chosen shape
+    hmc::MpmSched *d_sched = nullptr;     // R + 1 MPM schedules for the chosen variant
+    long long *d_cuts = nullptr;          // march: first work item of every CTA
     // MPM launch configuration (autotuned)
-    int mpm_shape = hmc::MPM_16x16, mpm_grid = 1;
-    long long mpm_total = 0;
+    int mpm_shape = 0, mpm_grid = 1;      // variant and CTAs
     bool tuned = false;
     int sweep_cta = 256;                  // sweep threads per CTA (tuned)
     double *plain_sig = nullptr, *plain_f = nullptr;   // the plain FP64 step's point stresses, cell forces
@@ -283,7 +283,7 @@ hmc::MpmArgs<T> mpm_args(hmc_handle *h, const void *u_in, void *u_out, void *v) 
     a.reps = h->d_reps;
     a.sched = h->d_sched;
     a.nrep = h->R;
-    a.total = h->mpm_total;
+    a.cuts = h->d_cuts;
     a.spins = h->spins;
     a.u_in = static_cast<const T *>(u_in);
     a.u_out = static_cast<T *>(u_out);
@@ -554,7 +554,7 @@ void destroy_buffers(hmc_handle *h) {
     for (int i = 0; i < 2; ++i)
         if (h->gexec[i]) cudaGraphExecDestroy(h->gexec[i]);
     void *bufs[] = {h->spins, h->stage16, h->u[0], h->u[1], h->v, h->sig, h->ctab, h->cubw, h->cfix, h->wtab, h->atab, h->thr, h->counts,
-                    h->bins, h->partials, h->fractions, h->binmap, h->st, h->d_reps, h->d_cta_rep, h->d_sched,
+                    h->bins, h->partials, h->fractions, h->binmap, h->st, h->d_reps, h->d_cta_rep, h->d_sched, h->d_cuts,
                     h->zone_work, h->snap, h->zone_count, h->ktab, h->zone_sched, h->cc_parent, h->cc_count,
                     h->stab, h->plain_sig, h->plain_f};
     for (void *b : bufs)
@@ -597,38 +597,140 @@ void pack_stress_host(const RepHost &R, const double *in, std::vector<T> &packed
 
 // ---- MPM schedule and autotuner --------------------------------------------
 
-hmc_status upload_sched(hmc_handle *h, int variant) {
-    const int shape = variant % hmc::MPM_NSHAPES;
-    const int ox = hmc::mpm_shape_cx(shape) - 1, oy = hmc::mpm_shape_cy(shape) - 1;
-    std::vector<hmc::MpmSched> sc(h->R + 1);
-    long long off = 0;
-    for (int r = 0; r < h->R; ++r) {
-        const RepHost &R = h->reps[r];
-        sc[r].tiles_x = (R.nbx + ox - 1) / ox;
-        sc[r].tiles_y = (R.nby + oy - 1) / oy;
-        sc[r].plane_off = off;
-        off += (long long)sc[r].tiles_x * sc[r].tiles_y * R.nbz;
+// Most nodes that a tile (march) or block of variant v owns per edge of a replica.
+void patch_of(int v, const RepHost &R, int (&o)[3]) {
+    const int n[3] = {R.nbx, R.nby, R.nbz};
+    if (v < hmc::MPM_FIT) {
+        const int fixed[3][2] = {{15, 15}, {31, 7}, {7, 31}};
+        o[0] = std::min(fixed[v][0], n[0]);
+        o[1] = std::min(fixed[v][1], n[1]);
+        o[2] = n[2];
+        return;
     }
-    sc[h->R].tiles_x = sc[h->R].tiles_y = 0;
-    sc[h->R].plane_off = off;
-    h->mpm_total = off;
-    HMC_CK(h, cudaStreamSynchronize(h->stream), "sync");
-    HMC_CK(h, cudaMemcpy(h->d_sched, sc.data(), sizeof(hmc::MpmSched) * sc.size(), cudaMemcpyHostToDevice),
-           "schedule upload");
-    return HMC_OK;
+    const bool block = hmc::mpm_is_block(v);
+    const int cells = v == hmc::MPM_BLOCK + 1 ? hmc::MPM_SMALL_BLOCK : hmc::MPM_THREADS;
+    const int nodes = block ? 2 * cells : hmc::MPM_NODES;
+    // over every division of the edges into tiles of even size that the CTA's threads and node
+    // buffer hold: fewest tiles, then fewest cells (variant 4: fewest cells, then fewest tiles)
+    long long best[2] = {0, 0};
+    auto tiles_of = [](int edge, int own) { return (edge + own - 1) / own; };
+    for (int x = 1; x <= n[0] && 2 * (x + 1) <= cells; ++x) {
+        const int tx = tiles_of(n[0], x);
+        if ((n[0] + tx - 1) / tx != x) continue;   // not the even size of its count
+        for (int y = 1; y <= n[1] && (x + 1) * (y + 1) <= cells; ++y) {
+            const int ty = tiles_of(n[1], y);
+            if ((n[1] + ty - 1) / ty != y) continue;
+            for (int z = block ? 1 : n[2]; z <= n[2]; ++z) {
+                const int tz = tiles_of(n[2], z);
+                if ((n[2] + tz - 1) / tz != z) continue;
+                if (block && ((x + 1) * (y + 1) * (z + 1) > cells || (x + 2) * (y + 2) * (z + 2) > nodes)) break;
+                if (!block && (x + 2) * (y + 2) > nodes) break;
+                const long long tiles = (long long)tx * ty * tz;
+                const long long work = (long long)(n[0] + tx) * (n[1] + ty) * (block ? n[2] + tz : 1);
+                const long long key[2] = {v == hmc::MPM_FIT + 1 ? work : tiles, v == hmc::MPM_FIT + 1 ? tiles : work};
+                if (best[0] == 0 || key[0] < best[0] || (key[0] == best[0] && key[1] < best[1])) {
+                    best[0] = key[0];
+                    best[1] = key[1];
+                    o[0] = x;
+                    o[1] = y;
+                    o[2] = z;
+                }
+            }
+        }
+    }
 }
 
-// Persistent MPM grid: resident CTAs per SM (at most per_sm_limit when positive) times the
-// SMs, and no more CTAs than leave min_planes work items (planes) to each.  Every CTA pays
-// one plane of restart for its range, so small grids trade that for parallelism.
-int grid_for_shape(hmc_handle *h, int shape, int per_sm_limit, int min_planes = 4) {
-    int per_sm = h->p.precision == HMC_FP32 ? hmc::mpm_per_sm<float>(shape, h->p.n_orient)
-                                            : hmc::mpm_per_sm<double>(shape, h->p.n_orient);
+// Work decomposition of a variant: the replicas' tiles or blocks, the CTAs and (march) the first
+// work item of each CTA.
+struct MpmPlan {
+    std::vector<hmc::MpmSched> sched;
+    std::vector<long long> cuts;
+    int grid = 1;
+};
+
+MpmPlan plan_mpm(const hmc_handle *h, int variant, int per_sm_limit) {
+    MpmPlan P;
+    P.sched.resize(h->R + 1);
+    const bool block = hmc::mpm_is_block(variant);
+    long long off = 0;
+    for (int r = 0; r <= h->R; ++r) {
+        hmc::MpmSched &S = P.sched[r];
+        S = hmc::MpmSched{};
+        S.off = off;
+        if (r == h->R) break;
+        const RepHost &R = h->reps[r];
+        int o[3] = {1, 1, 1};
+        patch_of(variant, R, o);
+        S.ox = o[0];
+        S.oy = o[1];
+        S.oz = o[2];
+        S.tiles_x = (R.nbx + o[0] - 1) / o[0];
+        S.tiles_y = (R.nby + o[1] - 1) / o[1];
+        S.tiles_z = (R.nbz + o[2] - 1) / o[2];
+        off += (long long)S.tiles_x * S.tiles_y * (block ? S.tiles_z : R.nbz);
+    }
+    if (block) {
+        P.grid = (int)off;
+        return P;
+    }
+    // March: a CTA that starts or enters a tile computes one plane of cells more than it owns of
+    // nodes.  With at most K planes of cells per CTA, filling the CTAs in order needs the fewest of
+    // them; take the smallest K that the resident CTAs hold.  (At 128^3 the even split left CTAs of
+    // 8 planes beside 6; now none has more than 6.)
+    int per_sm = h->p.precision == HMC_FP32 ? hmc::mpm_per_sm<float>(variant, h->p.n_orient)
+                                            : hmc::mpm_per_sm<double>(variant, h->p.n_orient);
     if (per_sm_limit > 0 && per_sm > per_sm_limit) per_sm = per_sm_limit;
-    long long g = (long long)per_sm * h->num_sms;
-    const long long cap = (h->mpm_total + min_planes - 1) / min_planes;
-    if (g > cap) g = cap;
-    return (int)(g < 1 ? 1 : g);
+    const long long slots = (long long)per_sm * h->num_sms;
+    auto fill = [&](long long K, std::vector<long long> *cuts) {
+        long long ctas = 1, room = K, w = 0;
+        if (cuts) cuts->assign(1, 0);
+        for (int r = 0; r < h->R; ++r) {
+            const long long planes = h->reps[r].nbz, tiles = (long long)P.sched[r].tiles_x * P.sched[r].tiles_y;
+            for (long long t = 0; t < tiles; ++t)
+                for (long long left = planes; left > 0;) {
+                    if (room < 2) {
+                        ++ctas;
+                        room = K;
+                        if (cuts) cuts->push_back(w);
+                    }
+                    const long long n = std::min(left, room - 1);
+                    room -= n + 1;
+                    left -= n;
+                    w += n;
+                }
+        }
+        if (cuts) cuts->push_back(w);
+        return ctas;
+    };
+    long long lo = 2, hi = 2 * off + 2;
+    while (lo < hi) {
+        const long long K = (lo + hi) / 2;
+        if (fill(K, nullptr) <= slots)
+            hi = K;
+        else
+            lo = K + 1;
+    }
+    P.grid = (int)fill(lo, &P.cuts);
+    // Long ranges: an even split over every resident CTA, unless it leaves one noticeably longer (at
+    // 256^3, 36 of 37 planes, the filled form needs 299 of 304 CTAs and its step took 101 us against 100)
+    if (lo >= 16 && P.grid < slots) {
+        P.grid = (int)slots;
+        P.cuts.resize(slots + 1);
+        for (long long c = 0; c <= slots; ++c) P.cuts[c] = off * c / slots;
+    }
+    return P;
+}
+
+hmc_status apply_plan(hmc_handle *h, int variant, const MpmPlan &P) {
+    HMC_CK(h, cudaStreamSynchronize(h->stream), "sync");
+    HMC_CK(h, cudaMemcpy(h->d_sched, P.sched.data(), sizeof(hmc::MpmSched) * P.sched.size(), cudaMemcpyHostToDevice),
+           "schedule upload");
+    if (!P.cuts.empty())
+        HMC_CK(h, cudaMemcpy(h->d_cuts, P.cuts.data(), sizeof(long long) * P.cuts.size(), cudaMemcpyHostToDevice),
+               "schedule upload");
+    h->mpm_shape = variant;
+    h->mpm_grid = P.grid;
+    return HMC_OK;
 }
 
 std::string tune_signature(const hmc_handle *h) {
@@ -645,12 +747,12 @@ std::string tune_signature(const hmc_handle *h) {
 // Every candidate computes bit-identical results: the per-cell arithmetic
 // (explicitly rounded, in one order, paired or not) and the order of each
 // node's force sum do not depend on the variant.
-hmc_status tune_mpm(hmc_handle *h, bool enabled, int &best_shape, int &best_grid) {
+hmc_status tune_mpm(hmc_handle *h, bool enabled, int &best_limit) {
     hmc_status s = HMC_OK;
-    best_shape = hmc::MPM_16x16;
-    if ((s = upload_sched(h, best_shape)) != HMC_OK) return s;
-    best_grid = grid_for_shape(h, best_shape, 0);
-    if (!enabled) return HMC_OK;
+    int best_variant = 0;
+    best_limit = 0;
+    MpmPlan best_plan = plan_mpm(h, best_variant, 0);
+    if (!enabled) return apply_plan(h, best_variant, best_plan);
     const size_t nb = node_bytes(h);
     void *uo = nullptr, *vs = nullptr;
     HMC_CK(h, cudaMalloc(&uo, nb), "autotune scratch");
@@ -663,36 +765,34 @@ hmc_status tune_mpm(hmc_handle *h, bool enabled, int &best_shape, int &best_grid
     cudaEventCreate(&e1);
     float best = 1e30f;
     cudaError_t err = cudaMemcpyAsync(vs, h->v, nb, cudaMemcpyDeviceToDevice, h->stream);
-    const int nvariants = hmc::mpm_nvariants(h->p.precision == HMC_FP32);
-    for (int shape = 0; shape < nvariants && err == cudaSuccess && s == HMC_OK; ++shape) {
-        if ((s = upload_sched(h, shape)) != HMC_OK) break;
-        // full occupancy and one CTA per SM with at least four planes per CTA, then (small grids)
-        // full occupancy with at least two planes and with at least one
-        std::vector<int> tried;
-        for (int cand = 0; cand < 4; ++cand) {
-            const int grid = grid_for_shape(h, shape, cand == 1 ? 1 : 0, cand < 2 ? 4 : cand == 2 ? 2 : 1);
-            if (std::find(tried.begin(), tried.end(), grid) != tried.end()) continue;
-            tried.push_back(grid);
-            const int saved_grid = h->mpm_grid;
-            h->mpm_grid = grid;
+    for (int v = 0; v < hmc::MPM_NVARIANTS && err == cudaSuccess && s == HMC_OK; ++v) {
+        // a march with every resident CTA and with one per SM; the block form where its blocks are
+        // few enough for it to be in question
+        for (int limit = 0; limit < (hmc::mpm_is_block(v) ? 1 : 2); ++limit) {
+            const MpmPlan P = plan_mpm(h, v, limit);
+            if (hmc::mpm_is_block(v) && P.grid > 16 * h->num_sms) continue;
+            if ((s = apply_plan(h, v, P)) != HMC_OK) break;
             auto launch = [&]() {
                 return h->p.precision == HMC_FP32
-                           ? hmc::launch_mpm_step<float>(mpm_args<float>(h, h->u[h->cur], uo, vs), shape, h->stream)
-                           : hmc::launch_mpm_step<double>(mpm_args<double>(h, h->u[h->cur], uo, vs), shape,
-                                                          h->stream);
+                           ? hmc::launch_mpm_step<float>(mpm_args<float>(h, h->u[h->cur], uo, vs), v, h->stream)
+                           : hmc::launch_mpm_step<double>(mpm_args<double>(h, h->u[h->cur], uo, vs), v, h->stream);
             };
             err = launch();
-            if (err == cudaSuccess) err = cudaEventRecord(e0, h->stream);
-            for (int k = 0; k < 3 && err == cudaSuccess; ++k) err = launch();
-            if (err == cudaSuccess) err = cudaEventRecord(e1, h->stream);
-            if (err == cudaSuccess) err = cudaEventSynchronize(e1);
-            float ms = 0;
-            if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
-            h->mpm_grid = saved_grid;
+            float ms = 1e30f;
+            for (int rep = 0; rep < 2 && err == cudaSuccess; ++rep) {   // the better of two runs of four
+                float t = 0;
+                err = cudaEventRecord(e0, h->stream);
+                for (int k = 0; k < 4 && err == cudaSuccess; ++k) err = launch();
+                if (err == cudaSuccess) err = cudaEventRecord(e1, h->stream);
+                if (err == cudaSuccess) err = cudaEventSynchronize(e1);
+                if (err == cudaSuccess) err = cudaEventElapsedTime(&t, e0, e1);
+                ms = std::min(ms, t);
+            }
             if (err == cudaSuccess && ms < best) {
                 best = ms;
-                best_shape = shape;
-                best_grid = grid;
+                best_variant = v;
+                best_limit = limit;
+                best_plan = P;
             }
             if (err != cudaSuccess) break;
         }
@@ -704,7 +804,7 @@ hmc_status tune_mpm(hmc_handle *h, bool enabled, int &best_shape, int &best_grid
     cudaFree(vs);
     if (s != HMC_OK) return s;
     if (err != cudaSuccess) return cuda_fail(h, err, "autotune");
-    return upload_sched(h, best_shape);
+    return apply_plan(h, best_variant, best_plan);
 }
 
 // Pick the sweep CTA size (256 threads per 256-block tile, or the tile split over two
@@ -811,39 +911,33 @@ hmc_status ensure_tuned(hmc_handle *h) {
     const bool enabled = !(env && env[0] == '0');
     const char *forced = std::getenv("HMC_MPM_SHAPE");
     const char *forced_cta = std::getenv("HMC_SWEEP_CTA");
-    const int nvar = hmc::mpm_nvariants(h->p.precision == HMC_FP32);
-    const bool force_mpm = forced && forced[0] >= '0' && forced[0] < '0' + nvar && forced[1] == 0;
+    const bool force_mpm = forced && forced[0] >= '0' && forced[0] < '0' + hmc::MPM_NVARIANTS && forced[1] == 0;
     const bool force_cta = forced_cta && (std::string(forced_cta) == "128" || std::string(forced_cta) == "256");
     const std::string sig = tune_signature(h);
     if (!force_mpm && !force_cta) {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         auto it = g_tune_cache.find(sig);
         if (it != g_tune_cache.end()) {
-            if ((s = upload_sched(h, it->second.mpm_shape)) != HMC_OK) return s;
-            h->mpm_shape = it->second.mpm_shape;
-            h->mpm_grid = it->second.mpm_grid;
+            const int v = it->second.mpm_variant;
+            if ((s = apply_plan(h, v, plan_mpm(h, v, it->second.mpm_limit))) != HMC_OK) return s;
             h->sweep_cta = it->second.sweep_cta;
             h->store_eff = it->second.store;
             h->tuned = true;
             return HMC_OK;
         }
     }
-    int shape = 0, grid = 1;
-    if (force_mpm) {
-        shape = forced[0] - '0';
-        if ((s = upload_sched(h, shape)) != HMC_OK) return s;
-        grid = grid_for_shape(h, shape, 0);
-    } else if ((s = tune_mpm(h, enabled, shape, grid)) != HMC_OK) {
-        return s;
-    }
-    h->mpm_shape = shape;
-    h->mpm_grid = grid;
+    int limit = 0;
+    if (force_mpm)
+        s = apply_plan(h, forced[0] - '0', plan_mpm(h, forced[0] - '0', 0));
+    else
+        s = tune_mpm(h, enabled, limit);
+    if (s != HMC_OK) return s;
     if ((s = tune_sweeps(h, enabled && !force_cta)) != HMC_OK) return s;
     if (force_cta) h->sweep_cta = std::atoi(forced_cta);
     h->tuned = true;
     if (!force_mpm && !force_cta) {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
-        g_tune_cache[sig] = TuneResult{h->mpm_shape, h->mpm_grid, h->sweep_cta, h->store_eff};
+        g_tune_cache[sig] = TuneResult{h->mpm_shape, limit, h->sweep_cta, h->store_eff};
     }
     return HMC_OK;
 }
@@ -1023,6 +1117,7 @@ hmc_status hmc_create_batch(const hmc_params *params, int32_t n_replicas, hmc_ha
         {(void **)&h->d_reps, sizeof(hmc::Replica) * (size_t)h->R, "replica table"},
         {(void **)&h->d_cta_rep, sizeof(int) * (size_t)h->nctas, "CTA table"},
         {(void **)&h->d_sched, sizeof(hmc::MpmSched) * (size_t)(h->R + 1), "MPM schedule"},
+        {(void **)&h->d_cuts, sizeof(long long) * (size_t)(32 * h->num_sms + 1), "MPM schedule"},
     };
     for (auto &a : allocs) {
         if ((e = cudaMalloc(a.ptr, a.bytes)) != cudaSuccess) return bail(cuda_fail(h, e, a.what));
@@ -1108,9 +1203,8 @@ hmc_status hmc_create_batch(const hmc_params *params, int32_t n_replicas, hmc_ha
         const int per_sm = p->precision == HMC_FP32 ? hmc::zone_per_sm<float>() : hmc::zone_per_sm<double>();
         h->zone_grid = h->num_sms * per_sm;
     }
-    hmc_status s = upload_sched(h, h->mpm_shape);
+    hmc_status s = apply_plan(h, h->mpm_shape, plan_mpm(h, h->mpm_shape, 0));
     if (s != HMC_OK) return bail(s);
-    h->mpm_grid = grid_for_shape(h, h->mpm_shape, 0);
     *out = h;
     return HMC_OK;
 }

@@ -92,6 +92,29 @@ __host__ __device__ __forceinline__ int wrapi(int a, int n) {
     return a < 0 ? a + n : a;
 }
 
+// The block form of the MPM step: block b of a replica owns the nodes from (i0, j0, k0), of which
+// there are (W-1)(H-1)(D-1), and computes the W x H x D cells around them; the nodes of those cells
+// lie W + 1 a row, H + 1 rows a plane.
+struct BlockPlace {
+    int i0, j0, k0, W, H, D;
+    __device__ __forceinline__ BlockPlace(const MpmSched &S, const Replica &R, int b) {
+        const int tx = b % S.tiles_x, t = b / S.tiles_x;
+        i0 = tx * S.ox;
+        j0 = t % S.tiles_y * S.oy;
+        k0 = t / S.tiles_y * S.oz;
+        W = min(S.ox, R.nbx - i0) + 1;
+        H = min(S.oy, R.nby - j0) + 1;
+        D = min(S.oz, R.nbz - k0) + 1;
+    }
+    // node t of the block's cells in the batch, -1 beyond them
+    __device__ __forceinline__ long long node(const Replica &R, int t) const {
+        const int P = W + 1, Q = H + 1, i = t % P, j = t / P % Q, k = t / (P * Q);
+        if (k > D) return -1;
+        return R.blk_off + wrapi(i0 - 1 + i, R.nbx) +
+               (long long)R.nbx * (wrapi(j0 - 1 + j, R.nby) + (long long)R.nby * wrapi(k0 - 1 + k, R.nbz));
+    }
+};
+
 // ---------------------------------------------------------------------------
 // One MPM cell = one 2x2x2 block with its eight material points at local
 // coordinates 1/4 and 3/4 of the cell edge h = 2 voxels.  Trilinear shape

@@ -90,11 +90,12 @@ static_assert(sizeof(Replica) % 16 == 0, "Replica must be a whole number of 16 B
 
 constexpr int BLOCK_THREADS = 256;   // threads of the sweep and stress CTAs
 
-// MPM work decomposition of one replica for the chosen patch shape: tiles of
-// owned nodes per edge and the first (tile-major, plane-minor) work item.
+// MPM work decomposition of one replica: most nodes that a tile or block owns per edge, their
+// numbers, and the first work item (march: tile-major, plane-minor; block form: a block).
 struct MpmSched {
-    int tiles_x, tiles_y;
-    long long plane_off;      // entry nrep holds the total
+    int ox, oy, oz;
+    int tiles_x, tiles_y, tiles_z;
+    long long off;            // entry nrep holds the total
 };
 
 template <typename T>
@@ -102,7 +103,7 @@ struct MpmArgs {
     const Replica *reps;
     const MpmSched *sched;   // nrep + 1 entries
     int nrep;
-    long long total;         // work items of the whole batch
+    const long long *cuts;   // march: first work item of every CTA, then the total (grid + 1)
     const uint4 *spins;
     const T *u_in;
     T *u_out;
@@ -113,10 +114,11 @@ struct MpmArgs {
     int cexp;                // ... entry = round(C' 2^cexp), x the signed low half, y the high half
     int nq;                  // orientations (the FP32 step stages cubw in shared memory up to MPM_STAB_MAX)
     T dt, dt_over_m, keep;   // keep = 1 - damping
-    int grid;                // persistent CTAs
+    int grid;                // CTAs
 };
 
 constexpr int MPM_STAB_MAX = 1024;   // orientations whose FP32 table the MPM step holds in shared memory
+constexpr int MPM_STAB_BLOCK = 256;  // ... in the block form
 
 // The plain (unfused, incremental) FP64 step of a single replica: point stresses
 // sig[6][nblk][8] (component, cell, local point a + 2b + 4c) and cell corner forces
@@ -206,14 +208,14 @@ struct ZoneArgs {
     T J, kT;
 };
 
-// MPM patch shapes (cells per patch edge; owned nodes = cells - 1).  A variant
-// index v in [0, 2 * MPM_NSHAPES) selects shape v % MPM_NSHAPES; v >= MPM_NSHAPES
-// selects the paired-FMA Hooke product (FP32 only); v = MPM_TWO_CELL is the
-// 16x16 shape with two cells per thread in paired FP32 registers (FP32 only).
-enum MpmShape { MPM_16x16 = 0, MPM_32x8 = 1, MPM_8x32 = 2, MPM_NSHAPES = 3, MPM_TWO_CELL = 6 };
-inline int mpm_nvariants(bool fp32) { return fp32 ? MPM_TWO_CELL + 1 : MPM_NSHAPES; }
-int mpm_shape_cx(int shape);
-int mpm_shape_cy(int shape);
+// MPM variants.  March with owned patches of 0: 15x15, 1: 31x7, 2: 7x31 nodes (cut off at the
+// high edges), 3: as few patches as can be of even size, 4: as few cells as can be; block form with
+// 5: blocks of at most 256 cells, 6: at most MPM_SMALL_BLOCK cells.
+enum { MPM_FIT = 3, MPM_BLOCK = 5, MPM_NVARIANTS = 7 };
+constexpr int MPM_THREADS = 256;     // threads of a step's CTA = most cells of a patch plane or block
+constexpr int MPM_SMALL_BLOCK = 96;  // ... of the small-block form
+constexpr int MPM_NODES = 304;       // most nodes of a patch's plane, (W+1)(H+1)
+inline bool mpm_is_block(int variant) { return variant >= MPM_BLOCK; }
 
 // Launchers (return cudaGetLastError of the launch).
 template <typename T>

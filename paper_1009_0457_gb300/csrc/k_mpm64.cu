@@ -45,13 +45,20 @@ struct FxHalf {   // 16 bytes: x and y, or z and the exponent
     ll a, b;
 };
 
-template <int CX, int CY>
-struct alignas(16) FxSmem {
-    static constexpr int NX = CX + 1, NY = CY + 1;
-    FxHalf uxy[3][NY][NX], uze[3][NY][NX];   // node planes
-    FxHalf fxy[2][8][CY][CX], fze[2][8][CY][CX];   // (buffer) cell contributions to corner I + 2J + 4K
-    FxHalf eb[3];                            // mean strain, m * 2^8 aligned to ebe
-    int ebe;
+struct FxMean {                              // mean strain, m * 2^8 aligned to the exponent e
+    FxHalf eb[3];
+    int e;
+};
+struct alignas(16) FxMarchSmem {
+    FxHalf uxy[3][MPM_NODES], uze[3][MPM_NODES];             // node planes, W + 1 nodes a row
+    FxHalf fxy[2][8][MPM_THREADS], fze[2][8][MPM_THREADS];   // (buffer) contributions to corner I + 2J + 4K
+    FxMean m;
+};
+template <int THREADS>
+struct alignas(16) FxBlockSmem {
+    FxHalf uxy[2 * THREADS], uze[2 * THREADS];
+    FxHalf fxy[8][THREADS], fze[8][THREADS];
+    FxMean m;
 };
 
 __device__ __forceinline__ int dexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
@@ -253,45 +260,141 @@ __device__ __forceinline__ Fx3 fx_sum(const ll (&x)[3][N], const int (&e)[N]) {
     return r;
 }
 
-template <int CX, int CY>
-__global__ void __launch_bounds__(CX *CY, 1) k_mpm_fixed(MpmArgs<double> a) {
-    constexpr int OX = CX - 1, OY = CY - 1, NX = CX + 1, NN = (CX + 1) * (CY + 1), NTHR = CX * CY;
-    constexpr int PER = (NN + NTHR - 1) / NTHR;
-    using Smem = FxSmem<CX, CY>;
+// a node's displacement into shared memory, its components aligned to the largest of them
+__device__ __forceinline__ void fx_put(FxHalf *xy, FxHalf *ze, int t, const double (&u)[3]) {
+    const int E = max(dexp(u[0]), max(dexp(u[1]), dexp(u[2])));
+    xy[t] = FxHalf{dfix<3>(u[0], E), dfix<3>(u[1], E)};
+    ze[t] = FxHalf{dfix<3>(u[2], E), (ll)E};
+}
+
+__device__ __forceinline__ void fx_mean(FxMean &m, const DevState *st) {   // by one thread
+    double e[6];
+    int E = 0;
+    for (int i = 0; i < 6; ++i) {
+        e[i] = st->ebar[i];
+        E = max(E, dexp(e[i]));
+    }
+    for (int i = 0; i < 3; ++i) m.eb[i] = FxHalf{dfix<8>(e[2 * i], E), dfix<8>(e[2 * i + 1], E)};
+    m.e = E;
+}
+
+// a cell: its corners lie at n0 and n1 (lower and upper plane), P nodes a row; returns its exponent
+__device__ __forceinline__ int fx_corners(const FxHalf *xy0, const FxHalf *ze0, const FxHalf *xy1, const FxHalf *ze1,
+                                          int P, const FxMean &m, ll (&u)[8][3], ll (&eb)[6]) {
+    int ne[8], E = m.e;
+#pragma unroll
+    for (int n = 0; n < 8; ++n) {
+        const int o = (n & 1) + (n & 2 ? P : 0);
+        const FxHalf p = (n & 4 ? xy1 : xy0)[o], q = (n & 4 ? ze1 : ze0)[o];
+        u[n][0] = p.a;
+        u[n][1] = p.b;
+        u[n][2] = q.a;
+        ne[n] = (int)q.b;
+        E = max(E, ne[n]);
+    }
+#pragma unroll
+    for (int n = 0; n < 8; ++n) {
+        const int s = min(E - ne[n], 63);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) u[n][d] >>= s;
+    }
+    const int se = min(E - m.e, 63);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const FxHalf t = m.eb[i];
+        eb[2 * i] = t.a >> se;
+        eb[2 * i + 1] = t.b >> se;
+    }
+    return E;
+}
+
+// the four cells (i-1, j-1), (i, j-1), (i-1, j), (i, j) of one plane, W cells a row, on their common
+// node: they see it as corner c + 3, c + 2, c + 1, c
+template <int THREADS>
+__device__ __forceinline__ Fx3 fx_sum4(const FxHalf (&xy)[8][THREADS], const FxHalf (&ze)[8][THREADS], int c, int t, int W) {
+    const FxHalf a3 = xy[c + 3][t - W - 1], b3 = ze[c + 3][t - W - 1], a2 = xy[c + 2][t - W], b2 = ze[c + 2][t - W];
+    const FxHalf a1 = xy[c + 1][t - 1], b1 = ze[c + 1][t - 1], a0 = xy[c][t], b0 = ze[c][t];
+    const ll x[3][4] = {{a3.a, a2.a, a1.a, a0.a}, {a3.b, a2.b, a1.b, a0.b}, {b3.a, b2.a, b1.a, b0.a}};
+    const int e[4] = {(int)b3.b, (int)b2.b, (int)b1.b, (int)b0.b};
+    return fx_sum<4>(x, e);
+}
+
+// the update of a node whose force is not finite or whose scale leaves the normal range; kept out of
+// line, since its FP64 multiplications would otherwise be formed for every node (6 % of a step)
+__device__ __noinline__ void fx_update_any(ll x, ll y, ll z, int e, double fscale, int shift, double keep, double dt,
+                                           const double *uold, const double *vold, double *u, double *v) {
+    for (int d = 0; d < 3; ++d) {
+        const double F = e >= 2047 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn((double)(d == 0 ? x : d == 1 ? y : z), shift);
+        const double vn = rfma(fscale, F, rmul(keep, vold[d]));
+        v[d] = vn;
+        u[d] = rfma(dt, vn, uold[d]);
+    }
+}
+
+// velocity and displacement of a node from the force sums of the cells below and above it
+struct FxUpdate {
+    double fscale, dt, keep;   // fscale = -dt / (32 m)
+    int cexp, fexp;
+    __device__ __forceinline__ explicit FxUpdate(const MpmArgs<double> &a)
+        : fscale(-a.dt_over_m * 0.03125), dt(a.dt), keep(a.keep), cexp(a.cexp) {
+        // the force integers of exponent E are 2^(E - cexp - 1013) of the FP32 step's units
+        fexp = dexp(fscale) ? dexp(fscale) - cexp - 1013 : -10000;   // (subnormal: the general form)
+    }
+    __device__ __forceinline__ void operator()(const Fx3 &lo, const Fx3 &hi, const double (&uold)[3],
+                                               const double (&vold)[3], double *u, double *v) const {
+        const ll x[3][2] = {{lo.v[0], hi.v[0]}, {lo.v[1], hi.v[1]}, {lo.v[2], hi.v[2]}};
+        const int e[2] = {lo.e, hi.e};
+        const Fx3 F = fx_sum<2>(x, e);
+        const int ef = fexp + F.e;   // exponent of fscale times the force's unit
+        if ((unsigned)(ef - 1) < 2045u && F.e < 2047) {
+            const double fs = __hiloint2double((__double2hiint(fscale) & 0x800fffff) | (ef << 20), __double2loint(fscale));
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const double vn = rfma(fs, (double)F.v[d], rmul(keep, vold[d]));
+                v[d] = vn;
+                u[d] = rfma(dt, vn, uold[d]);
+            }
+        } else {
+            fx_update_any(F.v[0], F.v[1], F.v[2], F.e, fscale, F.e - cexp - 1013, keep, dt, uold, vold, u, v);
+        }
+    }
+};
+
+__global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a) {
+    constexpr int PER = (MPM_NODES + MPM_THREADS - 1) / MPM_THREADS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
+    FxMarchSmem &sm = *reinterpret_cast<FxMarchSmem *>(smem_raw);
     const int tid = threadIdx.x;
-    const double fscale = -a.dt_over_m * 0.03125;          // -dt / (32 m)
-    // the force integers of exponent E are 2^(E - cexp - 1013) (16/9/.. units as in the FP32 step)
-    const int fexp = dexp(fscale) ? dexp(fscale) - a.cexp - 1013 : -10000;   // (subnormal: the general form)
+    const FxUpdate update(a);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    long long w = a.total * blockIdx.x / gridDim.x;
-    const long long wend = a.total * (blockIdx.x + 1) / gridDim.x;
+    long long w = a.cuts[blockIdx.x];
+    const long long wend = a.cuts[blockIdx.x + 1];
     int r = 0;
     while (w < wend) {
-        while (a.sched[r + 1].plane_off <= w) ++r;
+        while (a.sched[r + 1].off <= w) ++r;
         const Replica &R = a.reps[r];
         const MpmSched &SC = a.sched[r];
         const int nbx = R.nbx, nby = R.nby, nbz = R.nbz;
-        const long long lw = w - SC.plane_off;
+        const long long lw = w - SC.off;
         const int tile = (int)(lw / nbz);
         const int k0 = (int)(lw - (long long)tile * nbz);
-        const long long rem = min(wend, a.sched[r + 1].plane_off) - w;
+        const long long rem = min(wend, a.sched[r + 1].off) - w;
         const int kend = (int)min((long long)nbz, (long long)k0 + rem);
         w += kend - k0;
-        const int i0 = (tile % SC.tiles_x) * OX, j0 = (tile / SC.tiles_x) * OY;
-        const int W = min(CX, nbx - i0 + 1), H = min(CY, nby - j0 + 1);
+        const int i0 = (tile % SC.tiles_x) * SC.ox, j0 = (tile / SC.tiles_x) * SC.oy;
+        const int W = min(SC.ox, nbx - i0) + 1, H = min(SC.oy, nby - j0) + 1, P = W + 1;
         const int lci = tid % W, lcj = tid / W;
         const bool need = tid < W * H;
         const bool own = need && lci >= 1 && lcj >= 1;
         const int plane = nbx * nby;
         const long long col = R.blk_off + wrapi(i0 - 1 + lci, nbx) + nbx * wrapi(j0 - 1 + lcj, nby);
-        int ncol[PER];   // the tile's nodes that this thread loads, as (i + nbx j) in a node plane
+        const int nd = lci + P * lcj;
+        int ncol[PER];   // the patch's nodes that this thread loads, as (i + nbx j) in a node plane, -1 beyond it
 #pragma unroll
         for (int m = 0; m < PER; ++m) {
-            const int t = tid + m * NTHR;
-            ncol[m] = wrapi(i0 - 1 + t % NX, nbx) + nbx * wrapi(j0 - 1 + t / NX, nby);
+            const int t = tid + m * MPM_THREADS;
+            ncol[m] = t < P * (H + 1) ? wrapi(i0 - 1 + t % P, nbx) + nbx * wrapi(j0 - 1 + t / P, nby) : -1;
         }
         double pl[PER][3];
         auto fetch = [&](int k) {   // node plane k, -1 <= k <= nbz (periodic in z)
@@ -299,36 +402,21 @@ __global__ void __launch_bounds__(CX *CY, 1) k_mpm_fixed(MpmArgs<double> a) {
             const double *base = a.u_in + 3 * (R.blk_off + (long long)plane * gk);
 #pragma unroll
             for (int m = 0; m < PER; ++m)
-                if (tid + m * NTHR < NN)
+                if (ncol[m] >= 0)
 #pragma unroll
                     for (int d = 0; d < 3; ++d) pl[m][d] = __ldg(base + 3 * ncol[m] + d);
         };
         auto store = [&](int b) {
 #pragma unroll
-            for (int m = 0; m < PER; ++m) {
-                const int t = tid + m * NTHR;
-                if (t < NN) {
-                    const int E = max(dexp(pl[m][0]), max(dexp(pl[m][1]), dexp(pl[m][2])));
-                    (&sm.uxy[b][0][0])[t] = FxHalf{dfix<3>(pl[m][0], E), dfix<3>(pl[m][1], E)};
-                    (&sm.uze[b][0][0])[t] = FxHalf{dfix<3>(pl[m][2], E), (ll)E};
-                }
-            }
+            for (int m = 0; m < PER; ++m)
+                if (ncol[m] >= 0) fx_put(sm.uxy[b], sm.uze[b], tid + m * MPM_THREADS, pl[m]);
         };
         int b0 = 0, b1 = 1, b2 = 2, fb = 0;
         fetch(k0 - 1);
         store(b0);
         fetch(k0);
         store(b1);
-        if (tid == 0) {
-            double e[6];
-            int E = 0;
-            for (int i = 0; i < 6; ++i) {
-                e[i] = R.st->ebar[i];
-                E = max(E, dexp(e[i]));
-            }
-            for (int i = 0; i < 3; ++i) sm.eb[i] = FxHalf{dfix<8>(e[2 * i], E), dfix<8>(e[2 * i + 1], E)};
-            sm.ebe = E;
-        }
+        if (tid == 0) fx_mean(sm.m, R.st);
         uint4 sp = need ? __ldg(a.spins + col + (long long)plane * wrapi(k0 - 1, nbz)) : make_uint4(0, 0, 0, 0);
         __syncthreads();
 
@@ -353,78 +441,25 @@ __global__ void __launch_bounds__(CX *CY, 1) k_mpm_fixed(MpmArgs<double> a) {
             const bool more = kk + 1 < kend;
             if (more) fetch(kk + 2);
             if (need) {
-                ll u[8][3];
-                int ne[8], E = sm.ebe;
-#pragma unroll
-                for (int n = 0; n < 8; ++n) {
-                    const int b = n >> 2 ? b1 : b0, j = lcj + ((n >> 1) & 1), i = lci + (n & 1);
-                    const FxHalf p = sm.uxy[b][j][i], q = sm.uze[b][j][i];
-                    u[n][0] = p.a;
-                    u[n][1] = p.b;
-                    u[n][2] = q.a;
-                    ne[n] = (int)q.b;
-                    E = max(E, ne[n]);
-                }
-#pragma unroll
-                for (int n = 0; n < 8; ++n) {
-                    const int s = min(E - ne[n], 63);
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) u[n][d] >>= s;
-                }
-                ll eb[6];
-                const int se = min(E - sm.ebe, 63);
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    const FxHalf t = sm.eb[i];
-                    eb[2 * i] = t.a >> se;
-                    eb[2 * i + 1] = t.b >> se;
-                }
-                ll f[8][3];
+                ll u[8][3], eb[6], f[8][3];
+                const int E = fx_corners(sm.uxy[b0] + nd, sm.uze[b0] + nd, sm.uxy[b1] + nd, sm.uze[b1] + nd, P, sm.m, u, eb);
                 fx_cell(u, eb, sp, a.cfix, f);
 #pragma unroll
                 for (int n = 0; n < 8; ++n) {
-                    sm.fxy[fb][n][lcj][lci] = FxHalf{f[n][0], f[n][1]};
-                    sm.fze[fb][n][lcj][lci] = FxHalf{f[n][2], (ll)E};
+                    sm.fxy[fb][n][tid] = FxHalf{f[n][0], f[n][1]};
+                    sm.fze[fb][n][tid] = FxHalf{f[n][2], (ll)E};
                 }
             }
             if (more) store(b2);   // buffer b2 was last read before the previous barrier
             __syncthreads();
             if (own) {
-                auto sum4 = [&](int c) {
-                    const FxHalf a3 = sm.fxy[fb][c + 3][lcj - 1][lci - 1], b3 = sm.fze[fb][c + 3][lcj - 1][lci - 1];
-                    const FxHalf a2 = sm.fxy[fb][c + 2][lcj - 1][lci], b2 = sm.fze[fb][c + 2][lcj - 1][lci];
-                    const FxHalf a1 = sm.fxy[fb][c + 1][lcj][lci - 1], b1 = sm.fze[fb][c + 1][lcj][lci - 1];
-                    const FxHalf a0 = sm.fxy[fb][c][lcj][lci], b0 = sm.fze[fb][c][lcj][lci];
-                    const ll x[3][4] = {{a3.a, a2.a, a1.a, a0.a}, {a3.b, a2.b, a1.b, a0.b}, {b3.a, b2.a, b1.a, b0.a}};
-                    const int e[4] = {(int)b3.b, (int)b2.b, (int)b1.b, (int)b0.b};
-                    return fx_sum<4>(x, e);
-                };
                 if (kk >= k0) {
-                    const Fx3 up4 = sum4(0);
-                    const ll x2[3][2] = {{acc.v[0], up4.v[0]}, {acc.v[1], up4.v[1]}, {acc.v[2], up4.v[2]}};
-                    const int e2[2] = {acc.e, up4.e};
-                    const Fx3 F = fx_sum<2>(x2, e2);
-                    const int ef = fexp + F.e;   // exponent of the product's scale
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) {
-                        const double Fd = (double)F.v[d], kv = rmul(a.keep, vold[d]);
-                        double vn;
-                        if (F.e >= 2047)
-                            vn = __longlong_as_double(0x7ff8000000000000ll);
-                        else if ((unsigned)(ef - 1) < 2045u)
-                            vn = rfma(__hiloint2double((__double2hiint(fscale) & 0x800fffff) | (ef << 20),
-                                                       __double2loint(fscale)),
-                                      Fd, kv);
-                        else
-                            vn = rfma(fscale, scalbn(Fd, F.e - a.cexp - 1013), kv);
-                        vp[d] = vn;
-                        up[d] = rfma(a.dt, vn, uold[d]);
-                    }
+                    update(acc, fx_sum4(sm.fxy[fb], sm.fze[fb], 0, tid, W), uold, vold, up, vp);
                     vp += pstride;
                     up += pstride;
                     uip += pstride;
                 }
-                acc = sum4(4);
+                acc = fx_sum4(sm.fxy[fb], sm.fze[fb], 4, tid, W);
             }
             // one barrier a plane: the next plane writes the other force buffer and the node plane that
             // was last read before this one's barrier
@@ -439,52 +474,109 @@ __global__ void __launch_bounds__(CX *CY, 1) k_mpm_fixed(MpmArgs<double> a) {
     }
 }
 
-template <int CX, int CY>
-cudaError_t prepare_t() {
-    return cudaFuncSetAttribute(k_mpm_fixed<CX, CY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sizeof(FxSmem<CX, CY>));
+// The block form (k_mpm.cu): one block per CTA, every cell at once.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS > 128 ? 1 : 2) k_mpm_fixed_block(MpmArgs<double> a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    FxBlockSmem<THREADS> &sm = *reinterpret_cast<FxBlockSmem<THREADS> *>(smem_raw);
+    const int tid = threadIdx.x;
+    const FxUpdate update(a);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    int r = 0;
+    while (a.sched[r + 1].off <= blockIdx.x) ++r;
+    const Replica &R = a.reps[r];
+    const MpmSched &SC = a.sched[r];
+    const BlockPlace B(SC, R, blockIdx.x - (int)SC.off);
+    const int W = B.W, H = B.H, P = W + 1, PP = P * (H + 1);
+    const int lci = tid % W, lcj = tid / W % H, lck = tid / (W * H);
+    const bool need = lck < B.D;
+    const bool own = need && lci >= 1 && lcj >= 1 && lck >= 1;
+    const long long at = R.blk_off + wrapi(B.i0 - 1 + lci, R.nbx) +
+                         (long long)R.nbx * (wrapi(B.j0 - 1 + lcj, R.nby) + (long long)R.nby * wrapi(B.k0 - 1 + lck, R.nbz));
+    long long node[2];
+#pragma unroll
+    for (int m = 0; m < 2; ++m) node[m] = B.node(R, tid + m * THREADS);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint4 sp = need ? __ldg(a.spins + at) : make_uint4(0, 0, 0, 0);
+    double uold[3] = {0, 0, 0}, vold[3] = {0, 0, 0};
+    if (own) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            vold[d] = a.v[3 * at + d];
+            uold[d] = __ldg(a.u_in + 3 * at + d);
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+        if (node[m] >= 0) {
+            const double *p = a.u_in + 3 * node[m];
+            const double u[3] = {__ldg(p), __ldg(p + 1), __ldg(p + 2)};
+            fx_put(sm.uxy, sm.uze, tid + m * THREADS, u);
+        }
+    if (tid == 0) fx_mean(sm.m, R.st);
+    __syncthreads();
+    if (need) {
+        ll u[8][3], eb[6], f[8][3];
+        const int nd = lci + P * lcj + PP * lck;
+        const int E = fx_corners(sm.uxy + nd, sm.uze + nd, sm.uxy + nd + PP, sm.uze + nd + PP, P, sm.m, u, eb);
+        fx_cell(u, eb, sp, a.cfix, f);
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            sm.fxy[n][tid] = FxHalf{f[n][0], f[n][1]};
+            sm.fze[n][tid] = FxHalf{f[n][2], (ll)E};
+        }
+    }
+    __syncthreads();
+    if (own)
+        update(fx_sum4(sm.fxy, sm.fze, 4, tid - W * H, W), fx_sum4(sm.fxy, sm.fze, 0, tid, W), uold, vold,
+               a.u_out + 3 * at, a.v + 3 * at);
 }
-template <int CX, int CY>
-int per_sm_t() {
+
+struct Form {   // kernel, threads, shared memory
+    void (*kernel)(MpmArgs<double>);
+    int threads;
+    size_t smem;
+};
+Form form_of(int variant) {
+    if (!mpm_is_block(variant)) return Form{k_mpm_fixed, MPM_THREADS, sizeof(FxMarchSmem)};
+    if (variant == MPM_BLOCK) return Form{k_mpm_fixed_block<MPM_THREADS>, MPM_THREADS, sizeof(FxBlockSmem<MPM_THREADS>)};
+    return Form{k_mpm_fixed_block<MPM_SMALL_BLOCK>, MPM_SMALL_BLOCK, sizeof(FxBlockSmem<MPM_SMALL_BLOCK>)};
+}
+
+}  // namespace
+
+cudaError_t mpm64_prepare() {
+    for (int v : {0, (int)MPM_BLOCK, MPM_BLOCK + 1}) {
+        const Form f = form_of(v);
+        const cudaError_t e = cudaFuncSetAttribute(f.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+template <>
+int mpm_per_sm<double>(int variant, int) {
+    const Form f = form_of(variant);
     int n = 1;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_mpm_fixed<CX, CY>, CX * CY,
-                                                                       sizeof(FxSmem<CX, CY>));
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f.kernel, f.threads, f.smem);
     return (e != cudaSuccess || n < 1) ? 1 : n;
 }
+
 // programmatic stream serialisation, as the FP32 step
-template <int CX, int CY>
-cudaError_t launch_t(const MpmArgs<double> &a, cudaStream_t s) {
+template <>
+cudaError_t launch_mpm_step<double>(const MpmArgs<double> &a, int variant, cudaStream_t s) {
+    const Form f = form_of(variant);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.grid);
-    cfg.blockDim = dim3(CX * CY);
-    cfg.dynamicSmemBytes = sizeof(FxSmem<CX, CY>);
+    cfg.blockDim = dim3(f.threads);
+    cfg.dynamicSmemBytes = f.smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_mpm_fixed<CX, CY>, a);
-}
-
-}  // namespace
-
-cudaError_t mpm64_prepare() {
-    cudaError_t e;
-    if ((e = prepare_t<16, 16>()) != cudaSuccess || (e = prepare_t<32, 8>()) != cudaSuccess) return e;
-    return prepare_t<8, 32>();
-}
-
-template <>
-int mpm_per_sm<double>(int shape, int) {
-    const int sh = shape % MPM_NSHAPES;
-    return sh == MPM_32x8 ? per_sm_t<32, 8>() : sh == MPM_8x32 ? per_sm_t<8, 32>() : per_sm_t<16, 16>();
-}
-
-template <>
-cudaError_t launch_mpm_step<double>(const MpmArgs<double> &a, int shape, cudaStream_t s) {
-    const int sh = shape % MPM_NSHAPES;
-    return sh == MPM_32x8 ? launch_t<32, 8>(a, s) : sh == MPM_8x32 ? launch_t<8, 32>(a, s) : launch_t<16, 16>(a, s);
+    return cudaLaunchKernelEx(&cfg, f.kernel, a);
 }
 
 }  // namespace hmc
