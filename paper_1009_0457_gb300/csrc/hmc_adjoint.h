@@ -17,14 +17,15 @@ struct AdjArgs {
     int nx, ny, nz, nbx, nby, nbz, nblk;
 };
 
+// adds the sums of P, T and D (times 2^10) to the partials and lam to the sum of the lambdas
 template <typename T>
-cudaError_t launch_adj_params(const AdjArgs<T> &a, const T *lam, const T *u, cudaStream_t s);
+cudaError_t launch_adj_params(const AdjArgs<T> &a, const T *lam, const T *u, T *lsum, T *lerr, cudaStream_t s);
+template <typename T>
+cudaError_t launch_adj_mean(const AdjArgs<T> &a, const T *lsum, const T *lerr, cudaStream_t s);
 template <typename T>
 cudaError_t launch_adj_terminal(const AdjArgs<T> &a, const T *u, const T *g, T gW, T *w, T *fcell, cudaStream_t s);
 template <typename T>
 cudaError_t launch_adj_gather(const AdjArgs<T> &a, const T *fcell, T scale, T *out, cudaStream_t s);
-template <typename T>
-cudaError_t launch_adj_lambda(long long n, const T *x, T damping, T *lam, cudaStream_t s);
 cudaError_t launch_adj_reduce(const double *partials, int nparts, int nv, int stride, double scale, double *out,
                               cudaStream_t s);
 

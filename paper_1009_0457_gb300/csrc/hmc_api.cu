@@ -119,6 +119,8 @@ struct hmc_handle {
         int rtab_version = -1;
         void *rtab = nullptr, *lam = nullptr, *ubar = nullptr, *tmp = nullptr, *vtmp = nullptr, *seg = nullptr;
         void *ck_u = nullptr, *ck_v = nullptr, *w = nullptr, *g = nullptr, *fcell = nullptr;
+        void *lsum = nullptr, *lerr = nullptr;   // sum of the reverse steps' lambdas (FP32: with its error)
+        int seg_held = -1;                       // segment whose states `seg` holds
         double *partials = nullptr, *grad = nullptr;
         hmc::Replica *reps0 = nullptr;   // descriptors whose state has Ebar = 0
         DevState *st0 = nullptr;
@@ -299,6 +301,7 @@ hmc::MpmArgs<T> mpm_args(hmc_handle *h, const void *u_in, void *u_out, void *v) 
     a.dt = (T)h->dt;
     a.dt_over_m = (T)(h->dt / 8.0);  // lumped mass rho * V * sum_p N_I(x_p) = 8 voxels
     a.keep = (T)(1.0 - h->damping);
+    a.ukeep = (T)1;
     a.grid = h->mpm_grid;
     return a;
 }
@@ -536,12 +539,14 @@ std::string validate_shared(const hmc_params *a, const hmc_params *b) {
 void free_adjoint(hmc_handle *h) {
     void *bufs[] = {h->adj.rtab, h->adj.lam, h->adj.ubar, h->adj.tmp, h->adj.vtmp, h->adj.seg, h->adj.ck_u,
                     h->adj.ck_v, h->adj.w, h->adj.g, h->adj.fcell, h->adj.partials, h->adj.grad, h->adj.reps0,
-                    h->adj.st0};
+                    h->adj.st0, h->adj.lsum, h->adj.lerr};
     for (void *b : bufs)
         if (b) cudaFree(b);
     h->adj.rtab = h->adj.lam = h->adj.ubar = h->adj.tmp = h->adj.vtmp = h->adj.seg = nullptr;
     h->adj.ck_u = h->adj.ck_v = h->adj.w = h->adj.g = h->adj.fcell = nullptr;
     h->adj.partials = h->adj.grad = nullptr;
+    h->adj.lsum = h->adj.lerr = nullptr;
+    h->adj.seg_held = -1;
     h->adj.reps0 = nullptr;
     h->adj.st0 = nullptr;
     h->adj.steps = h->adj.ck = h->adj.nseg = 0;
@@ -1957,10 +1962,12 @@ const char *hmc_last_error(const hmc_handle *h) { return h ? h->err.c_str() : g_
 namespace {
 
 template <typename T>
-cudaError_t mpm_custom(hmc_handle *h, const void *uin, void *uout, void *v, const hmc::Replica *reps, double keep) {
+cudaError_t mpm_custom(hmc_handle *h, const void *uin, void *uout, void *v, const hmc::Replica *reps, double keep,
+                       double ukeep = 1.0) {
     hmc::MpmArgs<T> a = mpm_args<T>(h, uin, uout, v);
     a.reps = reps;
     a.keep = (T)keep;
+    a.ukeep = (T)ukeep;
     return hmc::launch_mpm_step<T>(a, h->mpm_shape, h->stream);
 }
 
@@ -2001,11 +2008,13 @@ hmc_status adj_alloc(hmc_handle *h, int steps, int ck) {
         {&A.w, h->tsize * (size_t)R.N, "field w"}, {&A.g, h->tsize * (size_t)R.N, "cotangent field"},
         {&A.fcell, h->tsize * 24 * (size_t)R.nblk, "cell contributions"},
         {(void **)&A.partials, sizeof(double) * 10 * (size_t)A.nctas, "adjoint partials"},
-        {(void **)&A.grad, sizeof(double) * 10, "gradient"},
+        {(void **)&A.grad, sizeof(double) * 13, "gradient"},
+        {&A.lsum, nb, "sum of lambdas"}, {&A.lerr, h->tsize == 4 ? nb : 0, "sum of lambdas"},
         {(void **)&A.reps0, sizeof(hmc::Replica), "adjoint descriptor"},
         {(void **)&A.st0, sizeof(DevState), "adjoint state"},
     };
     for (auto &a : allocs) {
+        if (a.bytes == 0) continue;
         cudaError_t e = cudaMalloc(a.ptr, a.bytes);
         if (e != cudaSuccess) {
             free_adjoint(h);
@@ -2085,7 +2094,7 @@ hmc_status adj_backward_t(hmc_handle *h, double gW, const double *g_field, doubl
         HMC_CK(h, cudaStreamSynchronize(h->stream), "sync");
         g = static_cast<const T *>(A.g);
     }
-    HMC_CK(h, cudaMemsetAsync(A.grad, 0, sizeof(double) * 10, h->stream), "memset");
+    HMC_CK(h, cudaMemsetAsync(A.grad, 0, sizeof(double) * 13, h->stream), "memset");
     // terminal: direct parameter terms and ubar^T = sum_p alpha_p B_p^T sigma_p, lambda^T = dt ubar^T
     HMC_CK(h, adj_terminal<T>(h, g, gW, nullptr), "terminal launch");
     HMC_CK(h, hmc::launch_adj_reduce(A.partials, A.nctas, 10, 10, 1.0, A.grad, h->stream), "reduce launch");
@@ -2097,33 +2106,47 @@ hmc_status adj_backward_t(hmc_handle *h, double gW, const double *g_field, doubl
            "gather launch");
     const size_t nb = node_bytes(h);
     // every reverse step adds its parameter terms to its CTA's partials; one reduction at the end
-    HMC_CK(h, cudaMemsetAsync(A.partials, 0, sizeof(double) * 9 * (size_t)A.nctas, h->stream), "memset");
+    HMC_CK(h, cudaMemsetAsync(A.partials, 0, sizeof(double) * 3 * (size_t)A.nctas, h->stream), "memset");
+    HMC_CK(h, cudaMemsetAsync(A.lsum, 0, nb, h->stream), "memset");
+    if (A.lerr) HMC_CK(h, cudaMemsetAsync(A.lerr, 0, nb, h->stream), "memset");
+    void *lam = A.lam, *lam_next = A.tmp;
     for (int s = A.nseg - 1; s >= 0; --s) {
         const int n0 = s * A.ck, len = std::min(A.ck, A.steps - n0);
-        // recompute the segment's forward states u^{n0} .. u^{n0+len-1} from its checkpoint
-        HMC_CK(h, cudaMemcpyAsync(seg_ptr(h, A.seg, 0), seg_ptr(h, A.ck_u, s), nb, cudaMemcpyDeviceToDevice, h->stream),
-               "checkpoint copy");
-        HMC_CK(h, cudaMemcpyAsync(A.vtmp, seg_ptr(h, A.ck_v, s), nb, cudaMemcpyDeviceToDevice, h->stream),
-               "checkpoint copy");
-        for (int j = 1; j < len; ++j)
-            HMC_CK(h, mpm_custom<T>(h, seg_ptr(h, A.seg, j - 1), seg_ptr(h, A.seg, j), A.vtmp, h->d_reps,
-                                    1.0 - h->damping),
-                   "recompute launch");
+        // the segment's forward states u^{n0} .. u^{n0+len-1}: recomputed from its checkpoint, unless the
+        // buffer still holds them (the last segment's, from the forward pass)
+        if (A.seg_held != s) {
+            HMC_CK(h, cudaMemcpyAsync(seg_ptr(h, A.seg, 0), seg_ptr(h, A.ck_u, s), nb, cudaMemcpyDeviceToDevice, h->stream),
+                   "checkpoint copy");
+            HMC_CK(h, cudaMemcpyAsync(A.vtmp, seg_ptr(h, A.ck_v, s), nb, cudaMemcpyDeviceToDevice, h->stream),
+                   "checkpoint copy");
+            A.seg_held = -1;
+            for (int j = 1; j < len; ++j)
+                HMC_CK(h, mpm_custom<T>(h, seg_ptr(h, A.seg, j - 1), seg_ptr(h, A.seg, j), A.vtmp, h->d_reps,
+                                        1.0 - h->damping),
+                       "recompute launch");
+            A.seg_held = s;
+        }
         for (int j = len - 1; j >= 0; --j) {
-            HMC_CK(h, hmc::launch_adj_params<T>(aa, static_cast<const T *>(A.lam),
-                                                reinterpret_cast<const T *>(seg_ptr(h, A.seg, j)), h->stream),
+            HMC_CK(h, hmc::launch_adj_params<T>(aa, static_cast<const T *>(lam),
+                                                reinterpret_cast<const T *>(seg_ptr(h, A.seg, j)),
+                                                static_cast<T *>(A.lsum), static_cast<T *>(A.lerr), h->stream),
                    "parameter launch");
-            // ubar^n = ubar^{n+1} + c F(lambda^{n+1}; 0); tmp = lambda^{n+1} + dt ubar^n
-            HMC_CK(h, mpm_custom<T>(h, A.lam, A.tmp, A.ubar, A.reps0, 1.0), "adjoint step launch");
-            HMC_CK(h, hmc::launch_adj_lambda<T>(3ll * R.nblk, static_cast<const T *>(A.tmp), (T)h->damping,
-                                                static_cast<T *>(A.lam), h->stream),
-                   "lambda launch");
+            // ubar^n = ubar^{n+1} + c F(lambda^{n+1}; 0); lambda^n = (1 - damping) lambda^{n+1} + dt ubar^n
+            HMC_CK(h, mpm_custom<T>(h, lam, lam_next, A.ubar, A.reps0, 1.0, 1.0 - h->damping), "adjoint step launch");
+            std::swap(lam, lam_next);
         }
     }
+    // the sums of P, T and D of every step, then the terms linear in lambda
+    HMC_CK(h, hmc::launch_adj_reduce(A.partials, A.nctas, 3, 3, -c / 1024.0, A.grad + 10, h->stream), "reduce launch");
+    HMC_CK(h, hmc::launch_adj_mean<T>(aa, static_cast<const T *>(A.lsum), static_cast<const T *>(A.lerr), h->stream),
+           "parameter launch");
     HMC_CK(h, hmc::launch_adj_reduce(A.partials, A.nctas, 9, 9, -c, A.grad + 1, h->stream), "reduce launch");
-    double out[10];
+    double out[13];
     HMC_CK(h, cudaMemcpyAsync(out, A.grad, sizeof(out), cudaMemcpyDeviceToHost, h->stream), "download");
     HMC_CK(h, cudaStreamSynchronize(h->stream), "sync");
+    out[1] += out[10];                     // x.R_1.y = P
+    out[2] += out[11] - out[10];           // x.R_2.y = T - P
+    out[3] += 2.0 * (out[12] - out[10]);   // x.R_3.y = 2 (D - P)
     for (int k = 0; k < 9; ++k) {
         if (!std::isfinite(out[1 + k])) return fail(h, HMC_ERR_NONFINITE, "non-finite gradient");
         grad[k] = out[1 + k];
@@ -2144,6 +2167,8 @@ hmc_status hmc_adjoint_forward(hmc_handle *h, int32_t nsteps, int32_t checkpoint
     if ((s = adj_alloc(h, nsteps, checkpoint_every)) != HMC_OK) return s;
     if ((s = adj_tables(h)) != HMC_OK) return s;
     auto &A = h->adj;
+    A.seg_held = -1;
+    A.have_forward = false;
     HMC_CK(h, cudaMemcpyAsync(A.ebar, h->st[0].ebar, sizeof(A.ebar), cudaMemcpyDeviceToHost, h->stream), "download");
     HMC_CK(h, cudaStreamSynchronize(h->stream), "sync");
     const size_t nb = node_bytes(h);
@@ -2152,7 +2177,22 @@ hmc_status hmc_adjoint_forward(hmc_handle *h, int32_t nsteps, int32_t checkpoint
                "checkpoint");
         HMC_CK(h, cudaMemcpyAsync(seg_ptr(h, A.ck_v, sg), h->v, nb, cudaMemcpyDeviceToDevice, h->stream), "checkpoint");
         const int len = std::min(A.ck, A.steps - sg * A.ck);
-        for (int j = 0; j < len; ++j) HMC_CK(h, enq_mpm(h, h->stream), "MPM launch");
+        if (sg + 1 < A.nseg) {
+            for (int j = 0; j < len; ++j) HMC_CK(h, enq_mpm(h, h->stream), "MPM launch");
+            continue;
+        }
+        // the last segment runs through the segment buffer, where the reverse sweep needs its states first
+        HMC_CK(h, cudaMemcpyAsync(seg_ptr(h, A.seg, 0), h->u[h->cur], nb, cudaMemcpyDeviceToDevice, h->stream),
+               "checkpoint");
+        h->cur ^= 1;
+        for (int j = 0; j < len; ++j) {
+            void *to = j + 1 < len ? static_cast<void *>(seg_ptr(h, A.seg, j + 1)) : h->u[h->cur];
+            const double keep = 1.0 - h->damping;
+            HMC_CK(h, h->p.precision == HMC_FP32 ? mpm_custom<float>(h, seg_ptr(h, A.seg, j), to, h->v, h->d_reps, keep)
+                                                 : mpm_custom<double>(h, seg_ptr(h, A.seg, j), to, h->v, h->d_reps, keep),
+                   "MPM launch");
+        }
+        A.seg_held = sg;
     }
     HMC_CK(h, cudaMemsetAsync(A.grad, 0, sizeof(double) * 10, h->stream), "memset");
     if (h->p.precision == HMC_FP32)

@@ -114,6 +114,7 @@ struct MpmArgs {
     int cexp;                // ... entry = round(C' 2^cexp), x the signed low half, y the high half
     int nq;                  // orientations (the FP32 step stages cubw in shared memory up to MPM_STAB_MAX)
     T dt, dt_over_m, keep;   // keep = 1 - damping
+    T ukeep;                 // u_out = ukeep u + dt v: 1, or 1 - damping in the adjoint's reverse step
     int grid;                // CTAs
 };
 

@@ -8,15 +8,14 @@
 //   ubar^T = sum_p alpha_p B_p^T C'_p eps_p,   lambda^T = dt ubar^T
 //   theta_bar += -c [ epsbar_p . R_i . eps_p^n , (C'_p epsbar_p)_k ] summed over p,  epsbar_p = B_p lambda^{n+1}
 //   ubar^n = ubar^{n+1} + c F(lambda^{n+1}; Ebar = 0)      (the forward MPM kernel with kappa = 1)
-//   lambda^n = kappa lambda^{n+1} + dt ubar^n
+//   lambda^n = kappa lambda^{n+1} + dt ubar^n              (its displacement update, scaled by kappa)
 // plus the terminal terms sum_p alpha_p [1/2 eps.R_i.eps, (C' eps)_k].  R_i are
 // the rotated basis tensors with C' = C11 R_1 + C12 R_2 + C44 R_3.
 //
 // These kernels: the per-step parameter terms (added to per-CTA partials that
 // are reduced once per reverse sweep), the terminal pass (field w, W,
 // alpha-weighted nodal vector through a per-cell buffer and a node gather,
-// terminal parameter terms), the lambda update, and the fixed-order FP64
-// reduction of per-CTA partials.  Single replica; one thread per cell.
+// terminal parameter terms), and the fixed-order FP64 reduction of per-CTA partials.  Single replica; one thread per cell.
 #include "hmc_device.cuh"
 #include "hmc_adjoint.h"
 
@@ -157,54 +156,198 @@ __device__ __forceinline__ void load_row(const T *__restrict__ p, int n, T *out)
     for (int k = 0; k < n; ++k) out[k] = __ldg(p + k);
 }
 
-// One reverse step's parameter terms: per point epsbar.R_i.eps (i = 1..3) and
-// C' epsbar (6); a cell's eight points are summed plainly, cells by the
-// accumulator, and the CTA's sums are added to its partials.  The axis weights and
-// the stiffness row are loaded when the orientation changes from one point to the next.
+// 2x2 -> 2x2 sums with weights 3 (same side) and 1 (other side), 16 times the interpolation
+template <typename T>
+__device__ __forceinline__ void interp31(T d00, T d10, T d01, T d11, T (&o)[2][2]) {
+    const T e00 = fma(T(3), d00, d10), e10 = fma(T(3), d10, d00);
+    const T e01 = fma(T(3), d01, d11), e11 = fma(T(3), d11, d01);
+    o[0][0] = fma(T(3), e00, e01);
+    o[0][1] = fma(T(3), e01, e00);
+    o[1][0] = fma(T(3), e10, e11);
+    o[1][1] = fma(T(3), e11, e10);
+}
+
+// 32 times the displacement gradients of the cell's points
+template <typename T>
+__device__ __forceinline__ void cell_gradients32(const T (&u)[8][3], CellGrad<T> &g) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        T o[2][2];
+        interp31<T>(u[1][d] - u[0][d], u[3][d] - u[2][d], u[5][d] - u[4][d], u[7][d] - u[6][d], o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) g.gx[i >> 1][i & 1][d] = o[i >> 1][i & 1];
+        interp31<T>(u[2][d] - u[0][d], u[3][d] - u[1][d], u[6][d] - u[4][d], u[7][d] - u[5][d], o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) g.gy[i >> 1][i & 1][d] = o[i >> 1][i & 1];
+        interp31<T>(u[4][d] - u[0][d], u[5][d] - u[1][d], u[6][d] - u[2][d], u[7][d] - u[3][d], o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) g.gz[i >> 1][i & 1][d] = o[i >> 1][i & 1];
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ void fluctuation(const CellGrad<T> &g, int a, int b, int c, T (&e)[6]) {
+    e[0] = g.gx[b][c][0];
+    e[1] = g.gy[a][c][1];
+    e[2] = g.gz[a][b][2];
+    e[3] = g.gz[a][b][1] + g.gy[a][c][2];
+    e[4] = g.gz[a][b][0] + g.gx[b][c][2];
+    e[5] = g.gy[a][c][0] + g.gx[b][c][1];
+}
+
+// Weights with a_m.x.a_m = W_m . x (engineering shear) of the first two crystal axes.
+template <typename T>
+__device__ __forceinline__ void load_axes(const T *p, T (&w)[12]) {
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float4 t = __ldg(reinterpret_cast<const float4 *>(p) + i);
+            w[4 * i] = t.x; w[4 * i + 1] = t.y; w[4 * i + 2] = t.z; w[4 * i + 3] = t.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            const double2 t = __ldg(reinterpret_cast<const double2 *>(p) + i);
+            w[2 * i] = t.x; w[2 * i + 1] = t.y;
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int k = 3; k < 6; ++k) w[6 * m + k] *= T(0.5);
+}
+
+// One reverse step's parameter terms.  With eps = Ebar + B u, everything that is linear in
+// lambda alone -- the forms against Ebar and the mean of C' epsbar -- is left to one pass over
+// the sum of the lambdas (k_adj_mean); what is left per step are the three forms of B lambda
+// and B u, and these are combinations of P = sum_m p_m p_m, T = tr tr and D = x:y (basis_forms),
+// so the sums of P, T and D are kept (times 2^10, from gradients times 32).  The third axis'
+// projection is the trace minus the other two.  Each thread also adds its node's lambda to the sum
+// (TwoSum pairs in FP32).  About 640 operations a cell where the full terms took 1530, and 12
+// table values per orientation change instead of 42: 40 -> 20 us per step at 128^3.
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_adj_params(AdjArgs<T> a, const T *__restrict__ lam,
-                                                    const T *__restrict__ u) {
+                                                    const T *__restrict__ u, T *__restrict__ lsum,
+                                                    T *__restrict__ lerr) {
+    AdjAcc<T, 3> acc;
+    acc.zero();
+    const int blk = blockIdx.x * blockDim.x + threadIdx.x;
+    if (blk < a.nblk) {
+        const int bx = blk % a.nbx, r = blk / a.nbx;
+        const int by = r % a.nby, bz = r / a.nby;
+        const uint4 sp = __ldg(a.spins + blk);
+        CellGrad<T> gl, gu;
+        {
+            T cl[8][3];
+            load_corners<T>(lam, bx, by, bz, a.nbx, a.nby, a.nbz, cl);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {   // corner 0 is node blk
+                const long long i = 3ll * blk + d;
+                if constexpr (sizeof(T) == 4) {
+                    TwoSumF s{lsum[i], lerr[i]};
+                    s.add(cl[0][d]);
+                    lsum[i] = s.hi;
+                    lerr[i] = s.lo;
+                } else {
+                    lsum[i] += cl[0][d];
+                }
+            }
+            cell_gradients32<T>(cl, gl);
+        }
+        {
+            T cu[8][3];
+            load_corners<T>(u, bx, by, bz, a.nbx, a.nby, a.nbz, cu);
+            cell_gradients32<T>(cu, gu);
+        }
+        T P = T(0), TT = T(0), D = T(0), Dh = T(0);   // D's shear terms count half
+        T w[12];
+        uint32_t qprev = 0xffffffffu;
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            const int L = n == 2 ? 3 : n == 3 ? 2 : n == 4 ? 6 : n == 5 ? 7 : n == 6 ? 5 : n == 7 ? 4 : n;   // Gray code
+            T x[6], y[6];
+            fluctuation<T>(gl, L & 1, (L >> 1) & 1, L >> 2, x);
+            fluctuation<T>(gu, L & 1, (L >> 1) & 1, L >> 2, y);
+            const uint32_t q = spin_of(sp, local_slot(L));
+            if (q != qprev) {
+                load_axes<T>(a.wtab + 20ll * q, w);
+                qprev = q;
+            }
+            T px[2], py[2];
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                px[m] = w[6 * m] * x[0];
+                py[m] = w[6 * m] * y[0];
+#pragma unroll
+                for (int k = 1; k < 6; ++k) {
+                    px[m] = fma(w[6 * m + k], x[k], px[m]);
+                    py[m] = fma(w[6 * m + k], y[k], py[m]);
+                }
+            }
+            const T tx = x[0] + x[1] + x[2], ty = y[0] + y[1] + y[2];
+            P = fma(px[0], py[0], P);
+            P = fma(px[1], py[1], P);
+            P = fma(tx - px[0] - px[1], ty - py[0] - py[1], P);
+            TT = fma(tx, ty, TT);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                D = fma(x[k], y[k], D);
+                Dh = fma(x[3 + k], y[3 + k], Dh);
+            }
+        }
+        acc.add(0, P);
+        acc.add(1, TT);
+        acc.add(2, fma(T(0.5), Dh, D));
+    }
+    cta_partials<T, 3>(acc, a.partials, true);
+}
+
+// The parameter terms that are linear in lambda, from the sum L of the reverse steps' lambdas:
+// per point (B L).R_i.Ebar (i = 1..3) and C' B L (6), added to the CTA's partials; a cell's eight
+// points are summed plainly, cells by the accumulator.
+template <typename T>
+__global__ void __launch_bounds__(256) k_adj_mean(AdjArgs<T> a, const T *__restrict__ lsum,
+                                                  const T *__restrict__ lerr) {
     AdjAcc<T, 9> acc;
     acc.zero();
     const int blk = blockIdx.x * blockDim.x + threadIdx.x;
     if (blk < a.nblk) {
         const int bx = blk % a.nbx, r = blk / a.nbx;
         const int by = r % a.nby, bz = r / a.nby;
-        T cl[8][3], cu[8][3];
-        load_corners<T>(lam, bx, by, bz, a.nbx, a.nby, a.nbz, cl);
-        load_corners<T>(u, bx, by, bz, a.nbx, a.nby, a.nbz, cu);
-        CellGrad<T> gl, gu;
+        T cl[8][3];
+        load_corners<T>(lsum, bx, by, bz, a.nbx, a.nby, a.nbz, cl);
+        if constexpr (sizeof(T) == 4) {
+            T ce[8][3];
+            load_corners<T>(lerr, bx, by, bz, a.nbx, a.nby, a.nbz, ce);
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) cl[c][d] += ce[c][d];
+        }
+        CellGrad<T> gl;
         cell_gradients<T>(cl, gl);
-        cell_gradients<T>(cu, gu);
         const uint4 sp = __ldg(a.spins + blk);
         const T zero[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
         T csum[9] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-        T w[18];
-        Row24<T> crow;
-        uint32_t qprev = 0xffffffffu;
 #pragma unroll
         for (int L = 0; L < 8; ++L) {
-            const int x = L & 1, y = (L >> 1) & 1, z = L >> 2;
-            T eb[6], e[6], s[6], rf[3];
-            point_strain<T>(gl, zero, x, y, z, eb);
-            point_strain<T>(gu, a.ebar, x, y, z, e);
+            T x[6], s[6], rf[3], w[18];
+            point_strain<T>(gl, zero, L & 1, (L >> 1) & 1, L >> 2, x);
             const uint32_t q = spin_of(sp, local_slot(L));
-            if (q != qprev) {
-                load_row<T>(a.wtab + 20ll * q, 18, w);
-                crow.load(a.ctab + 24ll * q);
-                qprev = q;
-            }
-            basis_forms<T>(w, eb, e, rf);
+            load_row<T>(a.wtab + 20ll * q, 18, w);
+            basis_forms<T>(w, x, a.ebar, rf);
+            Row24<T> crow;
+            crow.load(a.ctab + 24ll * q);
+            hooke21<T>(crow.v, x, s);
 #pragma unroll
             for (int i = 0; i < 3; ++i) csum[i] += rf[i];
-            hooke21<T>(crow.v, eb, s);
 #pragma unroll
             for (int k = 0; k < 6; ++k) csum[3 + k] += s[k];
         }
 #pragma unroll
         for (int i = 0; i < 9; ++i) acc.add(i, csum[i]);
     }
-    cta_partials<T, 9>(acc, a.partials, true);
+    cta_partials<T, 9>(acc, a.partials, false);
 }
 
 // Terminal pass at u^T: field w (natural order), per-CTA partials of
@@ -308,13 +451,6 @@ __global__ void k_adj_gather(AdjArgs<T> a, const T *__restrict__ fcell, T scale,
     for (int d = 0; d < 3; ++d) out[3ll * n + d] = scale * s[d];
 }
 
-// lambda <- x - damping * lambda (elementwise over 3 * nnodes values).
-template <typename T>
-__global__ void k_adj_lambda(long long n, const T *__restrict__ x, T damping, T *__restrict__ lam) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) lam[i] = x[i] - damping * lam[i];
-}
-
 // out[i] += scale * sum over CTAs of partials[., i] (fixed order), one CTA.
 __global__ void k_adj_reduce(const double *partials, int nparts, int nv, int stride, double scale, double *out) {
     __shared__ double red[256];
@@ -335,8 +471,13 @@ __global__ void k_adj_reduce(const double *partials, int nparts, int nv, int str
 }  // namespace
 
 template <typename T>
-cudaError_t launch_adj_params(const AdjArgs<T> &a, const T *lam, const T *u, cudaStream_t s) {
-    k_adj_params<T><<<(a.nblk + 255) / 256, 256, 0, s>>>(a, lam, u);
+cudaError_t launch_adj_params(const AdjArgs<T> &a, const T *lam, const T *u, T *lsum, T *lerr, cudaStream_t s) {
+    k_adj_params<T><<<(a.nblk + 255) / 256, 256, 0, s>>>(a, lam, u, lsum, lerr);
+    return cudaGetLastError();
+}
+template <typename T>
+cudaError_t launch_adj_mean(const AdjArgs<T> &a, const T *lsum, const T *lerr, cudaStream_t s) {
+    k_adj_mean<T><<<(a.nblk + 255) / 256, 256, 0, s>>>(a, lsum, lerr);
     return cudaGetLastError();
 }
 template <typename T>
@@ -349,11 +490,6 @@ cudaError_t launch_adj_gather(const AdjArgs<T> &a, const T *fcell, T scale, T *o
     k_adj_gather<T><<<(a.nblk + 255) / 256, 256, 0, s>>>(a, fcell, scale, out);
     return cudaGetLastError();
 }
-template <typename T>
-cudaError_t launch_adj_lambda(long long n, const T *x, T damping, T *lam, cudaStream_t s) {
-    k_adj_lambda<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, x, damping, lam);
-    return cudaGetLastError();
-}
 cudaError_t launch_adj_reduce(const double *partials, int nparts, int nv, int stride, double scale, double *out,
                               cudaStream_t s) {
     k_adj_reduce<<<1, 256, 0, s>>>(partials, nparts, nv, stride, scale, out);
@@ -361,11 +497,11 @@ cudaError_t launch_adj_reduce(const double *partials, int nparts, int nv, int st
 }
 
 #define HMC_ADJ_INST(T)                                                                                          \
-    template cudaError_t launch_adj_params<T>(const AdjArgs<T> &, const T *, const T *, cudaStream_t);         \
-    template cudaError_t launch_adj_terminal<T>(const AdjArgs<T> &, const T *, const T *, T, T *, T *,         \
-                                                cudaStream_t);                                                \
-    template cudaError_t launch_adj_gather<T>(const AdjArgs<T> &, const T *, T, T *, cudaStream_t);            \
-    template cudaError_t launch_adj_lambda<T>(long long, const T *, T, T *, cudaStream_t);
+    template cudaError_t launch_adj_params<T>(const AdjArgs<T> &, const T *, const T *, T *, T *, cudaStream_t); \
+    template cudaError_t launch_adj_mean<T>(const AdjArgs<T> &, const T *, const T *, cudaStream_t);             \
+    template cudaError_t launch_adj_terminal<T>(const AdjArgs<T> &, const T *, const T *, T, T *, T *,           \
+                                                cudaStream_t);                                                   \
+    template cudaError_t launch_adj_gather<T>(const AdjArgs<T> &, const T *, T, T *, cudaStream_t);
 HMC_ADJ_INST(float)
 HMC_ADJ_INST(double)
 

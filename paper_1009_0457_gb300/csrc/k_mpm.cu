@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(MPM_THREADS, 2) k_mpm_step(MpmArgs<float> a) {
                     for (int d = 0; d < 3; ++d) {
                         const float vn = rfma(fscale, F[d], rmul(a.keep, vold[d]));
                         vp[d] = vn;
-                        up[d] = rfma(a.dt, vn, uc[d] * 32.f);
+                        up[d] = rfma(a.dt, vn, rmul(a.ukeep, uc[d] * 32.f));
                     }
                     vp += pstride;
                     up += pstride;
@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_mpm_block(MpmArgs<fl
         for (int d = 0; d < 3; ++d) {
             const float vn = rfma(fscale, F[d], rmul(a.keep, vold[d]));
             a.v[3 * at + d] = vn;
-            a.u_out[3 * at + d] = rfma(a.dt, vn, (un[d] * 0.03125f) * 32.f);
+            a.u_out[3 * at + d] = rfma(a.dt, vn, rmul(a.ukeep, (un[d] * 0.03125f) * 32.f));
         }
     }
 }

@@ -322,21 +322,22 @@ __device__ __forceinline__ Fx3 fx_sum4(const FxHalf (&xy)[8][THREADS], const FxH
 // the update of a node whose force is not finite or whose scale leaves the normal range; kept out of
 // line, since its FP64 multiplications would otherwise be formed for every node (6 % of a step)
 __device__ __noinline__ void fx_update_any(ll x, ll y, ll z, int e, double fscale, int shift, double keep, double dt,
-                                           const double *uold, const double *vold, double *u, double *v) {
+                                           double ukeep, const double *uold, const double *vold, double *u, double *v) {
     for (int d = 0; d < 3; ++d) {
         const double F = e >= 2047 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn((double)(d == 0 ? x : d == 1 ? y : z), shift);
         const double vn = rfma(fscale, F, rmul(keep, vold[d]));
         v[d] = vn;
-        u[d] = rfma(dt, vn, uold[d]);
+        u[d] = rfma(dt, vn, rmul(ukeep, uold[d]));
     }
 }
 
 // velocity and displacement of a node from the force sums of the cells below and above it
 struct FxUpdate {
-    double fscale, dt, keep;   // fscale = -dt / (32 m)
+    double fscale, dt, keep, ukeep;   // fscale = -dt / (32 m)
     int cexp, fexp;
+    bool scaled;   // ukeep is not 1
     __device__ __forceinline__ explicit FxUpdate(const MpmArgs<double> &a)
-        : fscale(-a.dt_over_m * 0.03125), dt(a.dt), keep(a.keep), cexp(a.cexp) {
+        : fscale(-a.dt_over_m * 0.03125), dt(a.dt), keep(a.keep), ukeep(a.ukeep), cexp(a.cexp), scaled(a.ukeep != 1.0) {
         // the force integers of exponent E are 2^(E - cexp - 1013) of the FP32 step's units
         fexp = dexp(fscale) ? dexp(fscale) - cexp - 1013 : -10000;   // (subnormal: the general form)
     }
@@ -352,10 +353,10 @@ struct FxUpdate {
             for (int d = 0; d < 3; ++d) {
                 const double vn = rfma(fs, (double)F.v[d], rmul(keep, vold[d]));
                 v[d] = vn;
-                u[d] = rfma(dt, vn, uold[d]);
+                u[d] = rfma(dt, vn, scaled ? rmul(ukeep, uold[d]) : uold[d]);
             }
         } else {
-            fx_update_any(F.v[0], F.v[1], F.v[2], F.e, fscale, F.e - cexp - 1013, keep, dt, uold, vold, u, v);
+            fx_update_any(F.v[0], F.v[1], F.v[2], F.e, fscale, F.e - cexp - 1013, keep, dt, ukeep, uold, vold, u, v);
         }
     }
 };
