@@ -62,7 +62,7 @@ struct hmc_handle {
     std::vector<RepHost> reps;
     int R = 1, sel = 0;
     long long nblk_total = 0, N_total = 0, N_max = 0;
-    int nctas = 0;
+    int nctas = 0, max_ncta = 0;   // block-parallel CTAs of the batch, of its largest replica
     cudaStream_t stream = nullptr, cap = nullptr;
     bool own_stream = false, oriented = false;
     bool lost = false;    // a sweep returned with its stress copy outstanding: every later call is refused
@@ -417,7 +417,7 @@ cudaError_t enqueue_mcs(hmc_handle *h, cudaStream_t s) {
     if ((e = enq_stress(h, sweeps_read_stress(h), s)) != cudaSuccess) return e;
     if ((e = enq_sweep(h, 0, s)) != cudaSuccess) return e;
     if ((e = enq_sweep(h, 1, s)) != cudaSuccess) return e;
-    return hmc::launch_end_mcs(h->d_reps, h->R, h->partials, h->nctas, 1, 1, s);
+    return hmc::launch_end_mcs(h->d_reps, h->R, h->max_ncta, h->partials, h->nctas, 1, 1, s);
 }
 
 cudaError_t reset_accepted(hmc_handle *h) {
@@ -782,16 +782,23 @@ hmc_status tune_mpm(hmc_handle *h, bool enabled, int &best_limit) {
                            ? hmc::launch_mpm_step<float>(mpm_args<float>(h, h->u[h->cur], uo, vs), v, h->stream)
                            : hmc::launch_mpm_step<double>(mpm_args<double>(h, h->u[h->cur], uo, vs), v, h->stream);
             };
+            // the best of three runs, after one of four launches that says how many make about 0.3 ms (at
+            // 32^3 the candidates differ by 1 of 11 us, which four launches do not resolve)
             err = launch();
             float ms = 1e30f;
-            for (int rep = 0; rep < 2 && err == cudaSuccess; ++rep) {   // the better of two runs of four
+            int n = 4;
+            for (int rep = 0; rep < 4 && err == cudaSuccess; ++rep) {
                 float t = 0;
                 err = cudaEventRecord(e0, h->stream);
-                for (int k = 0; k < 4 && err == cudaSuccess; ++k) err = launch();
+                for (int k = 0; k < n && err == cudaSuccess; ++k) err = launch();
                 if (err == cudaSuccess) err = cudaEventRecord(e1, h->stream);
                 if (err == cudaSuccess) err = cudaEventSynchronize(e1);
                 if (err == cudaSuccess) err = cudaEventElapsedTime(&t, e0, e1);
-                ms = std::min(ms, t);
+                if (rep > 0) ms = std::min(ms, t / n);
+                if (rep == 0) {
+                    if (t / n > 2.f * best) break;   // not in question
+                    n = t > 0.f ? std::max(2, std::min(40, (int)(0.3f * n / t))) : n;
+                }
             }
             if (err == cudaSuccess && ms < best) {
                 best = ms;
@@ -1065,6 +1072,7 @@ hmc_status hmc_create_batch(const hmc_params *params, int32_t n_replicas, hmc_ha
         R.ncta = (int)((R.nblk + hmc::BLOCK_THREADS - 1) / hmc::BLOCK_THREADS);
         R.cta_off = cta;
         cta += R.ncta;
+        h->max_ncta = std::max(h->max_ncta, R.ncta);
         const int K = std::max(R.p.nx, std::max(R.p.ny, R.p.nz));
         R.lam = R.p.elastic_scale >= 0 ? R.p.elastic_scale : 1e9 * (1.0 / K) * kL0 * kGammaStar / (2.0 * kGammaS);
         R.lam_sd_half = 0.5 * R.lam * (h->S11 - h->S12 - 0.5 * h->S44);
@@ -1476,7 +1484,7 @@ hmc_status hmc_compute_stress(hmc_handle *h, double *mean, double *energy) {
         ++h->state_version;
     }
     HMC_CK(h, enq_stress(h, true, h->stream), "stress launch");
-    HMC_CK(h, hmc::launch_end_mcs(h->d_reps, h->R, h->partials, h->nctas, 0, 0, h->stream), "reduction launch");
+    HMC_CK(h, hmc::launch_end_mcs(h->d_reps, h->R, h->max_ncta, h->partials, h->nctas, 0, 0, h->stream), "reduction launch");
     if (mean || energy) return read_stats(h, mean, energy);
     return HMC_OK;
 }
@@ -1594,7 +1602,7 @@ hmc_status hmc_end_mcs(hmc_handle *h) {
     if (h) ++h->state_version;
     hmc_status s = need_oriented(h);
     if (s != HMC_OK) return s;
-    HMC_CK(h, hmc::launch_end_mcs(h->d_reps, h->R, h->partials, h->nctas, 1, 1, h->stream), "end-of-step launch");
+    HMC_CK(h, hmc::launch_end_mcs(h->d_reps, h->R, h->max_ncta, h->partials, h->nctas, 1, 1, h->stream), "end-of-step launch");
     return HMC_OK;
 }
 

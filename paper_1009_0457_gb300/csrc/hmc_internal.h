@@ -218,6 +218,25 @@ constexpr int MPM_SMALL_BLOCK = 96;  // ... of the small-block form
 constexpr int MPM_NODES = 304;       // most nodes of a patch's plane, (W+1)(H+1)
 inline bool mpm_is_block(int variant) { return variant >= MPM_BLOCK; }
 
+// A launch with programmatic stream serialisation: the kernel may be scheduled before the one ahead
+// of it in the stream has finished, and executes griddepcontrol.wait before it reads or writes
+// anything that another kernel touches.
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                       const A &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Launchers (return cudaGetLastError of the launch).
 template <typename T>
 cudaError_t launch_mpm_step(const MpmArgs<T> &a, int shape, cudaStream_t s);
@@ -243,16 +262,17 @@ cudaError_t sweep_prepare();  // opt the elastic sweeps into their shared memory
 template <typename T>
 int mpm_per_sm(int variant, int nq);  // resident MPM CTAs per SM
 
-// One CTA per replica: fixed-order FP64 sum of its stress partials, loading
-// update (update_strain) and MCS counter (advance).
-// End-of-step reduction: END_GROUPS CTAs per replica sum the stress partials in a fixed
-// order in FP64; the last to finish sums their group sums in group order and finishes the
-// step.  Its scratch lies behind the nctas x 7 stress partials: END_GROUPS x 7 group sums
-// per replica, then one arrival counter per replica (zero between launches).
+// End-of-step reduction, loading update (update_strain) and MCS counter (advance).  A replica's stress
+// partials are summed in a fixed order in FP64 by end_groups(its CTAs) CTAs, and the last of them to
+// finish sums the group sums in group order and finishes the step.  Its scratch lies behind the
+// nctas x 7 stress partials: END_GROUPS x 7 group sums per replica, then one arrival counter per
+// replica (zero between launches).
 constexpr int END_GROUPS = 32;
+// (one CTA up to 512 partials: the second stage's fence, atomic and reload cost 3 us)
+__host__ __device__ constexpr int end_groups(int ncta) { return ncta <= 512 ? 1 : ncta >= 256 * END_GROUPS ? END_GROUPS : (ncta + 255) / 256; }
 inline size_t end_scratch_doubles(int nrep) { return (size_t)nrep * END_GROUPS * 7 + (size_t)(nrep + 1) / 2; }
-cudaError_t launch_end_mcs(const Replica *reps, int nrep, double *partials, int nctas, int update_strain, int advance,
-                           cudaStream_t s);
+cudaError_t launch_end_mcs(const Replica *reps, int nrep, int max_ncta, double *partials, int nctas, int update_strain,
+                           int advance, cudaStream_t s);   // max_ncta: of the largest replica
 cudaError_t launch_check_spins(const uint16_t *nat, long long n, int nq, DevState *st, cudaStream_t s);
 cudaError_t launch_pack_spins(const uint16_t *nat, uint4 *blk, int nx, int ny, int nz, cudaStream_t s);
 cudaError_t launch_unpack_spins(const uint4 *blk, uint16_t *nat, int nx, int ny, int nz, cudaStream_t s);

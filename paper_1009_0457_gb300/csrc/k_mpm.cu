@@ -524,17 +524,7 @@ int mpm_per_sm<float>(int variant, int nq) {
 template <>
 cudaError_t launch_mpm_step<float>(const MpmArgs<float> &a, int variant, cudaStream_t s) {
     const Form f = form_of(variant, a.nq);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.grid);
-    cfg.blockDim = dim3(f.threads);
-    cfg.dynamicSmemBytes = f.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, f.kernel, a);
+    return launch_pdl(f.kernel, (unsigned)a.grid, (unsigned)f.threads, f.smem, s, a);
 }
 
 }  // namespace hmc

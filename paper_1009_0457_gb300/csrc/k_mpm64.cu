@@ -332,12 +332,14 @@ __device__ __noinline__ void fx_update_any(ll x, ll y, ll z, int e, double fscal
 }
 
 // velocity and displacement of a node from the force sums of the cells below and above it
+// (SCALED: the old displacement times ukeep, in the adjoint's reverse step; a form of its own, since an
+// FP64 multiplication of every node costs 2 % of a step even where it is not used)
+template <bool SCALED>
 struct FxUpdate {
     double fscale, dt, keep, ukeep;   // fscale = -dt / (32 m)
     int cexp, fexp;
-    bool scaled;   // ukeep is not 1
     __device__ __forceinline__ explicit FxUpdate(const MpmArgs<double> &a)
-        : fscale(-a.dt_over_m * 0.03125), dt(a.dt), keep(a.keep), ukeep(a.ukeep), cexp(a.cexp), scaled(a.ukeep != 1.0) {
+        : fscale(-a.dt_over_m * 0.03125), dt(a.dt), keep(a.keep), ukeep(a.ukeep), cexp(a.cexp) {
         // the force integers of exponent E are 2^(E - cexp - 1013) of the FP32 step's units
         fexp = dexp(fscale) ? dexp(fscale) - cexp - 1013 : -10000;   // (subnormal: the general form)
     }
@@ -353,7 +355,7 @@ struct FxUpdate {
             for (int d = 0; d < 3; ++d) {
                 const double vn = rfma(fs, (double)F.v[d], rmul(keep, vold[d]));
                 v[d] = vn;
-                u[d] = rfma(dt, vn, scaled ? rmul(ukeep, uold[d]) : uold[d]);
+                u[d] = rfma(dt, vn, SCALED ? rmul(ukeep, uold[d]) : uold[d]);
             }
         } else {
             fx_update_any(F.v[0], F.v[1], F.v[2], F.e, fscale, F.e - cexp - 1013, keep, dt, ukeep, uold, vold, u, v);
@@ -361,12 +363,13 @@ struct FxUpdate {
     }
 };
 
+template <bool SCALED>
 __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a) {
     constexpr int PER = (MPM_NODES + MPM_THREADS - 1) / MPM_THREADS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FxMarchSmem &sm = *reinterpret_cast<FxMarchSmem *>(smem_raw);
     const int tid = threadIdx.x;
-    const FxUpdate update(a);
+    const FxUpdate<SCALED> update(a);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     long long w = a.cuts[blockIdx.x];
@@ -476,12 +479,12 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
 }
 
 // The block form (k_mpm.cu): one block per CTA, every cell at once.
-template <int THREADS>
+template <int THREADS, bool SCALED>
 __global__ void __launch_bounds__(THREADS, THREADS > 128 ? 1 : 2) k_mpm_fixed_block(MpmArgs<double> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FxBlockSmem<THREADS> &sm = *reinterpret_cast<FxBlockSmem<THREADS> *>(smem_raw);
     const int tid = threadIdx.x;
-    const FxUpdate update(a);
+    const FxUpdate<SCALED> update(a);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     int r = 0;
     while (a.sched[r + 1].off <= blockIdx.x) ++r;
@@ -538,26 +541,29 @@ struct Form {   // kernel, threads, shared memory
     int threads;
     size_t smem;
 };
+template <bool SCALED>
 Form form_of(int variant) {
-    if (!mpm_is_block(variant)) return Form{k_mpm_fixed, MPM_THREADS, sizeof(FxMarchSmem)};
-    if (variant == MPM_BLOCK) return Form{k_mpm_fixed_block<MPM_THREADS>, MPM_THREADS, sizeof(FxBlockSmem<MPM_THREADS>)};
-    return Form{k_mpm_fixed_block<MPM_SMALL_BLOCK>, MPM_SMALL_BLOCK, sizeof(FxBlockSmem<MPM_SMALL_BLOCK>)};
+    if (!mpm_is_block(variant)) return Form{k_mpm_fixed<SCALED>, MPM_THREADS, sizeof(FxMarchSmem)};
+    if (variant == MPM_BLOCK)
+        return Form{k_mpm_fixed_block<MPM_THREADS, SCALED>, MPM_THREADS, sizeof(FxBlockSmem<MPM_THREADS>)};
+    return Form{k_mpm_fixed_block<MPM_SMALL_BLOCK, SCALED>, MPM_SMALL_BLOCK, sizeof(FxBlockSmem<MPM_SMALL_BLOCK>)};
 }
 
 }  // namespace
 
 cudaError_t mpm64_prepare() {
     for (int v : {0, (int)MPM_BLOCK, MPM_BLOCK + 1}) {
-        const Form f = form_of(v);
-        const cudaError_t e = cudaFuncSetAttribute(f.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem);
-        if (e != cudaSuccess) return e;
+        for (const Form &f : {form_of<false>(v), form_of<true>(v)}) {
+            const cudaError_t e = cudaFuncSetAttribute(f.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem);
+            if (e != cudaSuccess) return e;
+        }
     }
     return cudaSuccess;
 }
 
 template <>
 int mpm_per_sm<double>(int variant, int) {
-    const Form f = form_of(variant);
+    const Form f = form_of<false>(variant);
     int n = 1;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f.kernel, f.threads, f.smem);
     return (e != cudaSuccess || n < 1) ? 1 : n;
@@ -566,18 +572,8 @@ int mpm_per_sm<double>(int variant, int) {
 // programmatic stream serialisation, as the FP32 step
 template <>
 cudaError_t launch_mpm_step<double>(const MpmArgs<double> &a, int variant, cudaStream_t s) {
-    const Form f = form_of(variant);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.grid);
-    cfg.blockDim = dim3(f.threads);
-    cfg.dynamicSmemBytes = f.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, f.kernel, a);
+    const Form f = a.ukeep == 1.0 ? form_of<false>(variant) : form_of<true>(variant);
+    return launch_pdl(f.kernel, (unsigned)a.grid, (unsigned)f.threads, f.smem, s, a);
 }
 
 }  // namespace hmc

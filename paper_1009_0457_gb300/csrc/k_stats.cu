@@ -89,13 +89,25 @@ __device__ __forceinline__ void store4<double>(double *p, const double (&v)[4]) 
 // 128 threads 0.180 ms; 64 threads 0.156 ms; 32 threads 0.156 ms).  Each thread loads its next
 // block's corners and spins while it works on the current one (0.156 -> 0.150 ms), held to
 // 128 registers in FP32 (eight CTAs per SM).
+// WIDE: 256 threads with one block each, for grids of few CTAs, where the chain of four blocks is
+// longer than the pass; the blocks' sums go through shared memory and are added in the order
+// of the other form, so both give the same bits.  The line is one wave of its CTAs (profiler,
+// cold: FP32 106 CTAs 11.3 -> 7.8 us, 489 CTAs 14.2 -> 15.5 us; FP64 16 CTAs 91 -> 51 us).
 constexpr int STRESS_THREADS = 64;
 constexpr int STRESS_CELLS = BLOCK_THREADS / STRESS_THREADS;
 static_assert(BLOCK_THREADS % STRESS_THREADS == 0, "a tile splits evenly over the threads");
 
-template <typename T, bool STORE>
-__global__ void __launch_bounds__(STRESS_THREADS, sizeof(T) == 4 ? 8 : 1) k_stress(StressArgs<T> a) {
+// one wave of the wide form's CTAs on 152 SMs: two per SM in FP32, one in FP64
+template <typename T>
+constexpr int stress_wide() { return sizeof(T) == 4 ? 304 : 152; }
+
+template <typename T, bool STORE, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? BLOCK_THREADS : STRESS_THREADS, sizeof(T) == 4 ? (WIDE ? 2 : 8) : 1)
+    k_stress(StressArgs<T> a) {
     __shared__ double red[STRESS_THREADS / 32][7];
+    __shared__ T cells[WIDE ? BLOCK_THREADS : 1][7];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int rep = __ldg(a.cta_rep + blockIdx.x);
     const Replica &R = a.reps[rep];
     const int t0 = (blockIdx.x - R.cta_off) * BLOCK_THREADS;
@@ -130,7 +142,7 @@ __global__ void __launch_bounds__(STRESS_THREADS, sizeof(T) == 4 ? 8 : 1) k_stre
     int blk = t0 + threadIdx.x;
     if (blk < R.nblk) load_cell(blk, un, spn);
 #pragma unroll 1
-    for (int c8 = 0; c8 < STRESS_CELLS; ++c8) {
+    for (int c8 = 0; c8 < (WIDE ? 1 : STRESS_CELLS); ++c8) {
         if (blk >= R.nblk) break;
         T uc[8][3];
 #pragma unroll
@@ -139,7 +151,7 @@ __global__ void __launch_bounds__(STRESS_THREADS, sizeof(T) == 4 ? 8 : 1) k_stre
             for (int d = 0; d < 3; ++d) uc[i][d] = un[i][d];
         const uint4 sp = spn;
         const int blk_next = blk + STRESS_THREADS;
-        if (c8 + 1 < STRESS_CELLS && blk_next < R.nblk) load_cell(blk_next, un, spn);
+        if (!WIDE && c8 + 1 < STRESS_CELLS && blk_next < R.nblk) load_cell(blk_next, un, spn);
         CellGrad<T> g;
         cell_gradients<T>(uc, g);
         T csum[7] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0)};   // this cell's eight points, plain sums
@@ -175,14 +187,26 @@ __global__ void __launch_bounds__(STRESS_THREADS, sizeof(T) == 4 ? 8 : 1) k_stre
             }
         }
 #pragma unroll
-        for (int k = 0; k < 7; ++k) acc.add(k, csum[k]);
+        for (int k = 0; k < 7; ++k) {
+            if (WIDE)
+                cells[threadIdx.x][k] = csum[k];
+            else
+                acc.add(k, csum[k]);
+        }
         blk = blk_next;
+    }
+    if constexpr (WIDE) {
+        __syncthreads();
+        if (threadIdx.x >= STRESS_THREADS) return;
+        for (int t = threadIdx.x; t < BLOCK_THREADS && t0 + t < R.nblk; t += STRESS_THREADS)
+#pragma unroll
+            for (int k = 0; k < 7; ++k) acc.add(k, cells[t][k]);
     }
     acc.warp_reduce();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lane == 0)
         for (int i = 0; i < 7; ++i) red[warp][i] = acc.get(i);
-    __syncthreads();
+    asm volatile("bar.sync 1, %0;" ::"n"(STRESS_THREADS) : "memory");   // the two warps that sum
     if (threadIdx.x < 7) {
         double s = 0.0;
         for (int w = 0; w < STRESS_THREADS / 32; ++w) s += red[w][threadIdx.x];
@@ -190,94 +214,106 @@ __global__ void __launch_bounds__(STRESS_THREADS, sizeof(T) == 4 ? 8 : 1) k_stre
     }
 }
 
-// End of a step: fixed-order FP64 reduction of each replica's stress partials,
-// uniaxial control update of its mean strain, and its Monte Carlo step counter.
-// GB300 retires few FP64 operations per SM, so the partials (one set of seven per
-// stress CTA) are summed by END_GROUPS CTAs per replica: group g takes the CTAs
-// g, g + END_GROUPS, ... (each thread in that order, then a tree over the threads),
-// and the last group to arrive sums the group sums in group order and finishes.
-__global__ void __launch_bounds__(256) k_end_mcs(const Replica *reps, double *partials, int nctas, int update_strain,
-                                                  int advance) {
-    __shared__ double red[256][7];
+// sum over the lanes of a warp (a butterfly: every lane has it)
+__device__ __forceinline__ double lanes_sum(double x) {
+#pragma unroll
+    for (int off = 16; off; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    return x;
+}
+
+// End of a step: fixed-order FP64 reduction of each replica's stress partials (one set of seven
+// per stress CTA), uniaxial control update of its mean strain, and its Monte Carlo step counter.
+// Group g of G takes the CTAs g, g + G, ..., one warp per quantity; the last group to arrive sums the
+// group sums the same way and finishes with one lane per strain component.  A warp instruction of
+// the FP64 pipe takes 64 cycles however many lanes it serves, so what counts is the length of the
+// chain: 20 instead of about 150 of them (the 250-thread tree and the update by one thread took
+// 15 us; 4 us).
+__global__ void __launch_bounds__(224) k_end_mcs(const Replica *reps, int nrep, int gmax, double *partials, int nctas,
+                                                  int update_strain, int advance) {
+    __shared__ double tot[7];
     __shared__ int last;
-    const int r = blockIdx.x / END_GROUPS, grp = blockIdx.x % END_GROUPS;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int r = blockIdx.x / gmax, grp = blockIdx.x % gmax;
     const Replica &R = reps[r];
+    const int G = end_groups(R.ncta);
+    const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;   // quantity
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (grp >= G) return;
     DevState *st = R.st;
     double *gsum = partials + 7ll * nctas + 7ll * END_GROUPS * r;   // this replica's group sums
-    // the arrival counters follow the group sums of all replicas (gridDim.x = replicas x END_GROUPS)
-    unsigned *arrive = reinterpret_cast<unsigned *>(partials + 7ll * nctas + 7ll * gridDim.x) + r;
-    double s[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int p = grp + END_GROUPS * threadIdx.x; p < R.ncta; p += END_GROUPS * 256)
-        for (int i = 0; i < 7; ++i) s[i] += partials[7ll * (R.cta_off + p) + i];
-    for (int i = 0; i < 7; ++i) red[threadIdx.x][i] = s[i];
-    __syncthreads();
-    for (int w = 128; w; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int i = 0; i < 7; ++i) red[threadIdx.x][i] += red[threadIdx.x + w][i];
+    unsigned *arrive = reinterpret_cast<unsigned *>(partials + 7ll * nctas + 7ll * END_GROUPS * nrep) + r;
+    // the update's operands, loaded while the sums are formed (lane c: component c)
+    const int c = lane < 6 ? lane : 0;
+    double sr[6], axN = 0, axNs = 0, axB = 0, axNB = 1, eps0 = 0, sig0 = 0, ebar = 0;
+    if (i == 0) {
+#pragma unroll
+        for (int j = 0; j < 6; ++j) sr[j] = st->sr[6 * c + j];
+        axN = st->axN[c];
+        axNs = st->axNs[c];
+        axB = st->axB[c];
+        axNB = st->axNB;
+        eps0 = st->eps0;
+        sig0 = st->sig0;
+        ebar = st->ebar[c];
+    }
+    double s = 0.0;
+    for (int p = grp + G * lane; p < R.ncta; p += 32 * G) s += __ldcg(partials + 7ll * (R.cta_off + p) + i);
+    s = lanes_sum(s);
+    if (G == 1) {
+        if (lane == 0) tot[i] = s;
+        __syncthreads();
+    } else {
+        if (lane == 0) {
+            gsum[7 * grp + i] = s;
+            __threadfence();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(arrive, 1u) == (unsigned)G - 1u;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        double t = lane < G ? __ldcg(gsum + 7 * lane + i) : 0.0;
+        t = lanes_sum(t);
+        if (lane == 0) tot[i] = t;
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < 7; ++i) gsum[7 * grp + i] = red[0][i];
-        __threadfence();
-        last = atomicAdd(arrive, 1u) == END_GROUPS - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    // the last group of the replica: the group sums in group order
-    __threadfence();
-    if (threadIdx.x < 7) {
-        double t = 0.0;
-        for (int g = 0; g < END_GROUPS; ++g) t += __ldcg(gsum + 7 * g + threadIdx.x);
-        red[0][threadIdx.x] = t;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const double n_sites = 8.0 * (double)R.nblk;
-        double mean[6];
-        int bad = 0;
-        for (int i = 0; i < 6; ++i) {
-            mean[i] = red[0][i] / n_sites;
-            st->mean_sigma[i] = mean[i];
-            bad |= !isfinite(mean[i]);
-        }
-        st->energy = red[0][6];
-        bad |= !isfinite(red[0][6]);
+    if (i != 0) return;
+    const bool comp = lane < 6;
+    const double n_sites = 8.0 * (double)R.nblk;
+    const double mean = tot[c] / n_sites, energy = tot[6];
+    const bool bad = __any_sync(0xffffffffu, !isfinite(mean) || !isfinite(energy));
+    if (comp) st->mean_sigma[lane] = mean;
+    if (lane == 0) {
+        st->energy = energy;
         if (bad) st->nonfinite = 1;
-        if (update_strain && st->bc == 0 && !bad) {
-            // remove the lateral mean stress with the Reuss compliance, then restore
-            // the axial strain along the uniaxial-stress direction S_R (n(x)n)
-            double nsn = 0.0;
-            for (int i = 0; i < 6; ++i) nsn += st->axNs[i] * mean[i];
-            double r[6], e[6];
-            for (int i = 0; i < 6; ++i) r[i] = mean[i] - nsn * st->axN[i];
-            for (int i = 0; i < 6; ++i) {
-                double d = 0.0;
-                for (int j = 0; j < 6; ++j) d += st->sr[6 * i + j] * r[j];
-                e[i] = st->ebar[i] - d;
-            }
-            double ne = 0.0;
-            for (int i = 0; i < 6; ++i) ne += st->axN[i] * e[i];
-            const double beta = (st->eps0 - ne) / st->axNB;
-            for (int i = 0; i < 6; ++i) {
-                st->ebar[i] = e[i] + beta * st->axB[i];
-                st->ebar_f[i] = (float)st->ebar[i];
-            }
-        }
-        if (update_strain && st->bc == 2 && !bad) {
-            // stress control: Ebar += S_R (sig0 n(x)n - <sigma>)
-            double e[6];
-            for (int i = 0; i < 6; ++i) {
-                double d = 0.0;
-                for (int j = 0; j < 6; ++j) d += st->sr[6 * i + j] * (st->sig0 * st->axN[j] - mean[j]);
-                e[i] = st->ebar[i] + d;
-            }
-            for (int i = 0; i < 6; ++i) {
-                st->ebar[i] = e[i];
-                st->ebar_f[i] = (float)e[i];
-            }
-        }
         if (advance) st->mcs += 1;
         *arrive = 0u;   // ready for the next launch
+    }
+    if (!update_strain || bad) return;
+    if (st->bc == 0) {
+        // remove the lateral mean stress with the Reuss compliance, then restore
+        // the axial strain along the uniaxial-stress direction S_R (n(x)n)
+        const double nsn = lanes_sum(comp ? axNs * mean : 0.0);
+        const double q = mean - nsn * axN;
+        double d = 0.0;
+#pragma unroll
+        for (int j = 0; j < 6; ++j) d += sr[j] * __shfl_sync(0xffffffffu, q, j);
+        const double e = ebar - d;
+        const double beta = (eps0 - lanes_sum(comp ? axN * e : 0.0)) / axNB;
+        ebar = e + beta * axB;
+    } else if (st->bc == 2) {
+        // stress control: Ebar += S_R (sig0 n(x)n - <sigma>)
+        const double q = sig0 * axN - mean;
+        double d = 0.0;
+#pragma unroll
+        for (int j = 0; j < 6; ++j) d += sr[j] * __shfl_sync(0xffffffffu, q, j);
+        ebar += d;
+    } else {
+        return;
+    }
+    if (comp) {
+        st->ebar[lane] = ebar;
+        st->ebar_f[lane] = (float)ebar;
     }
 }
 
@@ -384,19 +420,18 @@ __global__ void k_bins(const unsigned long long *counts, const int32_t *binmap, 
 
 template <typename T>
 cudaError_t launch_stress(const StressArgs<T> &a, bool store, cudaStream_t s) {
-    if (store)
-        k_stress<T, true><<<a.nctas, STRESS_THREADS, 0, s>>>(a);
-    else
-        k_stress<T, false><<<a.nctas, STRESS_THREADS, 0, s>>>(a);
-    return cudaGetLastError();
+    if (a.nctas <= stress_wide<T>())
+        return launch_pdl(store ? k_stress<T, true, true> : k_stress<T, false, true>, a.nctas, BLOCK_THREADS, 0, s, a);
+    return launch_pdl(store ? k_stress<T, true, false> : k_stress<T, false, false>, a.nctas, STRESS_THREADS, 0, s, a);
 }
 template cudaError_t launch_stress<float>(const StressArgs<float> &, bool, cudaStream_t);
 template cudaError_t launch_stress<double>(const StressArgs<double> &, bool, cudaStream_t);
 
-cudaError_t launch_end_mcs(const Replica *reps, int nrep, double *partials, int nctas, int update_strain, int advance,
-                           cudaStream_t s) {
-    k_end_mcs<<<nrep * END_GROUPS, 256, 0, s>>>(reps, partials, nctas, update_strain, advance);
-    return cudaGetLastError();
+cudaError_t launch_end_mcs(const Replica *reps, int nrep, int max_ncta, double *partials, int nctas, int update_strain,
+                           int advance, cudaStream_t s) {
+    const int gmax = end_groups(max_ncta);
+    return launch_pdl(k_end_mcs, (unsigned)(nrep * gmax), 224u, 0, s, reps, nrep, gmax, partials, nctas, update_strain,
+                      advance);
 }
 
 static int grid_for(long long n) {

@@ -355,6 +355,9 @@ __global__ void __launch_bounds__(CTA, flat_min_ctas<T, MODE, RECOMP, CTA>())
     constexpr bool STORED = ELASTIC && !RECOMP;                               // ... from the stored stress
     constexpr bool LIST = MODE == SWEEP_ZONE_LIST;
     extern __shared__ __align__(128) unsigned char sweep_smem[];
+    // the next kernel may be scheduled; everything below waits for the kernels before this one
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     FlatSmem<T, STORED, CTA> &fs = *reinterpret_cast<FlatSmem<T, STORED, CTA> *>(sweep_smem);
     auto &sl = fs.list;
     // the red half sweep follows the stress pass: its CTAs take the tiles in reverse order, so
@@ -621,9 +624,9 @@ void launch_flat_cta(const SweepArgs<T> &a, cudaStream_t s) {
     constexpr int SPLIT = split_of<CTA>();
     constexpr size_t smem = flat_smem_bytes<T, MODE, RECOMP, CTA>();
     if (a.nrep == 1)
-        k_sweep<T, MODE, RECOMP, COL, true, false, CTA><<<a.nctas * SPLIT, CTA, smem, s>>>(a);
+        launch_pdl(k_sweep<T, MODE, RECOMP, COL, true, false, CTA>, a.nctas * SPLIT, CTA, smem, s, a);
     else
-        k_sweep<T, MODE, RECOMP, COL, false, false, CTA><<<a.nctas * SPLIT, CTA, smem, s>>>(a);
+        launch_pdl(k_sweep<T, MODE, RECOMP, COL, false, false, CTA>, a.nctas * SPLIT, CTA, smem, s, a);
 }
 
 template <typename T, int MODE, bool RECOMP, int COL>
