@@ -80,8 +80,9 @@ struct hmc_handle {
     int cexp = 0;
     // 27-point zone (HMC_ELASTIC_ZONE1): trial list, start-of-step spins, element tables, schedule
     uint4 *zone_work = nullptr, *snap = nullptr;
-    unsigned *zone_count = nullptr;
-    void *ktab = nullptr;
+    unsigned *zone_count = nullptr;       // listed trials, trials that the bounds leave open
+    unsigned *zone_open = nullptr;        // the open ones; NULL: every trial is decided by the elimination
+    void *ktab = nullptr, *btab = nullptr;   // element tables; forms of the bounds
     void *stab = nullptr;                 // compliance rows (constant-strain zone)
     uint16_t *zone_sched = nullptr;
     int zone_nsched = 0, zone_grid = 1, zone_scatter_off = 0;
@@ -372,7 +373,7 @@ cudaError_t enqueue_sweep(hmc_handle *h, int colour, cudaStream_t s) {
     // 27-point zone: list the trials, copy the spins as they are at the start of the half step,
     // then decide every listed trial against that copy
     cudaError_t e;
-    if ((e = cudaMemsetAsync(h->zone_count, 0, sizeof(unsigned), s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(h->zone_count, 0, 2 * sizeof(unsigned), s)) != cudaSuccess) return e;
     if ((e = hmc::launch_sweep<T>(a, colour, hmc::SWEEP_ZONE_LIST, false, s)) != cudaSuccess) return e;
     if ((e = cudaMemcpyAsync(h->snap, h->spins, sizeof(uint4) * (size_t)h->nblk_total, cudaMemcpyDeviceToDevice,
                              s)) != cudaSuccess)
@@ -384,7 +385,9 @@ cudaError_t enqueue_sweep(hmc_handle *h, int colour, cudaStream_t s) {
     z.u = static_cast<const T *>(h->u[h->cur]);
     z.ctab = static_cast<const T *>(h->ctab);
     z.ktab = static_cast<const T *>(h->ktab);
+    z.btab = static_cast<const T *>(h->btab);
     z.work = h->zone_work;
+    z.open = h->zone_open;
     z.count = h->zone_count;
     z.thr = h->thr;
     z.sched = h->zone_sched;
@@ -392,6 +395,10 @@ cudaError_t enqueue_sweep(hmc_handle *h, int colour, cudaStream_t s) {
     z.nsched = h->zone_nsched;
     z.J = (T)h->p.J;
     z.kT = (T)h->p.kT;
+    // The bounds hold for any stiffness, but far from isotropic ones (ratio of the largest to the
+    // smallest of C11 + 2 C12, C11 - C12, 2 C44 above 30) may break down in the elimination, which fails
+    // the trial (HMC_ERR_NONFINITE), and lie past the margin: such handles decide every trial by it
+    if (h->zone_open && (e = hmc::launch_zone_bounds<T>(z, 8 * h->num_sms, s)) != cudaSuccess) return e;
     return hmc::launch_zone<T>(z, h->zone_grid, s);
 }
 
@@ -560,7 +567,7 @@ void destroy_buffers(hmc_handle *h) {
         if (h->gexec[i]) cudaGraphExecDestroy(h->gexec[i]);
     void *bufs[] = {h->spins, h->stage16, h->u[0], h->u[1], h->v, h->sig, h->ctab, h->cubw, h->cfix, h->wtab, h->atab, h->thr, h->counts,
                     h->bins, h->partials, h->fractions, h->binmap, h->st, h->d_reps, h->d_cta_rep, h->d_sched, h->d_cuts,
-                    h->zone_work, h->snap, h->zone_count, h->ktab, h->zone_sched, h->cc_parent, h->cc_count,
+                    h->zone_work, h->snap, h->zone_count, h->zone_open, h->btab, h->ktab, h->zone_sched, h->cc_parent, h->cc_count,
                     h->stab, h->plain_sig, h->plain_f};
     for (void *b : bufs)
         if (b) cudaFree(b);
@@ -1200,15 +1207,20 @@ hmc_status hmc_create_batch(const hmc_params *params, int32_t n_replicas, hmc_ha
         zs.resize((zs.size() + 7) & ~size_t(7), 0);   // the scatter table starts 16-byte aligned
         h->zone_scatter_off = (int)zs.size();
         zs.insert(zs.end(), scat.begin(), scat.end());
+        const double stiffest = std::fmax(std::fmax(p->c11 + 2 * p->c12, p->c11 - p->c12), 2 * p->c44);
+        const double softest = std::fmin(std::fmin(p->c11 + 2 * p->c12, p->c11 - p->c12), 2 * p->c44);
+        const bool well = stiffest <= 30 * softest;
         Alloc za[] = {
             {(void **)&h->zone_work, sizeof(uint4) * 4 * (size_t)h->nblk_total, "zone trial list"},
             {(void **)&h->snap, sizeof(uint4) * (size_t)h->nblk_total, "spin copy"},
-            {(void **)&h->zone_count, sizeof(unsigned), "zone trial count"},
+            {(void **)&h->zone_count, 2 * sizeof(unsigned), "zone trial count"},
+            {(void **)&h->zone_open, well ? sizeof(unsigned) * 4 * (size_t)h->nblk_total : 0, "zone trial list"},
+            {&h->btab, well ? h->tsize * 8 * 48 * (size_t)p->n_orient : 0, "zone bound tables"},
             {&h->ktab, h->tsize * 8 * 320 * (size_t)p->n_orient, "zone element tables"},
             {(void **)&h->zone_sched, sizeof(uint16_t) * zs.size(), "zone schedule"},
         };
         for (auto &a : za)
-            if ((e = cudaMalloc(a.ptr, a.bytes)) != cudaSuccess) return bail(cuda_fail(h, e, a.what));
+            if (a.bytes > 0 && (e = cudaMalloc(a.ptr, a.bytes)) != cudaSuccess) return bail(cuda_fail(h, e, a.what));
         if ((e = cudaMemcpy(h->zone_sched, zs.data(), sizeof(uint16_t) * zs.size(), cudaMemcpyHostToDevice)) !=
             cudaSuccess)
             return bail(cuda_fail(h, e, "zone schedule upload"));
@@ -1364,15 +1376,15 @@ hmc_status hmc_set_orientations(hmc_handle *h, const double *euler, const uint16
         }
     }
     if (h->p.elastic == HMC_ELASTIC_ZONE1) {
-        std::vector<double> kt;
+        std::vector<double> kt, bt;
         hmc::zone_element_tables(h->Cv.data(), Q, kt);
-        if (h->p.precision == HMC_FP32) {
-            std::vector<float> kf(kt.begin(), kt.end());
-            HMC_CK(h, cudaMemcpy(h->ktab, kf.data(), kf.size() * sizeof(float), cudaMemcpyHostToDevice),
-                   "zone table upload");
-        } else {
-            HMC_CK(h, cudaMemcpy(h->ktab, kt.data(), kt.size() * sizeof(double), cudaMemcpyHostToDevice),
-                   "zone table upload");
+        if (h->btab) hmc::zone_bound_tables(h->Cv.data(), Q, h->p.c11, h->p.c12, h->p.c44, bt);
+        const std::pair<void *, const std::vector<double> *> up[] = {{h->ktab, &kt}, {h->btab, &bt}};
+        for (const auto &[dev, t] : up) {
+            if (t->empty()) continue;
+            const std::vector<float> f(h->tsize == 4 ? t->begin() : t->end(), t->end());
+            const void *src = h->tsize == 4 ? static_cast<const void *>(f.data()) : t->data();
+            HMC_CK(h, cudaMemcpy(dev, src, t->size() * h->tsize, cudaMemcpyHostToDevice), "zone table upload");
         }
     }
     const size_t nodes_b = node_bytes(h);

@@ -162,7 +162,7 @@ struct SweepArgs {
     int trial, nq;
     T J, kT;
     int nctas;
-    uint4 *work;                     // zone mode: trial list {site, replica, q_new | q_old << 16, r1}
+    uint4 *work;                     // zone mode: trial list {site, replica | (dE + 8) << 28, q_new | q_old << 16, r1}
     unsigned *count;                 // zone mode: entries in the list
     const T *ctab, *stab;            // constant-strain mode: stiffness and compliance rows (Q x 24)
     const T *u;                      // recompute mode: nodal displacement (the stress of a trial site
@@ -200,8 +200,10 @@ struct ZoneArgs {
     const T *u;                      // nodal displacement
     const T *ctab;                   // Q x 24 rotated stiffness
     const T *ktab;                   // Q x 8 x 300 element stiffness of a point per position in its cell
-    const uint4 *work;
-    const unsigned *count;
+    const T *btab;                   // Q x 8 x 48: per position in its cell, two forms of the relaxing energy
+    const uint4 *work;               // trials: {site, replica | (dE + 8) << 28, q_new | q_old << 16, r1}
+    unsigned *open;                  // trials that the bounds leave open (indices into work); NULL: no bounds
+    unsigned *count;                 // entries of work, entries of open
     const unsigned long long *thr;
     const uint16_t *sched;           // elimination schedule (zone_schedule)
     const uint16_t *scatter;         // element-matrix places per reflection and zone cell (zone_scatter_table)
@@ -249,6 +251,8 @@ cudaError_t launch_sweep(const SweepArgs<T> &a, int colour, int mode, bool recom
 template <typename T>
 cudaError_t launch_sweep_margin(const SweepArgs<T> &a, int colour, int mode, cudaStream_t s);
 template <typename T>
+cudaError_t launch_zone_bounds(const ZoneArgs<T> &a, int grid, cudaStream_t s);
+template <typename T>
 cudaError_t launch_zone(const ZoneArgs<T> &a, int grid, cudaStream_t s);
 template <typename T>
 int zone_per_sm();                 // resident zone CTAs per SM
@@ -256,6 +260,7 @@ cudaError_t zone_prepare();        // opt the zone kernels into their dynamic sh
 std::vector<uint16_t> zone_schedule();   // empty if it does not fit the kernel's table
 std::vector<uint16_t> zone_scatter_table(const std::vector<uint16_t> &schedule);
 void zone_element_tables(const double *Cv, int Q, std::vector<double> &out);
+void zone_bound_tables(const double *Cv, int Q, double c11, double c12, double c44, std::vector<double> &out);
 cudaError_t mpm_prepare();  // opt the MPM kernels into their dynamic shared memory (once, before any capture)
 cudaError_t mpm64_prepare();  // ... those of the FP64 step
 cudaError_t sweep_prepare();  // opt the elastic sweeps into their shared memory

@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(CTA, flat_min_ctas<T, MODE, RECOMP, CTA>())
             const int lx = L & 1, ly = (L >> 1) & 1, lz = L >> 2;
             if (LIST) {
                 const uint32_t x = 2u * bx + lx, y = 2u * by + ly, z = 2u * bz + lz;
-                const uint4 en = make_uint4(x + (uint32_t)R.nx * (y + (uint32_t)R.ny * z), (uint32_t)r,
+                const uint4 en = make_uint4(x + (uint32_t)R.nx * (y + (uint32_t)R.ny * z), (uint32_t)r | (uint32_t)(dE[i] + 8) << 28,
                                             (uint32_t)qn[i] | ((uint32_t)q[i] << 16), rnd[i].y);
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
