@@ -163,7 +163,7 @@ def kernel_traffic(kernel):
 
 def mpm_variant_name(v):
     return ["march 16x16", "march 32x8", "march 8x32", "march, fewest patches", "march, fewest cells", "block",
-            "small block"][v]
+            "small block", "march 16x8, four to a CTA", "march 16x8", "half march, fewest cells"][v]
 
 
 def dist_reduce(t_local, units_local, device="cpu"):

@@ -173,7 +173,9 @@ hmc_status hmc_select_replica(hmc_handle *h, int32_t r);
  * default before it): MPM variant v and the number of CTAs of a step.  March
  * up z over patches that own 0: 15x15, 1: 31x7, 2: 7x31 nodes, 3: as many as
  * make the fewest patches of even size, 4: as many as make the fewest cells;
- * one pass over blocks of at most 5: 256, 6: 96 cells.  The autotuner times
+ * one pass over blocks of at most 5: 256, 6: 96 cells; FP32 also marches of
+ * 128 threads over patches of 7: 15x7 nodes, four marches to a CTA, 8: 15x7,
+ * 9: as many as make the fewest cells.  The autotuner times
  * the candidates on scratch copies of the nodal state; all variants give
  * bit-identical results.  Environment variable HMC_AUTOTUNE=0 keeps variant
  * 0; HMC_MPM_SHAPE=<v> forces one. */

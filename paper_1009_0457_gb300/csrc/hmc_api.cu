@@ -100,7 +100,7 @@ struct hmc_handle {
     hmc::MpmSched *d_sched = nullptr;     // R + 1 MPM schedules for the chosen variant
     long long *d_cuts = nullptr;          // march: first work item of every CTA
     // MPM launch configuration (autotuned)
-    int mpm_shape = 0, mpm_grid = 1;      // variant and CTAs
+    int mpm_shape = 0, mpm_grid = 1, mpm_ranges = 1;   // variant, CTAs, ranges of work
     bool tuned = false;
     int sweep_cta = 256;                  // sweep threads per CTA (tuned)
     double *plain_sig = nullptr, *plain_f = nullptr;   // the plain FP64 step's point stresses, cell forces
@@ -287,6 +287,7 @@ hmc::MpmArgs<T> mpm_args(hmc_handle *h, const void *u_in, void *u_out, void *v) 
     a.sched = h->d_sched;
     a.nrep = h->R;
     a.cuts = h->d_cuts;
+    a.ranges = h->mpm_ranges;
     a.spins = h->spins;
     a.u_in = static_cast<const T *>(u_in);
     a.u_out = static_cast<T *>(u_out);
@@ -611,19 +612,21 @@ void pack_stress_host(const RepHost &R, const double *in, std::vector<T> &packed
 
 // Most nodes that a tile (march) or block of variant v owns per edge of a replica.
 void patch_of(int v, const RepHost &R, int (&o)[3]) {
+    const bool half = v >= hmc::MPM_HALF;   // a march of 128 threads
     const int n[3] = {R.nbx, R.nby, R.nbz};
-    if (v < hmc::MPM_FIT) {
-        const int fixed[3][2] = {{15, 15}, {31, 7}, {7, 31}};
-        o[0] = std::min(fixed[v][0], n[0]);
-        o[1] = std::min(fixed[v][1], n[1]);
+    if (v < hmc::MPM_FIT || v == hmc::MPM_QUAD || v == hmc::MPM_HALF + 1) {
+        const int fixed[4][2] = {{15, 15}, {31, 7}, {7, 31}, {15, 7}};
+        o[0] = std::min(fixed[half ? 3 : v][0], n[0]);
+        o[1] = std::min(fixed[half ? 3 : v][1], n[1]);
         o[2] = n[2];
         return;
     }
     const bool block = hmc::mpm_is_block(v);
-    const int cells = v == hmc::MPM_BLOCK + 1 ? hmc::MPM_SMALL_BLOCK : hmc::MPM_THREADS;
-    const int nodes = block ? 2 * cells : hmc::MPM_NODES;
+    const int cells = v == hmc::MPM_BLOCK + 1 ? hmc::MPM_SMALL_BLOCK : half ? hmc::MPM_HALF_THREADS : hmc::MPM_THREADS;
+    const int nodes = block ? 2 * cells : half ? hmc::MPM_HALF_NODES : hmc::MPM_NODES;
     // over every division of the edges into tiles of even size that the CTA's threads and node
-    // buffer hold: fewest tiles, then fewest cells (variant 4: fewest cells, then fewest tiles)
+    // buffer hold: fewest tiles, then fewest cells (variants 4 and 9: fewest cells, then fewest tiles)
+    const bool by_cells = v == hmc::MPM_FIT + 1 || half;
     long long best[2] = {0, 0};
     auto tiles_of = [](int edge, int own) { return (edge + own - 1) / own; };
     for (int x = 1; x <= n[0] && 2 * (x + 1) <= cells; ++x) {
@@ -639,7 +642,7 @@ void patch_of(int v, const RepHost &R, int (&o)[3]) {
                 if (!block && (x + 2) * (y + 2) > nodes) break;
                 const long long tiles = (long long)tx * ty * tz;
                 const long long work = (long long)(n[0] + tx) * (n[1] + ty) * (block ? n[2] + tz : 1);
-                const long long key[2] = {v == hmc::MPM_FIT + 1 ? work : tiles, v == hmc::MPM_FIT + 1 ? tiles : work};
+                const long long key[2] = {by_cells ? work : tiles, by_cells ? tiles : work};
                 if (best[0] == 0 || key[0] < best[0] || (key[0] == best[0] && key[1] < best[1])) {
                     best[0] = key[0];
                     best[1] = key[1];
@@ -657,7 +660,7 @@ void patch_of(int v, const RepHost &R, int (&o)[3]) {
 struct MpmPlan {
     std::vector<hmc::MpmSched> sched;
     std::vector<long long> cuts;
-    int grid = 1;
+    int grid = 1, ranges = 1;   // CTAs of a step; march: ranges of work items
 };
 
 MpmPlan plan_mpm(const hmc_handle *h, int variant, int per_sm_limit) {
@@ -682,10 +685,10 @@ MpmPlan plan_mpm(const hmc_handle *h, int variant, int per_sm_limit) {
         off += (long long)S.tiles_x * S.tiles_y * (block ? S.tiles_z : R.nbz);
     }
     if (block) {
-        P.grid = (int)off;
+        P.grid = P.ranges = (int)off;
         return P;
     }
-    // March: a CTA that starts or enters a tile computes one plane of cells more than it owns of
+    // March: a march that starts or enters a tile computes one plane of cells more than it owns of
     // nodes.  With at most K planes of cells per CTA, filling the CTAs in order needs the fewest of
     // them; take the smallest K that the resident CTAs hold.  (At 128^3 the even split left CTAs of
     // 8 planes beside 6; now none has more than 6.)
@@ -722,14 +725,15 @@ MpmPlan plan_mpm(const hmc_handle *h, int variant, int per_sm_limit) {
         else
             lo = K + 1;
     }
-    P.grid = (int)fill(lo, &P.cuts);
+    P.ranges = (int)fill(lo, &P.cuts);
     // Long ranges: an even split over every resident CTA, unless it leaves one noticeably longer (at
     // 256^3, 36 of 37 planes, the filled form needs 299 of 304 CTAs and its step took 101 us against 100)
-    if (lo >= 16 && P.grid < slots) {
-        P.grid = (int)slots;
+    if (lo >= 16 && P.ranges < slots) {
+        P.ranges = (int)slots;
         P.cuts.resize(slots + 1);
         for (long long c = 0; c <= slots; ++c) P.cuts[c] = off * c / slots;
     }
+    P.grid = std::min(P.ranges, (int)(slots / hmc::mpm_groups(variant)));
     return P;
 }
 
@@ -742,6 +746,7 @@ hmc_status apply_plan(hmc_handle *h, int variant, const MpmPlan &P) {
                "schedule upload");
     h->mpm_shape = variant;
     h->mpm_grid = P.grid;
+    h->mpm_ranges = P.ranges;
     return HMC_OK;
 }
 
@@ -777,10 +782,11 @@ hmc_status tune_mpm(hmc_handle *h, bool enabled, int &best_limit) {
     cudaEventCreate(&e1);
     float best = 1e30f;
     cudaError_t err = cudaMemcpyAsync(vs, h->v, nb, cudaMemcpyDeviceToDevice, h->stream);
-    for (int v = 0; v < hmc::MPM_NVARIANTS && err == cudaSuccess && s == HMC_OK; ++v) {
+    const int nvariants = hmc::mpm_nvariants(h->p.precision == HMC_FP32);
+    for (int v = 0; v < nvariants && err == cudaSuccess && s == HMC_OK; ++v) {
         // a march with every resident CTA and with one per SM; the block form where its blocks are
         // few enough for it to be in question
-        for (int limit = 0; limit < (hmc::mpm_is_block(v) ? 1 : 2); ++limit) {
+        for (int limit = 0; limit < (v >= hmc::MPM_BLOCK ? 1 : 2); ++limit) {
             const MpmPlan P = plan_mpm(h, v, limit);
             if (hmc::mpm_is_block(v) && P.grid > 16 * h->num_sms) continue;
             if ((s = apply_plan(h, v, P)) != HMC_OK) break;
@@ -930,7 +936,8 @@ hmc_status ensure_tuned(hmc_handle *h) {
     const bool enabled = !(env && env[0] == '0');
     const char *forced = std::getenv("HMC_MPM_SHAPE");
     const char *forced_cta = std::getenv("HMC_SWEEP_CTA");
-    const bool force_mpm = forced && forced[0] >= '0' && forced[0] < '0' + hmc::MPM_NVARIANTS && forced[1] == 0;
+    const bool force_mpm = forced && forced[0] >= '0' && forced[0] < '0' + hmc::mpm_nvariants(h->p.precision == HMC_FP32) &&
+                           forced[1] == 0;
     const bool force_cta = forced_cta && (std::string(forced_cta) == "128" || std::string(forced_cta) == "256");
     const std::string sig = tune_signature(h);
     if (!force_mpm && !force_cta) {

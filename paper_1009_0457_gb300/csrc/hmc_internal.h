@@ -103,7 +103,8 @@ struct MpmArgs {
     const Replica *reps;
     const MpmSched *sched;   // nrep + 1 entries
     int nrep;
-    const long long *cuts;   // march: first work item of every CTA, then the total (grid + 1)
+    const long long *cuts;   // march: first work item of every range, then the total (ranges + 1)
+    int ranges;
     const uint4 *spins;
     const T *u_in;
     T *u_out;
@@ -213,12 +214,17 @@ struct ZoneArgs {
 
 // MPM variants.  March with owned patches of 0: 15x15, 1: 31x7, 2: 7x31 nodes (cut off at the
 // high edges), 3: as few patches as can be of even size, 4: as few cells as can be; block form with
-// 5: blocks of at most 256 cells, 6: at most MPM_SMALL_BLOCK cells.
-enum { MPM_FIT = 3, MPM_BLOCK = 5, MPM_NVARIANTS = 7 };
+// 5: blocks of at most 256 cells, 6: at most MPM_SMALL_BLOCK cells; FP32 march of 128 threads with
+// 7: owned patches of 15x7, four marches to a CTA, 8: 15x7, 9: as few cells as can be.
+enum { MPM_FIT = 3, MPM_BLOCK = 5, MPM_HALF = 7, MPM_QUAD = 7 };
+inline int mpm_nvariants(bool fp32) { return fp32 ? 10 : 7; }
+inline int mpm_groups(int variant) { return variant == MPM_QUAD ? 4 : 1; }   // marches to a CTA
 constexpr int MPM_THREADS = 256;     // threads of a step's CTA = most cells of a patch plane or block
 constexpr int MPM_SMALL_BLOCK = 96;  // ... of the small-block form
+constexpr int MPM_HALF_THREADS = 128;
 constexpr int MPM_NODES = 304;       // most nodes of a patch's plane, (W+1)(H+1)
-inline bool mpm_is_block(int variant) { return variant >= MPM_BLOCK; }
+constexpr int MPM_HALF_NODES = 176;  // ... of a march of 128 threads
+inline bool mpm_is_block(int variant) { return variant == MPM_BLOCK || variant == MPM_BLOCK + 1; }
 
 // A launch with programmatic stream serialisation: the kernel may be scheduled before the one ahead
 // of it in the stream has finished, and executes griddepcontrol.wait before it reads or writes
@@ -265,7 +271,7 @@ cudaError_t mpm_prepare();  // opt the MPM kernels into their dynamic shared mem
 cudaError_t mpm64_prepare();  // ... those of the FP64 step
 cudaError_t sweep_prepare();  // opt the elastic sweeps into their shared memory
 template <typename T>
-int mpm_per_sm(int variant, int nq);  // resident MPM CTAs per SM
+int mpm_per_sm(int variant, int nq);  // resident marches (block form: blocks) per SM
 
 // End-of-step reduction, loading update (update_strain) and MCS counter (advance).  A replica's stress
 // partials are summed in a fixed order in FP64 by end_groups(its CTAs) CTAs, and the last of them to

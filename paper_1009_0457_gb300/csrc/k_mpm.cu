@@ -6,7 +6,7 @@
 //
 // Two forms, chosen per batch by the autotuner; both give the same bits.
 //
-// March (k_mpm_step): a CTA of 256 threads computes a patch of W x H <= 256 cells per cell
+// March (k_mpm_step): 256 or 128 threads compute a patch of W x H <= 256 or 128 cells per cell
 // plane (one thread per cell, all eight points of the cell) and owns the (W-1) x (H-1) nodes
 // whose four lower and four upper cells all lie in the patch.  It marches up a chunk of planes
 // in z: each cell writes its eight nodal force contributions to shared memory, and a node's
@@ -42,10 +42,12 @@ struct alignas(16) Vec4 {
     float x, y, z, p;
 };
 
+template <int GT>
 struct MarchSmem {
-    Vec4 us[3][MPM_NODES];         // node planes, row-major with W + 1 nodes a row, held as u/32
-    Vec4 fb[4][MPM_THREADS];       // cell contributions to their lower corner nodes (corner I+2J)
-    Vec4 ft[4][MPM_THREADS];       // ... to their upper corner nodes
+    static constexpr int NODES = GT == MPM_THREADS ? MPM_NODES : MPM_HALF_NODES;
+    Vec4 us[3][NODES];             // node planes, row-major with a patch's nodes a row, held as u/32
+    Vec4 fb[4][GT];                // cell contributions to their lower corner nodes (corner I+2J)
+    Vec4 ft[4][GT];                // ... to their upper corner nodes
 };
 template <int THREADS>
 struct BlockSmem {
@@ -55,15 +57,16 @@ struct BlockSmem {
 
 // Node plane k of a patch with origin node (i0-1, j0-1) and P nodes a row, read from global
 // memory into registers / written to shared memory.
+template <int GT>
 struct PlaneLoad {
-    static constexpr int PER = (MPM_NODES + MPM_THREADS - 1) / MPM_THREADS;
+    static constexpr int PER = (MarchSmem<GT>::NODES + GT - 1) / GT;
     float r[PER][3];
     int col[PER];   // this thread's nodes as (i + nbx j) in the replica's node plane, -1 beyond the patch
     // once per tile: the periodic (i, j) of each node this thread loads
     __device__ __forceinline__ void prepare(int i0, int j0, int P, int n, int nbx, int nby) {
 #pragma unroll
         for (int m = 0; m < PER; ++m) {
-            const int t = threadIdx.x + m * MPM_THREADS;
+            const int t = threadIdx.x % GT + m * GT;
             col[m] = t < n ? wrapi(i0 - 1 + t % P, nbx) + nbx * wrapi(j0 - 1 + t / P, nby) : -1;
         }
     }
@@ -84,7 +87,7 @@ struct PlaneLoad {
 #pragma unroll
         for (int m = 0; m < PER; ++m)
             if (col[m] >= 0)
-                us[threadIdx.x + m * MPM_THREADS] =
+                us[threadIdx.x % GT + m * GT] =
                     Vec4{r[m][0] * 0.03125f, r[m][1] * 0.03125f, r[m][2] * 0.03125f, 0.f};
     }
 };
@@ -280,31 +283,52 @@ __device__ __forceinline__ void take(float (&u)[3], const Vec4 &n) {
     u[2] = n.z;
 }
 
+// barrier of one march (barrier 0 is the CTA's own)
+template <int GT, int GROUPS>
+__device__ __forceinline__ void march_sync() {
+    if constexpr (GROUPS == 1)
+        __syncthreads();
+    else
+        asm volatile("bar.sync %0, %1;" ::"r"((int)(threadIdx.x / GT) + 1), "n"(GT) : "memory");
+}
+
 // PITCH: nodes a row of the patch, 0 for W + 1 (the 16x16 patch's constant 17 saves 1 % at 256^3)
-template <bool STAB, int PITCH>
-__global__ void __launch_bounds__(MPM_THREADS, 2) k_mpm_step(MpmArgs<float> a) {
+// GT: threads of a march, GROUPS: marches to a CTA, which share its orientation table and run on
+// their own behind barriers of their own.  A march of 128 threads computes 8 % more halo than one of
+// 256, but four of them per SM are out of step with each other, so that one's barriers and node
+// updates lie under the others' cells: at 200^3 (256 orientations) 50.0 -> 48.8 us a step.  At 256^3
+// (1024 orientations, a table of 48 KB) four tables would not fit; with one for four marches, which
+// also leaves L1 43 KB more than two CTAs of 256 do, 96.7 -> 88.1 us.
+template <int GT, int GROUPS, bool STAB, int PITCH>
+__global__ void __launch_bounds__(GT *GROUPS, 512 / (GT * GROUPS)) k_mpm_step(MpmArgs<float> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    MarchSmem &sm = *reinterpret_cast<MarchSmem *>(smem_raw);
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x % GT;
+    MarchSmem<GT> &sm = reinterpret_cast<MarchSmem<GT> *>(smem_raw)[threadIdx.x / GT];
     const float fscale = -a.dt_over_m * 0.03125f;          // -dt / (32 m)
     // the next step may be launched now: its CTAs take the SM slots this grid's CTAs free
     // and stage their table while this grid finishes
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const float *cw = stage_table<STAB>(a, smem_raw + sizeof(MarchSmem));
+    const float *cw = stage_table<STAB>(a, smem_raw + GROUPS * sizeof(MarchSmem<GT>));
     float cub[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) cub[i] = a.cub[i];
     // everything above reads only constant tables; u, v, the spins and the mean strain come
     // from the kernels before this one
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    // this CTA's contiguous range of the linear (replica, tile, plane) index
-    long long w = a.cuts[blockIdx.x];
-    const long long wend = a.cuts[blockIdx.x + 1];
+    // this march's contiguous range of the linear (replica, tile, plane) index; those of a CTA lie far
+    // apart, so that fewer ranges than there is room for load the SMs evenly
+    const int range = GROUPS == 1 ? (int)blockIdx.x : (int)(threadIdx.x / GT * gridDim.x + blockIdx.x);
+    if (GROUPS > 1 && range >= a.ranges) return;
+    long long w = a.cuts[range];
+    const long long wend = a.cuts[range + 1];
     int r = 0;
     while (w < wend) {
         while (a.sched[r + 1].off <= w) ++r;              // replica of work item w (ranges are ascending)
         const Replica &R = a.reps[r];
         const MpmSched &SC = a.sched[r];
+        // in a register: read through the table it is loaded again in every plane, because the stores of
+        // u and v might alias it (at 256^3 97 -> 88 us with four marches a CTA, 99.6 -> 96.7 with one)
+        const long long node0 = R.blk_off;
         const int nbx = R.nbx, nby = R.nby, nbz = R.nbz;
         const long long lw = w - SC.off;
         const int tile = (int)(lw / nbz);
@@ -321,20 +345,20 @@ __global__ void __launch_bounds__(MPM_THREADS, 2) k_mpm_step(MpmArgs<float> a) {
         const bool need = tid < W * H;
         const bool own = need && lci >= 1 && lcj >= 1;        // it owns the node at its cell's lower corner
         const int plane = nbx * nby;
-        const long long col = R.blk_off + wrapi(i0 - 1 + lci, nbx) + nbx * wrapi(j0 - 1 + lcj, nby);
+        const long long col = node0 + wrapi(i0 - 1 + lci, nbx) + nbx * wrapi(j0 - 1 + lcj, nby);
         const int nd = lci + P * lcj;                         // that node in the patch
         float eb[6];
         load_ebar<float>(R.st, eb);
 
-        PlaneLoad pl;
+        PlaneLoad<GT> pl;
         int b0 = 0, b1 = 1, b2 = 2;
         pl.prepare(i0, j0, P, P * (H + 1), nbx, nby);
-        pl.fetch(a.u_in, R.blk_off, k0 - 1, nbz, plane);
+        pl.fetch(a.u_in, node0, k0 - 1, nbz, plane);
         pl.store(sm.us[b0]);
-        pl.fetch(a.u_in, R.blk_off, k0, nbz, plane);
+        pl.fetch(a.u_in, node0, k0, nbz, plane);
         pl.store(sm.us[b1]);
         uint4 sp = need ? __ldg(a.spins + col + (long long)plane * wrapi(k0 - 1, nbz)) : make_uint4(0, 0, 0, 0);
-        __syncthreads();
+        march_sync<GT, GROUPS>();
 
         float acc[3] = {0.f, 0.f, 0.f};
         // this column's spins of the next plane, and its node's velocity and new displacement in
@@ -354,13 +378,16 @@ __global__ void __launch_bounds__(MPM_THREADS, 2) k_mpm_step(MpmArgs<float> a) {
                 for (int d = 0; d < 3; ++d) vold[d] = vp[d];
             }
             const bool more = kk + 1 < kend;
-            if (more) pl.fetch(a.u_in, R.blk_off, kk + 2, nbz, plane);
+            if (more) pl.fetch(a.u_in, node0, kk + 2, nbz, plane);
+            float uc[3] = {0.f, 0.f, 0.f};   // the owned node's u/32: corner 0 of this thread's cell
             if (need) {
                 float u[8][3];
                 const Vec4 *n0 = sm.us[b0] + nd, *n1 = sm.us[b1] + nd;
 #pragma unroll
                 for (int c = 0; c < 8; ++c) take(u[c], (c & 4 ? n1 : n0)[(c & 1) + (c & 2 ? P : 0)]);
                 float f[8][3];
+#pragma unroll
+                for (int d = 0; d < 3; ++d) uc[d] = u[0][d];
                 cell_forces<STAB>(u, sp, cw, cub, eb, f);
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
@@ -369,16 +396,14 @@ __global__ void __launch_bounds__(MPM_THREADS, 2) k_mpm_step(MpmArgs<float> a) {
                 }
             }
             if (more) pl.store(sm.us[b2]);   // buffer b2 was last read before the previous barrier
-            __syncthreads();
+            march_sync<GT, GROUPS>();
             if (own) {
                 // cells (lci-1, lcj-1), (lci, lcj-1), (lci-1, lcj), (lci, lcj) see this node as corner 3, 2, 1, 0
                 if (kk >= k0) {
                     const Vec4 c3 = sm.fb[3][tid - W - 1], c2 = sm.fb[2][tid - W];
                     const Vec4 c1 = sm.fb[1][tid - 1], c0 = sm.fb[0][tid];
-                    const Vec4 un = sm.us[b0][nd];
                     const float F[3] = {acc[0] + c3.x + c2.x + c1.x + c0.x, acc[1] + c3.y + c2.y + c1.y + c0.y,
                                         acc[2] + c3.z + c2.z + c1.z + c0.z};
-                    const float uc[3] = {un.x, un.y, un.z};
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
                         const float vn = rfma(fscale, F[d], rmul(a.keep, vold[d]));
@@ -394,7 +419,7 @@ __global__ void __launch_bounds__(MPM_THREADS, 2) k_mpm_step(MpmArgs<float> a) {
                 acc[1] = c3.y + c2.y + c1.y + c0.y;
                 acc[2] = c3.z + c2.z + c1.z + c0.z;
             }
-            __syncthreads();
+            march_sync<GT, GROUPS>();
             const int t = b0;
             b0 = b1;
             b1 = b2;
@@ -485,24 +510,34 @@ struct Form {
     int threads;
     size_t smem;
 };
+template <int GT, int GROUPS, bool STAB, int PITCH>
+Form march(size_t table) {
+    return Form{k_mpm_step<GT, GROUPS, STAB, PITCH>, GT * GROUPS, GROUPS * sizeof(MarchSmem<GT>) + (STAB ? table : 0)};
+}
+template <int THREADS, bool STAB>
+Form block(size_t table) {
+    return Form{k_mpm_block<THREADS, STAB>, THREADS, sizeof(BlockSmem<THREADS>) + (STAB ? table : 0)};
+}
 Form form_of(int variant, int nq) {
+    constexpr int T = MPM_THREADS, H = MPM_HALF_THREADS, S = MPM_SMALL_BLOCK;
     const size_t table = sizeof(float) * 12 * (size_t)nq;
-    if (!mpm_is_block(variant))
-        return nq <= MPM_STAB_MAX ? Form{variant == 0 ? k_mpm_step<true, 17> : k_mpm_step<true, 0>, MPM_THREADS,
-                                         sizeof(MarchSmem) + table}
-                                  : Form{k_mpm_step<false, 0>, MPM_THREADS, sizeof(MarchSmem)};
-    const bool st = nq <= MPM_STAB_BLOCK;   // a block stages the table only while it is small beside its loads
-    if (variant == MPM_BLOCK)
-        return Form{st ? k_mpm_block<MPM_THREADS, true> : k_mpm_block<MPM_THREADS, false>, MPM_THREADS,
-                    sizeof(BlockSmem<MPM_THREADS>) + (st ? table : 0)};
-    return Form{st ? k_mpm_block<MPM_SMALL_BLOCK, true> : k_mpm_block<MPM_SMALL_BLOCK, false>, MPM_SMALL_BLOCK,
-                sizeof(BlockSmem<MPM_SMALL_BLOCK>) + (st ? table : 0)};
+    const bool st = nq <= MPM_STAB_MAX;
+    const bool stb = nq <= MPM_STAB_BLOCK;   // a block stages the table only while it is small beside its loads
+    switch (variant) {
+        case 0: return st ? march<T, 1, true, 17>(table) : march<T, 1, false, 0>(0);
+        case MPM_BLOCK: return stb ? block<T, true>(table) : block<T, false>(0);
+        case MPM_BLOCK + 1: return stb ? block<S, true>(table) : block<S, false>(0);
+        case MPM_QUAD: return st ? march<H, 4, true, 17>(table) : march<H, 4, false, 17>(0);
+        case MPM_HALF + 1: return st ? march<H, 1, true, 17>(table) : march<H, 1, false, 0>(0);
+        case MPM_HALF + 2: return st ? march<H, 1, true, 0>(table) : march<H, 1, false, 0>(0);
+        default: return st ? march<T, 1, true, 0>(table) : march<T, 1, false, 0>(0);
+    }
 }
 
 }  // namespace
 
 cudaError_t mpm_prepare() {
-    for (int v : {0, 1, (int)MPM_BLOCK, MPM_BLOCK + 1})
+    for (int v = 0; v < mpm_nvariants(true); ++v)
         for (int nq : {MPM_STAB_BLOCK, MPM_STAB_MAX, MPM_STAB_MAX + 1}) {
             const Form f = form_of(v, nq);
             const cudaError_t e = cudaFuncSetAttribute(f.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem);
@@ -516,7 +551,7 @@ int mpm_per_sm<float>(int variant, int nq) {
     const Form f = form_of(variant, nq);
     int n = 1;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f.kernel, f.threads, f.smem);
-    return (e != cudaSuccess || n < 1) ? 1 : n;
+    return mpm_groups(variant) * ((e != cudaSuccess || n < 1) ? 1 : n);
 }
 
 // launched with programmatic stream serialisation: the kernel waits for the grid before it

@@ -392,7 +392,8 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
         const bool need = tid < W * H;
         const bool own = need && lci >= 1 && lcj >= 1;
         const int plane = nbx * nby;
-        const long long col = R.blk_off + wrapi(i0 - 1 + lci, nbx) + nbx * wrapi(j0 - 1 + lcj, nby);
+        const long long node0 = R.blk_off;   // not read again in every plane: 1 % from 100^3 on
+        const long long col = node0 + wrapi(i0 - 1 + lci, nbx) + nbx * wrapi(j0 - 1 + lcj, nby);
         const int nd = lci + P * lcj;
         int ncol[PER];   // the patch's nodes that this thread loads, as (i + nbx j) in a node plane, -1 beyond it
 #pragma unroll
@@ -403,7 +404,7 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
         double pl[PER][3];
         auto fetch = [&](int k) {   // node plane k, -1 <= k <= nbz (periodic in z)
             const int gk = k < 0 ? k + nbz : (k >= nbz ? k - nbz : k);
-            const double *base = a.u_in + 3 * (R.blk_off + (long long)plane * gk);
+            const double *base = a.u_in + 3 * (node0 + (long long)plane * gk);
 #pragma unroll
             for (int m = 0; m < PER; ++m)
                 if (ncol[m] >= 0)
