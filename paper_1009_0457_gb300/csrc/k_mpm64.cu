@@ -371,7 +371,6 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
     const int tid = threadIdx.x;
     const FxUpdate<SCALED> update(a);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     long long w = a.cuts[blockIdx.x];
     const long long wend = a.cuts[blockIdx.x + 1];
     int r = 0;
@@ -417,6 +416,9 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
                 if (ncol[m] >= 0) fx_put(sm.uxy[b], sm.uze[b], tid + m * MPM_THREADS, pl[m]);
         };
         int b0 = 0, b1 = 1, b2 = 2, fb = 0;
+        // nothing above reads what the kernels before this one write: 1.2 us a step against a wait ahead
+        // of the range's look-ups
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         fetch(k0 - 1);
         store(b0);
         fetch(k0);
