@@ -425,7 +425,7 @@ cudaError_t enqueue_mcs(hmc_handle *h, cudaStream_t s) {
     if ((e = enq_stress(h, sweeps_read_stress(h), s)) != cudaSuccess) return e;
     if ((e = enq_sweep(h, 0, s)) != cudaSuccess) return e;
     if ((e = enq_sweep(h, 1, s)) != cudaSuccess) return e;
-    return hmc::launch_end_mcs(h->d_reps, h->R, h->max_ncta, h->partials, h->nctas, 1, 1, s);
+    return hmc::launch_end_mcs(h->d_reps, h->R, h->max_ncta, h->partials, h->nctas, 1, 1, 1, s);
 }
 
 cudaError_t reset_accepted(hmc_handle *h) {
@@ -1503,7 +1503,7 @@ hmc_status hmc_compute_stress(hmc_handle *h, double *mean, double *energy) {
         ++h->state_version;
     }
     HMC_CK(h, enq_stress(h, true, h->stream), "stress launch");
-    HMC_CK(h, hmc::launch_end_mcs(h->d_reps, h->R, h->max_ncta, h->partials, h->nctas, 0, 0, h->stream), "reduction launch");
+    HMC_CK(h, hmc::launch_end_mcs(h->d_reps, h->R, h->max_ncta, h->partials, h->nctas, 0, 0, 0, h->stream), "reduction launch");
     if (mean || energy) return read_stats(h, mean, energy);
     return HMC_OK;
 }
@@ -1621,7 +1621,7 @@ hmc_status hmc_end_mcs(hmc_handle *h) {
     if (h) ++h->state_version;
     hmc_status s = need_oriented(h);
     if (s != HMC_OK) return s;
-    HMC_CK(h, hmc::launch_end_mcs(h->d_reps, h->R, h->max_ncta, h->partials, h->nctas, 1, 1, h->stream), "end-of-step launch");
+    HMC_CK(h, hmc::launch_end_mcs(h->d_reps, h->R, h->max_ncta, h->partials, h->nctas, 1, 1, 0, h->stream), "end-of-step launch");
     return HMC_OK;
 }
 

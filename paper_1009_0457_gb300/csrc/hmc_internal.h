@@ -283,7 +283,7 @@ constexpr int END_GROUPS = 32;
 __host__ __device__ constexpr int end_groups(int ncta) { return ncta <= 512 ? 1 : ncta >= 256 * END_GROUPS ? END_GROUPS : (ncta + 255) / 256; }
 inline size_t end_scratch_doubles(int nrep) { return (size_t)nrep * END_GROUPS * 7 + (size_t)(nrep + 1) / 2; }
 cudaError_t launch_end_mcs(const Replica *reps, int nrep, int max_ncta, double *partials, int nctas, int update_strain,
-                           int advance, cudaStream_t s);   // max_ncta: of the largest replica
+                           int advance, int after_sweeps, cudaStream_t s);   // max_ncta: of the largest replica
 cudaError_t launch_check_spins(const uint16_t *nat, long long n, int nq, DevState *st, cudaStream_t s);
 cudaError_t launch_pack_spins(const uint16_t *nat, uint4 *blk, int nx, int ny, int nz, cudaStream_t s);
 cudaError_t launch_unpack_spins(const uint4 *blk, uint16_t *nat, int nx, int ny, int nz, cudaStream_t s);

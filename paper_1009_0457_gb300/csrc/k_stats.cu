@@ -107,14 +107,13 @@ __global__ void __launch_bounds__(WIDE ? BLOCK_THREADS : STRESS_THREADS, sizeof(
     __shared__ double red[STRESS_THREADS / 32][7];
     __shared__ T cells[WIDE ? BLOCK_THREADS : 1][7];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int rep = __ldg(a.cta_rep + blockIdx.x);
     const Replica &R = a.reps[rep];
     const int t0 = (blockIdx.x - R.cta_off) * BLOCK_THREADS;
     Acc7<T> acc;
     acc.zero();
     T eb[6];
-    load_ebar<T>(R.st, eb);
+    load_ebar<T>(R.st, eb);   // written only by the end of a step, which lets no kernel start early
     const int nbx = R.nbx, nby = R.nby, nbz = R.nbz;
     const T *u = a.u + 3 * R.blk_off;
     T *sig = a.sig + 48ll * R.blk_off;
@@ -140,6 +139,7 @@ __global__ void __launch_bounds__(WIDE ? BLOCK_THREADS : STRESS_THREADS, sizeof(
     T un[8][3];
     uint4 spn = make_uint4(0, 0, 0, 0);
     int blk = t0 + threadIdx.x;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (blk < R.nblk) load_cell(blk, un, spn);
 #pragma unroll 1
     for (int c8 = 0; c8 < (WIDE ? 1 : STRESS_CELLS); ++c8) {
@@ -228,16 +228,18 @@ __device__ __forceinline__ double lanes_sum(double x) {
 // the FP64 pipe takes 64 cycles however many lanes it serves, so what counts is the length of the
 // chain: 20 instead of about 150 of them (the 250-thread tree and the update by one thread took
 // 15 us; 4 us).
+// after_sweeps: the kernel before this one is the black half sweep, which lets this one start only
+// when the stress pass has finished: all but the results' stores runs beside it.  This kernel lets
+// none start early, so that the step counter and the mean strain may be read before waiting.
 __global__ void __launch_bounds__(224) k_end_mcs(const Replica *reps, int nrep, int gmax, double *partials, int nctas,
-                                                  int update_strain, int advance) {
+                                                  int update_strain, int advance, int after_sweeps) {
     __shared__ double tot[7];
     __shared__ int last;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = blockIdx.x / gmax, grp = blockIdx.x % gmax;
     const Replica &R = reps[r];
     const int G = end_groups(R.ncta);
     const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;   // quantity
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!after_sweeps) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (grp >= G) return;
     DevState *st = R.st;
     double *gsum = partials + 7ll * nctas + 7ll * END_GROUPS * r;   // this replica's group sums
@@ -282,15 +284,8 @@ __global__ void __launch_bounds__(224) k_end_mcs(const Replica *reps, int nrep, 
     const double n_sites = 8.0 * (double)R.nblk;
     const double mean = tot[c] / n_sites, energy = tot[6];
     const bool bad = __any_sync(0xffffffffu, !isfinite(mean) || !isfinite(energy));
-    if (comp) st->mean_sigma[lane] = mean;
-    if (lane == 0) {
-        st->energy = energy;
-        if (bad) st->nonfinite = 1;
-        if (advance) st->mcs += 1;
-        *arrive = 0u;   // ready for the next launch
-    }
-    if (!update_strain || bad) return;
-    if (st->bc == 0) {
+    const int bc = update_strain && !bad ? st->bc : -1;
+    if (bc == 0) {
         // remove the lateral mean stress with the Reuss compliance, then restore
         // the axial strain along the uniaxial-stress direction S_R (n(x)n)
         const double nsn = lanes_sum(comp ? axNs * mean : 0.0);
@@ -301,19 +296,28 @@ __global__ void __launch_bounds__(224) k_end_mcs(const Replica *reps, int nrep, 
         const double e = ebar - d;
         const double beta = (eps0 - lanes_sum(comp ? axN * e : 0.0)) / axNB;
         ebar = e + beta * axB;
-    } else if (st->bc == 2) {
+    } else if (bc == 2) {
         // stress control: Ebar += S_R (sig0 n(x)n - <sigma>)
         const double q = sig0 * axN - mean;
         double d = 0.0;
 #pragma unroll
         for (int j = 0; j < 6; ++j) d += sr[j] * __shfl_sync(0xffffffffu, q, j);
         ebar += d;
-    } else {
-        return;
     }
+    // the black half sweep reads the step counter and the mean strain
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (comp) {
-        st->ebar[lane] = ebar;
-        st->ebar_f[lane] = (float)ebar;
+        st->mean_sigma[lane] = mean;
+        if (bc == 0 || bc == 2) {
+            st->ebar[lane] = ebar;
+            st->ebar_f[lane] = (float)ebar;
+        }
+    }
+    if (lane == 0) {
+        st->energy = energy;
+        if (bad) st->nonfinite = 1;
+        if (advance) st->mcs += 1;
+        *arrive = 0u;   // ready for the next launch
     }
 }
 
@@ -428,10 +432,10 @@ template cudaError_t launch_stress<float>(const StressArgs<float> &, bool, cudaS
 template cudaError_t launch_stress<double>(const StressArgs<double> &, bool, cudaStream_t);
 
 cudaError_t launch_end_mcs(const Replica *reps, int nrep, int max_ncta, double *partials, int nctas, int update_strain,
-                           int advance, cudaStream_t s) {
+                           int advance, int after_sweeps, cudaStream_t s) {
     const int gmax = end_groups(max_ncta);
     return launch_pdl(k_end_mcs, (unsigned)(nrep * gmax), 224u, 0, s, reps, nrep, gmax, partials, nctas, update_strain,
-                      advance);
+                      advance, after_sweeps);
 }
 
 static int grid_for(long long n) {

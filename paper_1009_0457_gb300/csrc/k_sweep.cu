@@ -355,9 +355,9 @@ __global__ void __launch_bounds__(CTA, flat_min_ctas<T, MODE, RECOMP, CTA>())
     constexpr bool STORED = ELASTIC && !RECOMP;                               // ... from the stored stress
     constexpr bool LIST = MODE == SWEEP_ZONE_LIST;
     extern __shared__ __align__(128) unsigned char sweep_smem[];
-    // the next kernel may be scheduled; everything below waits for the kernels before this one
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // The next kernel may be scheduled: after the red half sweep now, after the black one when it has
+    // waited, since the end of the step reads the stress pass's sums without waiting again.
+    if (COL == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     FlatSmem<T, STORED, CTA> &fs = *reinterpret_cast<FlatSmem<T, STORED, CTA> *>(sweep_smem);
     auto &sl = fs.list;
     // the red half sweep follows the stress pass: its CTAs take the tiles in reverse order, so
@@ -370,6 +370,17 @@ __global__ void __launch_bounds__(CTA, flat_min_ctas<T, MODE, RECOMP, CTA>())
     const int t0 = (tile - R.cta_off) * BLOCK_THREADS + (bid % SPLIT) * CTA;
     if (t0 >= R.nblk) return;  // the empty part of a replica's last tile
     const int blk = t0 + tid;  // block within the replica
+    const bool live = blk < R.nblk;
+    // What the kernel before this one does not write comes first: the block's place and its random
+    // numbers (the step counter is advanced only by the end of a step, which lets no kernel start early)
+    int bx = 0, by = 0, bz = 0;
+    uint2 rnd[4];
+    if (live) {
+        block_xyz(R, blk, bx, by, bz);
+        block_draws<COL, ONE>(R, a.rkey, a.trial, bx, by, bz, R.st->mcs, rnd);
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (COL == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (ELASTIC) {
         if (tid == 0) {
             sl.nacc = 0;
@@ -396,13 +407,9 @@ __global__ void __launch_bounds__(CTA, flat_min_ctas<T, MODE, RECOMP, CTA>())
     uint16_t out[4] = {0, 0, 0, 0}, qn[4] = {0, 0, 0, 0};
     uint32_t pend = 0;   // elastic modes: slots with a listed trial
     T sg[6][4];          // recompute mode: strain of the colour's four sites
-    uint2 rnd[4];
     int dE[4] = {0, 0, 0, 0};
-    const bool live = blk < R.nblk;
     if (live) {
         const int nbx = R.nbx, nby = R.nby, nbz = R.nbz;
-        int bx, by, bz;
-        block_xyz(R, blk, bx, by, bz);
         const int sxy = nbx, sxz = nbx * nby;
         const uint4 *spins = a.spins + R.blk_off;
         const uint2 *q2 = reinterpret_cast<const uint2 *>(spins);
@@ -417,7 +424,6 @@ __global__ void __launch_bounds__(CTA, flat_min_ctas<T, MODE, RECOMP, CTA>())
         N[3] = __ldg(q2 + 2 * (blk + (by == nby - 1 ? -(nby - 1) * sxy : sxy)) + oc);
         N[4] = __ldg(q2 + 2 * (blk + (bz == 0 ? (nbz - 1) * sxz : -sxz)) + oc);
         N[5] = __ldg(q2 + 2 * (blk + (bz == nbz - 1 ? -(nbz - 1) * sxz : sxz)) + oc);
-        block_draws<COL, ONE>(R, a.rkey, a.trial, bx, by, bz, R.st->mcs, rnd);
         uint16_t q[4];
         block_trials<COL>(a.trial, a.nq, mine, O, N, rnd, q, qn, dE);
         // recompute mode: the cell's displacement gradients, formed at the first listed trial
