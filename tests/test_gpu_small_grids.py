@@ -1,7 +1,8 @@
 """The forms that small grids take: the stress pass with one block per thread gives the bits of the
 other form (a batch large enough for the other form equals the solo runs), the end-of-step
 reduction with one and with several CTAs per replica agrees with the oracle's means, and the
-grain count by block labels equals a flood fill on grids two blocks wide and on checkered ones."""
+grain count by block labels equals a flood fill on grids two blocks wide and on checkered ones;
+steps run several to a graph equal single steps."""
 import numpy as np
 import pytest
 
@@ -70,3 +71,21 @@ def test_grain_count_by_block_labels(G, shape, Q, kind):
     n = g.grain_count()
     g.close()
     assert n == O.grain_count(sp)
+
+
+# steps of at most eight launches run in graphs of eight steps, the rest of them one by one: equal to
+# single steps for counts around the multiples, with an even and an odd number of MPM steps
+@pytest.mark.parametrize("mpm", [0, 1, 3, 4, 5])
+def test_many_steps_equal_single_steps(G, mpm):
+    shape, Q = (12, 14, 10), 9
+    eul, sp = S.euler_uniform_so3(Q, 2), S.voronoi_spins(shape, 40, Q, 3)
+    out = []
+    for counts in ([1] * 35, [7, 8, 19, 1], [35]):
+        g = G.HMC(shape, Q, precision=1, strain=2e-3, mpm_steps_per_mcs=mpm, seed=5, **C3)
+        g.set_orientations(eul, sp)
+        acc = sum(g.mc_sweeps(n) for n in counts)
+        out.append((acc, g.spins(), g.strain(), *g.nodal()))
+        g.close()
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            assert np.array_equal(a, b)
