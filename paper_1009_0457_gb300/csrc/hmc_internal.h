@@ -285,7 +285,8 @@ inline size_t end_scratch_doubles(int nrep) { return (size_t)nrep * END_GROUPS *
 cudaError_t launch_end_mcs(const Replica *reps, int nrep, int max_ncta, double *partials, int nctas, int update_strain,
                            int advance, int after_sweeps, cudaStream_t s);   // max_ncta: of the largest replica
 cudaError_t launch_check_spins(const uint16_t *nat, long long n, int nq, DevState *st, cudaStream_t s);
-cudaError_t launch_pack_spins(const uint16_t *nat, uint4 *blk, int nx, int ny, int nz, cudaStream_t s);
+cudaError_t launch_pack_spins(const uint16_t *nat, uint4 *blk, int nx, int ny, int nz, const int32_t *bad,
+                              cudaStream_t s);
 cudaError_t launch_unpack_spins(const uint4 *blk, uint16_t *nat, int nx, int ny, int nz, cudaStream_t s);
 cudaError_t launch_bonds_counts(const uint4 *blk, int nbx, int nby, int nbz, int nq,
                                 unsigned long long *counts, DevState *st, cudaStream_t s);

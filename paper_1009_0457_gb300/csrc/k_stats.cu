@@ -334,8 +334,10 @@ __global__ void k_check_spins(const uint16_t *__restrict__ nat, long long n, int
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&st->bad_spin, 1);
 }
 
-// natural uint16 field <-> 2x2x2 blocks in slot order
-__global__ void k_pack_spins(const uint16_t *__restrict__ nat, uint4 *__restrict__ blk, int nx, int ny, int nz) {
+// natural uint16 field <-> 2x2x2 blocks in slot order; a field that the check flagged stays out
+__global__ void k_pack_spins(const uint16_t *__restrict__ nat, uint4 *__restrict__ blk, int nx, int ny, int nz,
+                             const int32_t *bad) {
+    if (*bad) return;
     const int nbx = nx >> 1, nby = ny >> 1, nbz = nz >> 1;
     const long long nblk = (long long)nbx * nby * nbz;
     for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x; b < nblk; b += (long long)gridDim.x * blockDim.x) {
@@ -450,9 +452,10 @@ cudaError_t launch_check_spins(const uint16_t *nat, long long n, int nq, DevStat
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_spins(const uint16_t *nat, uint4 *blk, int nx, int ny, int nz, cudaStream_t s) {
+cudaError_t launch_pack_spins(const uint16_t *nat, uint4 *blk, int nx, int ny, int nz, const int32_t *bad,
+                              cudaStream_t s) {
     const long long nblk = (long long)(nx / 2) * (ny / 2) * (nz / 2);
-    k_pack_spins<<<grid_for(nblk), 256, 0, s>>>(nat, blk, nx, ny, nz);
+    k_pack_spins<<<grid_for(nblk), 256, 0, s>>>(nat, blk, nx, ny, nz, bad);
     return cudaGetLastError();
 }
 
