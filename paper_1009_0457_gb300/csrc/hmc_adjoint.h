@@ -17,9 +17,17 @@ struct AdjArgs {
     int nx, ny, nz, nbx, nby, nbz, nblk;
 };
 
-// adds the sums of P, T and D (times 2^10) to the partials and lam to the sum of the lambdas
+// Reverse steps that one parameter launch takes.  Their lambdas are kept in the buffer of the cell
+// contributions, which the reverse sweep does not need: 24 values a cell, the size of eight.
+constexpr int ADJ_BATCH = 8;
 template <typename T>
-cudaError_t launch_adj_params(const AdjArgs<T> &a, const T *lam, const T *u, T *lsum, T *lerr, cudaStream_t s);
+struct AdjSteps {
+    const T *lam[ADJ_BATCH], *u[ADJ_BATCH];
+    int n;
+};
+// adds the sums of P, T and D (times 2^10) to the partials and the lambdas to their sum
+template <typename T>
+cudaError_t launch_adj_params(const AdjArgs<T> &a, const AdjSteps<T> &st, T *lsum, T *lerr, cudaStream_t s);
 template <typename T>
 cudaError_t launch_adj_mean(const AdjArgs<T> &a, const T *lsum, const T *lerr, cudaStream_t s);
 template <typename T>

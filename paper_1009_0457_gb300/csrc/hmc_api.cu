@@ -119,7 +119,7 @@ struct hmc_handle {
         bool have_forward = false;
         long long state_version = -1;
         int rtab_version = -1;
-        void *rtab = nullptr, *lam = nullptr, *ubar = nullptr, *tmp = nullptr, *vtmp = nullptr, *seg = nullptr;
+        void *rtab = nullptr, *lam = nullptr, *ubar = nullptr, *vtmp = nullptr, *seg = nullptr;
         void *ck_u = nullptr, *ck_v = nullptr, *w = nullptr, *g = nullptr, *fcell = nullptr;
         void *lsum = nullptr, *lerr = nullptr;   // sum of the reverse steps' lambdas (FP32: with its error)
         int seg_held = -1;                       // segment whose states `seg` holds
@@ -540,12 +540,12 @@ std::string validate_shared(const hmc_params *a, const hmc_params *b) {
 }
 
 void free_adjoint(hmc_handle *h) {
-    void *bufs[] = {h->adj.rtab, h->adj.lam, h->adj.ubar, h->adj.tmp, h->adj.vtmp, h->adj.seg, h->adj.ck_u,
+    void *bufs[] = {h->adj.rtab, h->adj.lam, h->adj.ubar, h->adj.vtmp, h->adj.seg, h->adj.ck_u,
                     h->adj.ck_v, h->adj.w, h->adj.g, h->adj.fcell, h->adj.partials, h->adj.grad, h->adj.reps0,
                     h->adj.st0, h->adj.lsum, h->adj.lerr};
     for (void *b : bufs)
         if (b) cudaFree(b);
-    h->adj.rtab = h->adj.lam = h->adj.ubar = h->adj.tmp = h->adj.vtmp = h->adj.seg = nullptr;
+    h->adj.rtab = h->adj.lam = h->adj.ubar = h->adj.vtmp = h->adj.seg = nullptr;
     h->adj.ck_u = h->adj.ck_v = h->adj.w = h->adj.g = h->adj.fcell = nullptr;
     h->adj.partials = h->adj.grad = nullptr;
     h->adj.lsum = h->adj.lerr = nullptr;
@@ -2031,7 +2031,7 @@ hmc_status adj_alloc(hmc_handle *h, int steps, int ck) {
     struct Alloc { void **ptr; size_t bytes; const char *what; };
     Alloc allocs[] = {
         {&A.rtab, h->tsize * 72 * (size_t)h->p.n_orient, "basis tables"},
-        {&A.lam, nb, "adjoint lambda"}, {&A.ubar, nb, "adjoint u"}, {&A.tmp, nb, "adjoint scratch"},
+        {&A.lam, nb, "adjoint lambda"}, {&A.ubar, nb, "adjoint u"},
         {&A.vtmp, nb, "segment velocity"}, {&A.seg, nb * (size_t)ck, "segment states"},
         {&A.ck_u, nb * (size_t)nseg, "checkpoints u"}, {&A.ck_v, nb * (size_t)nseg, "checkpoints v"},
         {&A.w, h->tsize * (size_t)R.N, "field w"}, {&A.g, h->tsize * (size_t)R.N, "cotangent field"},
@@ -2138,7 +2138,9 @@ hmc_status adj_backward_t(hmc_handle *h, double gW, const double *g_field, doubl
     HMC_CK(h, cudaMemsetAsync(A.partials, 0, sizeof(double) * 3 * (size_t)A.nctas, h->stream), "memset");
     HMC_CK(h, cudaMemsetAsync(A.lsum, 0, nb, h->stream), "memset");
     if (A.lerr) HMC_CK(h, cudaMemsetAsync(A.lerr, 0, nb, h->stream), "memset");
-    void *lam = A.lam, *lam_next = A.tmp;
+    // lambda's states: A.lam and the eight arrays of A.fcell (read for the last time above), in turn
+    auto lam_at = [&](int k) -> void * { return k == 0 ? A.lam : seg_ptr(h, A.fcell, k - 1); };
+    int at = 0;
     for (int s = A.nseg - 1; s >= 0; --s) {
         const int n0 = s * A.ck, len = std::min(A.ck, A.steps - n0);
         // the segment's forward states u^{n0} .. u^{n0+len-1}: recomputed from its checkpoint, unless the
@@ -2155,14 +2157,23 @@ hmc_status adj_backward_t(hmc_handle *h, double gW, const double *g_field, doubl
                        "recompute launch");
             A.seg_held = s;
         }
-        for (int j = len - 1; j >= 0; --j) {
-            HMC_CK(h, hmc::launch_adj_params<T>(aa, static_cast<const T *>(lam),
-                                                reinterpret_cast<const T *>(seg_ptr(h, A.seg, j)),
-                                                static_cast<T *>(A.lsum), static_cast<T *>(A.lerr), h->stream),
+        // even batches: at most ADJ_BATCH steps of lambda, then their parameter terms
+        const int nbatch = (len + hmc::ADJ_BATCH - 1) / hmc::ADJ_BATCH;
+        for (int b = nbatch - 1; b >= 0; --b) {
+            const int lo = (int)((long long)len * b / nbatch), hi = (int)((long long)len * (b + 1) / nbatch);
+            hmc::AdjSteps<T> st;
+            st.n = 0;
+            for (int j = hi - 1; j >= lo; --j) {
+                const int next = (at + 1) % (hmc::ADJ_BATCH + 1);
+                st.lam[st.n] = static_cast<const T *>(lam_at(at));
+                st.u[st.n++] = reinterpret_cast<const T *>(seg_ptr(h, A.seg, j));
+                // ubar^n = ubar^{n+1} + c F(lambda^{n+1}; 0); lambda^n = (1 - damping) lambda^{n+1} + dt ubar^n
+                HMC_CK(h, mpm_custom<T>(h, lam_at(at), lam_at(next), A.ubar, A.reps0, 1.0, 1.0 - h->damping),
+                       "adjoint step launch");
+                at = next;
+            }
+            HMC_CK(h, hmc::launch_adj_params<T>(aa, st, static_cast<T *>(A.lsum), static_cast<T *>(A.lerr), h->stream),
                    "parameter launch");
-            // ubar^n = ubar^{n+1} + c F(lambda^{n+1}; 0); lambda^n = (1 - damping) lambda^{n+1} + dt ubar^n
-            HMC_CK(h, mpm_custom<T>(h, lam, lam_next, A.ubar, A.reps0, 1.0, 1.0 - h->damping), "adjoint step launch");
-            std::swap(lam, lam_next);
         }
     }
     // the sums of P, T and D of every step, then the terms linear in lambda

@@ -217,18 +217,21 @@ __device__ __forceinline__ void load_axes(const T *p, T (&w)[12]) {
         for (int k = 3; k < 6; ++k) w[6 * m + k] *= T(0.5);
 }
 
-// One reverse step's parameter terms.  With eps = Ebar + B u, everything that is linear in
+// The parameter terms of st.n reverse steps.  With eps = Ebar + B u, everything that is linear in
 // lambda alone -- the forms against Ebar and the mean of C' epsbar -- is left to one pass over
 // the sum of the lambdas (k_adj_mean); what is left per step are the three forms of B lambda
 // and B u, and these are combinations of P = sum_m p_m p_m, T = tr tr and D = x:y (basis_forms),
 // so the sums of P, T and D are kept (times 2^10, from gradients times 32).  The third axis'
-// projection is the trace minus the other two.  Each thread also adds its node's lambda to the sum
-// (TwoSum pairs in FP32).  About 640 operations a cell where the full terms took 1530, and 12
-// table values per orientation change instead of 42: 40 -> 20 us per step at 128^3.
+// projection is the trace minus the other two.  Each thread also adds its node's lambdas to the sum
+// (TwoSum pairs in FP32).  About 640 operations a cell and step where the full terms took 1530,
+// and 12 table values per orientation change instead of 42.
+// What bounds it: the latency of a cell's loads, with 16 warps per SM at 128 registers.  One step to
+// a launch (20 us and a gap of 3 at 128^3) also paid the reduction over the CTA, the node's sum and
+// the table's rows every step; with ADJ_BATCH steps of a cell in one thread a step takes 11 us.  In
+// FP64 (bound by its pipe) the batch is 7 % faster over a whole gradient, spills of 480 B included.
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_adj_params(AdjArgs<T> a, const T *__restrict__ lam,
-                                                    const T *__restrict__ u, T *__restrict__ lsum,
-                                                    T *__restrict__ lerr) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_adj_params(AdjArgs<T> a, AdjSteps<T> st,
+                                                    T *__restrict__ lsum, T *__restrict__ lerr) {
     AdjAcc<T, 3> acc;
     acc.zero();
     const int blk = blockIdx.x * blockDim.x + threadIdx.x;
@@ -236,68 +239,75 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_adj_params(AdjA
         const int bx = blk % a.nbx, r = blk / a.nbx;
         const int by = r % a.nby, bz = r / a.nby;
         const uint4 sp = __ldg(a.spins + blk);
-        CellGrad<T> gl, gu;
-        {
-            T cl[8][3];
-            load_corners<T>(lam, bx, by, bz, a.nbx, a.nby, a.nbz, cl);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {   // corner 0 is node blk
-                const long long i = 3ll * blk + d;
-                if constexpr (sizeof(T) == 4) {
-                    TwoSumF s{lsum[i], lerr[i]};
-                    s.add(cl[0][d]);
-                    lsum[i] = s.hi;
-                    lerr[i] = s.lo;
-                } else {
-                    lsum[i] += cl[0][d];
-                }
-            }
-            cell_gradients32<T>(cl, gl);
-        }
-        {
-            T cu[8][3];
-            load_corners<T>(u, bx, by, bz, a.nbx, a.nby, a.nbz, cu);
-            cell_gradients32<T>(cu, gu);
-        }
-        T P = T(0), TT = T(0), D = T(0), Dh = T(0);   // D's shear terms count half
+        AdjAcc<T, 3> node;   // the sum of the lambdas at corner 0, node blk
+        node.zero();
         T w[12];
         uint32_t qprev = 0xffffffffu;
+#pragma unroll 1
+        for (int j = 0; j < st.n; ++j) {
+            CellGrad<T> gl, gu;
+            {
+                T cl[8][3];
+                load_corners<T>(st.lam[j], bx, by, bz, a.nbx, a.nby, a.nbz, cl);
 #pragma unroll
-        for (int n = 0; n < 8; ++n) {
-            const int L = n == 2 ? 3 : n == 3 ? 2 : n == 4 ? 6 : n == 5 ? 7 : n == 6 ? 5 : n == 7 ? 4 : n;   // Gray code
-            T x[6], y[6];
-            fluctuation<T>(gl, L & 1, (L >> 1) & 1, L >> 2, x);
-            fluctuation<T>(gu, L & 1, (L >> 1) & 1, L >> 2, y);
-            const uint32_t q = spin_of(sp, local_slot(L));
-            if (q != qprev) {
-                load_axes<T>(a.wtab + 20ll * q, w);
-                qprev = q;
+                for (int d = 0; d < 3; ++d) node.add(d, cl[0][d]);
+                cell_gradients32<T>(cl, gl);
             }
-            T px[2], py[2];
+            {
+                T cu[8][3];
+                load_corners<T>(st.u[j], bx, by, bz, a.nbx, a.nby, a.nbz, cu);
+                cell_gradients32<T>(cu, gu);
+            }
+            T P = T(0), TT = T(0), D = T(0), Dh = T(0);   // D's shear terms count half
 #pragma unroll
-            for (int m = 0; m < 2; ++m) {
-                px[m] = w[6 * m] * x[0];
-                py[m] = w[6 * m] * y[0];
+            for (int n = 0; n < 8; ++n) {
+                const int L = n == 2 ? 3 : n == 3 ? 2 : n == 4 ? 6 : n == 5 ? 7 : n == 6 ? 5 : n == 7 ? 4 : n;   // Gray code
+                T x[6], y[6];
+                fluctuation<T>(gl, L & 1, (L >> 1) & 1, L >> 2, x);
+                fluctuation<T>(gu, L & 1, (L >> 1) & 1, L >> 2, y);
+                const uint32_t q = spin_of(sp, local_slot(L));
+                if (q != qprev) {
+                    load_axes<T>(a.wtab + 20ll * q, w);
+                    qprev = q;
+                }
+                T px[2], py[2];
 #pragma unroll
-                for (int k = 1; k < 6; ++k) {
-                    px[m] = fma(w[6 * m + k], x[k], px[m]);
-                    py[m] = fma(w[6 * m + k], y[k], py[m]);
+                for (int m = 0; m < 2; ++m) {
+                    px[m] = w[6 * m] * x[0];
+                    py[m] = w[6 * m] * y[0];
+#pragma unroll
+                    for (int k = 1; k < 6; ++k) {
+                        px[m] = fma(w[6 * m + k], x[k], px[m]);
+                        py[m] = fma(w[6 * m + k], y[k], py[m]);
+                    }
+                }
+                const T tx = x[0] + x[1] + x[2], ty = y[0] + y[1] + y[2];
+                P = fma(px[0], py[0], P);
+                P = fma(px[1], py[1], P);
+                P = fma(tx - px[0] - px[1], ty - py[0] - py[1], P);
+                TT = fma(tx, ty, TT);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    D = fma(x[k], y[k], D);
+                    Dh = fma(x[3 + k], y[3 + k], Dh);
                 }
             }
-            const T tx = x[0] + x[1] + x[2], ty = y[0] + y[1] + y[2];
-            P = fma(px[0], py[0], P);
-            P = fma(px[1], py[1], P);
-            P = fma(tx - px[0] - px[1], ty - py[0] - py[1], P);
-            TT = fma(tx, ty, TT);
+            acc.add(0, P);
+            acc.add(1, TT);
+            acc.add(2, fma(T(0.5), Dh, D));
+        }
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                D = fma(x[k], y[k], D);
-                Dh = fma(x[3 + k], y[3 + k], Dh);
+        for (int d = 0; d < 3; ++d) {
+            const long long i = 3ll * blk + d;
+            if constexpr (sizeof(T) == 4) {
+                TwoSumF s{lsum[i], lerr[i]};
+                s.add(node.v[d].hi);
+                lsum[i] = s.hi;
+                lerr[i] = s.lo + node.v[d].lo;
+            } else {
+                lsum[i] += node.v[d];
             }
         }
-        acc.add(0, P);
-        acc.add(1, TT);
-        acc.add(2, fma(T(0.5), Dh, D));
     }
     cta_partials<T, 3>(acc, a.partials, true);
 }
@@ -471,8 +481,8 @@ __global__ void k_adj_reduce(const double *partials, int nparts, int nv, int str
 }  // namespace
 
 template <typename T>
-cudaError_t launch_adj_params(const AdjArgs<T> &a, const T *lam, const T *u, T *lsum, T *lerr, cudaStream_t s) {
-    k_adj_params<T><<<(a.nblk + 255) / 256, 256, 0, s>>>(a, lam, u, lsum, lerr);
+cudaError_t launch_adj_params(const AdjArgs<T> &a, const AdjSteps<T> &st, T *lsum, T *lerr, cudaStream_t s) {
+    k_adj_params<T><<<(a.nblk + 255) / 256, 256, 0, s>>>(a, st, lsum, lerr);
     return cudaGetLastError();
 }
 template <typename T>
@@ -497,7 +507,7 @@ cudaError_t launch_adj_reduce(const double *partials, int nparts, int nv, int st
 }
 
 #define HMC_ADJ_INST(T)                                                                                          \
-    template cudaError_t launch_adj_params<T>(const AdjArgs<T> &, const T *, const T *, T *, T *, cudaStream_t); \
+    template cudaError_t launch_adj_params<T>(const AdjArgs<T> &, const AdjSteps<T> &, T *, T *, cudaStream_t);     \
     template cudaError_t launch_adj_mean<T>(const AdjArgs<T> &, const T *, const T *, cudaStream_t);             \
     template cudaError_t launch_adj_terminal<T>(const AdjArgs<T> &, const T *, const T *, T, T *, T *,           \
                                                 cudaStream_t);                                                   \
