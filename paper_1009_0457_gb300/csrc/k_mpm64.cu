@@ -32,7 +32,7 @@
 // barrier per plane.
 // What bounds it: 244 registers leave eight warps per SM, which issue 36 % of the cycles (the
 // busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
-// 32^3 20 (70), 96x90x100 67 (288), 128^3 129 (420), 256^3 714 (3330).
+// 32^3 8.5 (70), 100^3 52 (308), 128^3 102 (420), 256^3 709 (3330).
 #include "hmc_device.cuh"
 
 namespace hmc {
@@ -195,6 +195,87 @@ __device__ __forceinline__ void fx_cell(const ll (&u)[8][3], const ll (&eb)[6], 
     }
 }
 
+// the cell of a thread: 16 cells a warp, their halves on lanes 0..15 and 16..31
+__device__ __forceinline__ int half_cell(int tid) { return (tid >> 5) * 16 + (tid & 15); }
+
+// 3 x + y
+__device__ __forceinline__ ll x3(ll x, ll y) { return (x << 1) + x + y; }
+__device__ __forceinline__ ll other_half(ll x) { return __shfl_xor_sync(0xffffffffu, x, 16); }
+
+// Half h of a cell: its four points with c = h.  u holds the corners I + 2J of the near node plane, on
+// the points' side, and I + 2J + 4 of the far one; f takes the forces (times 32, with the sign of -f)
+// on the near corners.  The cell's other half runs on the lane 16 away, all 32 lanes together.  The
+// same integers are summed and rounded as in fx_cell, so the results are the same bits.
+__device__ __forceinline__ void fx_half(const ll (&u)[8][3], const ll (&eb)[6], const uint4 &sp, int h,
+                                        const int2 *tab, ll (&f)[4][3]) {
+    FxRow row;
+    uint32_t qprev = 0xffffffffu;
+    const ll up = h ? -1 : 0;   // a sign: d/dz points from near to far for h = 0
+    ll gx[2][3], gy[2][3], gz[2][2][3];   // [b], [a], [a][b]: d u_d / dx, dy, dz at the points
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        ll m[4], z[4];   // the corners' mean over z with the points' weights; their differences in z
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            m[n] = x3(u[n][d], u[n + 4][d]);
+            z[n] = ((u[n + 4][d] - u[n][d]) ^ up) - up;
+        }
+        const ll dx[2] = {m[1] - m[0], m[3] - m[2]}, dy[2] = {m[2] - m[0], m[3] - m[1]};
+        ll o[2][2];
+        interp31<0>(z[0], z[1], z[2], z[3], o);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            gx[i][d] = x3(dx[i], dx[1 - i]) + (d == 0 ? eb[0] : 0);
+            gy[i][d] = x3(dy[i], dy[1 - i]) + (d == 1 ? eb[1] : d == 0 ? eb[5] : 0);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) gz[i][k][d] = o[i][k] + (d == 2 ? eb[2] : d == 1 ? eb[3] : eb[4]);
+        }
+    }
+    ll tx[2][3], ty[2][3], tz[2][2][3];   // this half's traction sums over a, b and c
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {   // one coordinate changes from one point to the next
+        const int a = n == 1 || n == 2, b = n >> 1;
+        ll e[6], s[6];
+        e[0] = gx[b][0];
+        e[1] = gy[a][1];
+        e[2] = gz[a][b][2];
+        e[3] = gz[a][b][1] + gy[a][2];
+        e[4] = gz[a][b][0] + gx[b][2];
+        e[5] = gy[a][0] + gx[b][1];
+        const uint32_t q = h ? spin_of(sp, local_slot(a + 2 * b + 4)) : spin_of(sp, local_slot(a + 2 * b));
+        if (q != qprev) {
+            row.load(tab, q);
+            qprev = q;
+        }
+        fx_hooke(row, e, s);
+        const ll x[3] = {s[0], s[5], s[4]}, y[3] = {s[5], s[1], s[3]}, z[3] = {s[4], s[3], s[2]};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            tx[b][d] = n == 0 || n == 2 ? x[d] : tx[b][d] + x[d];
+            ty[a][d] = n == 0 || n == 1 ? y[d] : ty[a][d] + y[d];
+            tz[a][b][d] = z[d];
+        }
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        ll X[2], Y[2], Z[2][2];   // X[J], Y[I] on the near plane, Z[I][J]
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const ll ex = x3(tx[i][d], tx[1 - i][d]) >> 3, ey = x3(ty[i][d], ty[1 - i][d]) >> 3;
+            X[i] = x3(ex, other_half(ex));
+            Y[i] = x3(ey, other_half(ey));
+#pragma unroll
+            for (int k = 0; k < 2; ++k) tz[i][k][d] += other_half(tz[i][k][d]);
+        }
+        interp31<3>(tz[0][0][d], tz[1][0][d], tz[0][1][d], tz[1][1][d], Z);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            const int I = n & 1, J = n >> 1;
+            f[n][d] = (I ? X[J] : -X[J]) + (J ? Y[I] : -Y[I]) + (((Z[I][J]) ^ ~up) - ~up);
+        }
+    }
+}
+
 // three integers with one exponent (that of the cells' displacements; 2047 = not finite)
 struct Fx3 {
     ll v[3];
@@ -278,7 +359,8 @@ __device__ __forceinline__ void fx_mean(FxMean &m, const DevState *st) {   // by
     m.e = E;
 }
 
-// a cell: its corners lie at n0 and n1 (lower and upper plane), P nodes a row; returns its exponent
+// a cell: its corners lie at n0 and n1 (lower and upper plane; for a half cell the near and the far
+// one), P nodes a row; returns its exponent
 __device__ __forceinline__ int fx_corners(const FxHalf *xy0, const FxHalf *ze0, const FxHalf *xy1, const FxHalf *ze1,
                                           int P, const FxMean &m, ll (&u)[8][3], ll (&eb)[6]) {
     int ne[8], E = m.e;
@@ -481,12 +563,17 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
     }
 }
 
-// The block form (k_mpm.cu): one block per CTA, every cell at once.
-template <int THREADS, bool SCALED>
-__global__ void __launch_bounds__(THREADS, THREADS > 128 ? 1 : 2) k_mpm_fixed_block(MpmArgs<double> a) {
+// The block form (k_mpm.cu): one block per CTA, every cell at once, on SPLIT threads each.  Blocks of
+// at most 96 cells run where there is one to an SM, three warps of whole cells: what bounds them is
+// the length of a cell's code, and halves take 8.6 us a step at 32^3 where whole cells took 11.4.
+// Blocks of 256 cells fill the registers as they are (halves at 128 registers: 24.6 -> 30.3 us at 64^3;
+// the march likewise, 102 -> 133 us at 128^3).
+template <int CELLS, int SPLIT, bool SCALED>
+__global__ void __launch_bounds__(CELLS *SPLIT, 1) k_mpm_fixed_block(MpmArgs<double> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    FxBlockSmem<THREADS> &sm = *reinterpret_cast<FxBlockSmem<THREADS> *>(smem_raw);
+    FxBlockSmem<CELLS> &sm = *reinterpret_cast<FxBlockSmem<CELLS> *>(smem_raw);
     const int tid = threadIdx.x;
+    const int cell = SPLIT == 2 ? half_cell(tid) : tid, h = SPLIT == 2 ? tid >> 4 & 1 : 0;
     const FxUpdate<SCALED> update(a);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     int r = 0;
@@ -495,16 +582,21 @@ __global__ void __launch_bounds__(THREADS, THREADS > 128 ? 1 : 2) k_mpm_fixed_bl
     const MpmSched &SC = a.sched[r];
     const BlockPlace B(SC, R, blockIdx.x - (int)SC.off);
     const int W = B.W, H = B.H, P = W + 1, PP = P * (H + 1);
-    const int lci = tid % W, lcj = tid / W % H, lck = tid / (W * H);
-    const bool need = lck < B.D;
-    const bool own = need && lci >= 1 && lcj >= 1 && lck >= 1;
-    const long long at = R.blk_off + wrapi(B.i0 - 1 + lci, R.nbx) +
-                         (long long)R.nbx * (wrapi(B.j0 - 1 + lcj, R.nby) + (long long)R.nby * wrapi(B.k0 - 1 + lck, R.nbz));
-    long long node[2];
+    auto block_at = [&](int i, int j, int k) {
+        return R.blk_off + wrapi(B.i0 - 1 + i, R.nbx) +
+               (long long)R.nbx * (wrapi(B.j0 - 1 + j, R.nby) + (long long)R.nby * wrapi(B.k0 - 1 + k, R.nbz));
+    };
+    const int cells = W * H * B.D;
+    const int ci = cell % W, cj = cell / W % H, ck = cell / (W * H);
+    const bool need = cell < cells, some = SPLIT == 2 ? (tid >> 5) * 16 < cells : need;   // (halves: the whole warp)
+    const int lci = tid % W, lcj = tid / W % H, lck = tid / (W * H);   // the first threads own nodes
+    const bool own = tid < cells && lci >= 1 && lcj >= 1 && lck >= 1;
+    const long long at = own ? block_at(lci, lcj, lck) : 0, cat = need ? block_at(ci, cj, ck) : 0;
+    long long node[2 / SPLIT];
 #pragma unroll
-    for (int m = 0; m < 2; ++m) node[m] = B.node(R, tid + m * THREADS);
+    for (int m = 0; m < 2 / SPLIT; ++m) node[m] = B.node(R, tid + m * CELLS);
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const uint4 sp = need ? __ldg(a.spins + at) : make_uint4(0, 0, 0, 0);
+    const uint4 sp = need ? __ldg(a.spins + cat) : make_uint4(0, 0, 0, 0);
     double uold[3] = {0, 0, 0}, vold[3] = {0, 0, 0};
     if (own) {
 #pragma unroll
@@ -514,23 +606,26 @@ __global__ void __launch_bounds__(THREADS, THREADS > 128 ? 1 : 2) k_mpm_fixed_bl
         }
     }
 #pragma unroll
-    for (int m = 0; m < 2; ++m)
+    for (int m = 0; m < 2 / SPLIT; ++m)
         if (node[m] >= 0) {
             const double *p = a.u_in + 3 * node[m];
             const double u[3] = {__ldg(p), __ldg(p + 1), __ldg(p + 2)};
-            fx_put(sm.uxy, sm.uze, tid + m * THREADS, u);
+            fx_put(sm.uxy, sm.uze, tid + m * CELLS, u);
         }
     if (tid == 0) fx_mean(sm.m, R.st);
     __syncthreads();
-    if (need) {
-        ll u[8][3], eb[6], f[8][3];
-        const int nd = lci + P * lcj + PP * lck;
-        const int E = fx_corners(sm.uxy + nd, sm.uze + nd, sm.uxy + nd + PP, sm.uze + nd + PP, P, sm.m, u, eb);
-        fx_cell(u, eb, sp, a.cfix, f);
+    if (some) {
+        ll u[8][3], eb[6], f[8 / SPLIT][3];
+        const int nd = need ? ci + P * cj + PP * ck : 0, n0 = nd + (h ? PP : 0), n1 = nd + (h ? 0 : PP);
+        const int E = fx_corners(sm.uxy + n0, sm.uze + n0, sm.uxy + n1, sm.uze + n1, P, sm.m, u, eb);
+        if constexpr (SPLIT == 2)
+            fx_half(u, eb, sp, h, a.cfix, f);
+        else
+            fx_cell(u, eb, sp, a.cfix, f);
 #pragma unroll
-        for (int n = 0; n < 8; ++n) {
-            sm.fxy[n][tid] = FxHalf{f[n][0], f[n][1]};
-            sm.fze[n][tid] = FxHalf{f[n][2], (ll)E};
+        for (int n = 0; n < 8 / SPLIT; ++n) {
+            sm.fxy[4 * h + n][cell] = FxHalf{f[n][0], f[n][1]};
+            sm.fze[4 * h + n][cell] = FxHalf{f[n][2], (ll)E};
         }
     }
     __syncthreads();
@@ -548,8 +643,9 @@ template <bool SCALED>
 Form form_of(int variant) {
     if (!mpm_is_block(variant)) return Form{k_mpm_fixed<SCALED>, MPM_THREADS, sizeof(FxMarchSmem)};
     if (variant == MPM_BLOCK)
-        return Form{k_mpm_fixed_block<MPM_THREADS, SCALED>, MPM_THREADS, sizeof(FxBlockSmem<MPM_THREADS>)};
-    return Form{k_mpm_fixed_block<MPM_SMALL_BLOCK, SCALED>, MPM_SMALL_BLOCK, sizeof(FxBlockSmem<MPM_SMALL_BLOCK>)};
+        return Form{k_mpm_fixed_block<MPM_THREADS, 1, SCALED>, MPM_THREADS, sizeof(FxBlockSmem<MPM_THREADS>)};
+    return Form{k_mpm_fixed_block<MPM_SMALL_BLOCK, 2, SCALED>, 2 * MPM_SMALL_BLOCK,
+                sizeof(FxBlockSmem<MPM_SMALL_BLOCK>)};
 }
 
 }  // namespace
