@@ -32,7 +32,7 @@
 // barrier per plane.
 // What bounds it: 244 registers leave eight warps per SM, which issue 36 % of the cycles (the
 // busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
-// 32^3 8.5 (70), 100^3 52 (308), 128^3 102 (420), 256^3 709 (3330).
+// 32^3 7.8 (70), 100^3 52 (308), 128^3 102 (420), 256^3 709 (3330).
 #include "hmc_device.cuh"
 
 namespace hmc {
@@ -195,83 +195,77 @@ __device__ __forceinline__ void fx_cell(const ll (&u)[8][3], const ll (&eb)[6], 
     }
 }
 
-// the cell of a thread: 16 cells a warp, their halves on lanes 0..15 and 16..31
-__device__ __forceinline__ int half_cell(int tid) { return (tid >> 5) * 16 + (tid & 15); }
-
 // 3 x + y
 __device__ __forceinline__ ll x3(ll x, ll y) { return (x << 1) + x + y; }
-__device__ __forceinline__ ll other_half(ll x) { return __shfl_xor_sync(0xffffffffu, x, 16); }
+// the value on the lane of the quarter beyond the cell's middle in y (8) or z (16)
+__device__ __forceinline__ ll across(ll x, int lane) { return __shfl_xor_sync(0xffffffffu, x, lane); }
+__device__ __forceinline__ ll flip(ll x, ll sign) { return (x ^ sign) - sign; }   // sign: 0 or -1
 
-// Half h of a cell: its four points with c = h.  u holds the corners I + 2J of the near node plane, on
-// the points' side, and I + 2J + 4 of the far one; f takes the forces (times 32, with the sign of -f)
-// on the near corners.  The cell's other half runs on the lane 16 away, all 32 lanes together.  The
-// same integers are summed and rounded as in fx_cell, so the results are the same bits.
-__device__ __forceinline__ void fx_half(const ll (&u)[8][3], const ll (&eb)[6], const uint4 &sp, int h,
-                                        const int2 *tab, ll (&f)[4][3]) {
-    FxRow row;
-    uint32_t qprev = 0xffffffffu;
-    const ll up = h ? -1 : 0;   // a sign: d/dz points from near to far for h = 0
-    ll gx[2][3], gy[2][3], gz[2][2][3];   // [b], [a], [a][b]: d u_d / dx, dy, dz at the points
+// Quarter (b, c) of a cell: its two points with that b and c, on lane 8 (b + 2c) + (cell of the warp),
+// all 32 lanes together.  u holds the corners with I = 0, 1 that are near in y and z (0, 1), far in y
+// (2, 3), far in z (4, 5) and far in both; f takes the forces (times 32, with the sign of -f) on the two
+// near corners.  The same integers are summed and rounded as in fx_cell, so the results are the same bits.
+__device__ __forceinline__ void fx_quarter(const ll (&u)[8][3], const ll (&eb)[6], const uint4 &sp, int b, int c,
+                                           const int2 *tab, ll (&f)[2][3]) {
+    const ll sb = b ? -1 : 0, sc = c ? -1 : 0;   // d/dy and d/dz point from near to far for b = 0, c = 0
+    ll gx[3], gy[2][3], gz[2][3];                // [d], [a][d]: d u_d / dx, dy, dz at the points
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         ll m[4], z[4];   // the corners' mean over z with the points' weights; their differences in z
 #pragma unroll
         for (int n = 0; n < 4; ++n) {
             m[n] = x3(u[n][d], u[n + 4][d]);
-            z[n] = ((u[n + 4][d] - u[n][d]) ^ up) - up;
+            z[n] = u[n + 4][d] - u[n][d];
         }
-        const ll dx[2] = {m[1] - m[0], m[3] - m[2]}, dy[2] = {m[2] - m[0], m[3] - m[1]};
-        ll o[2][2];
-        interp31<0>(z[0], z[1], z[2], z[3], o);
+        gx[d] = x3(m[1] - m[0], m[3] - m[2]) + (d == 0 ? eb[0] : 0);
+        const ll dy[2] = {flip(m[2] - m[0], sb), flip(m[3] - m[1], sb)};
+        const ll dz[2] = {flip(x3(z[0], z[2]), sc), flip(x3(z[1], z[3]), sc)};
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            gx[i][d] = x3(dx[i], dx[1 - i]) + (d == 0 ? eb[0] : 0);
             gy[i][d] = x3(dy[i], dy[1 - i]) + (d == 1 ? eb[1] : d == 0 ? eb[5] : 0);
-#pragma unroll
-            for (int k = 0; k < 2; ++k) gz[i][k][d] = o[i][k] + (d == 2 ? eb[2] : d == 1 ? eb[3] : eb[4]);
+            gz[i][d] = x3(dz[i], dz[1 - i]) + (d == 2 ? eb[2] : d == 1 ? eb[3] : eb[4]);
         }
     }
-    ll tx[2][3], ty[2][3], tz[2][2][3];   // this half's traction sums over a, b and c
+    // the words of the packed field that hold point a = 0 and 1 of this quarter
+    uint32_t q[2];
 #pragma unroll
-    for (int n = 0; n < 4; ++n) {   // one coordinate changes from one point to the next
-        const int a = n == 1 || n == 2, b = n >> 1;
-        ll e[6], s[6];
-        e[0] = gx[b][0];
-        e[1] = gy[a][1];
-        e[2] = gz[a][b][2];
-        e[3] = gz[a][b][1] + gy[a][2];
-        e[4] = gz[a][b][0] + gx[b][2];
-        e[5] = gy[a][0] + gx[b][1];
-        const uint32_t q = h ? spin_of(sp, local_slot(a + 2 * b + 4)) : spin_of(sp, local_slot(a + 2 * b));
-        if (q != qprev) {
-            row.load(tab, q);
-            qprev = q;
-        }
+    for (int a = 0; a < 2; ++a) {
+        const uint32_t q0 = b ? spin_of(sp, local_slot(a + 2)) : spin_of(sp, local_slot(a));
+        const uint32_t q1 = b ? spin_of(sp, local_slot(a + 6)) : spin_of(sp, local_slot(a + 4));
+        q[a] = c ? q1 : q0;
+    }
+    FxRow row;
+    row.load(tab, q[0]);
+    ll tx[3], ty[2][3], tz[2][3];   // this quarter's share of the traction sums over a, b and c
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+        ll s[6];
+        const ll e[6] = {gx[0], gy[a][1], gz[a][2], gz[a][1] + gy[a][2], gz[a][0] + gx[2], gy[a][0] + gx[1]};
+        if (a == 1 && q[1] != q[0]) row.load(tab, q[1]);
         fx_hooke(row, e, s);
         const ll x[3] = {s[0], s[5], s[4]}, y[3] = {s[5], s[1], s[3]}, z[3] = {s[4], s[3], s[2]};
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            tx[b][d] = n == 0 || n == 2 ? x[d] : tx[b][d] + x[d];
-            ty[a][d] = n == 0 || n == 1 ? y[d] : ty[a][d] + y[d];
-            tz[a][b][d] = z[d];
+            tx[d] = a ? tx[d] + x[d] : x[d];
+            ty[a][d] = y[d];
+            tz[a][d] = z[d];
         }
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        ll X[2], Y[2], Z[2][2];   // X[J], Y[I] on the near plane, Z[I][J]
+        const ll ex = x3(tx[d], across(tx[d], 8)) >> 3, X = x3(ex, across(ex, 16));   // X[b][c]
+        ll Y[2], Z[2];                                                                 // Y[I][c], Z[I][b]
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const ll ex = x3(tx[i][d], tx[1 - i][d]) >> 3, ey = x3(ty[i][d], ty[1 - i][d]) >> 3;
-            X[i] = x3(ex, other_half(ex));
-            Y[i] = x3(ey, other_half(ey));
-#pragma unroll
-            for (int k = 0; k < 2; ++k) tz[i][k][d] += other_half(tz[i][k][d]);
+            ty[i][d] += across(ty[i][d], 8);
+            tz[i][d] += across(tz[i][d], 16);
         }
-        interp31<3>(tz[0][0][d], tz[1][0][d], tz[0][1][d], tz[1][1][d], Z);
 #pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            const int I = n & 1, J = n >> 1;
-            f[n][d] = (I ? X[J] : -X[J]) + (J ? Y[I] : -Y[I]) + (((Z[I][J]) ^ ~up) - ~up);
+        for (int i = 0; i < 2; ++i) {
+            const ll ey = x3(ty[i][d], ty[1 - i][d]) >> 3, ez = x3(tz[i][d], tz[1 - i][d]) >> 3;
+            Y[i] = x3(ey, across(ey, 16));
+            Z[i] = x3(ez, across(ez, 8));
+            f[i][d] = (i ? X : -X) + flip(Y[i], ~sb) + flip(Z[i], ~sc);
         }
     }
 }
@@ -359,14 +353,14 @@ __device__ __forceinline__ void fx_mean(FxMean &m, const DevState *st) {   // by
     m.e = E;
 }
 
-// a cell: its corners lie at n0 and n1 (lower and upper plane; for a half cell the near and the far
-// one), P nodes a row; returns its exponent
+// a cell: its corners lie at n0 and n1 (lower and upper plane; for a quarter near and far), dy apart in
+// y; returns its exponent
 __device__ __forceinline__ int fx_corners(const FxHalf *xy0, const FxHalf *ze0, const FxHalf *xy1, const FxHalf *ze1,
-                                          int P, const FxMean &m, ll (&u)[8][3], ll (&eb)[6]) {
+                                          int dy, const FxMean &m, ll (&u)[8][3], ll (&eb)[6]) {
     int ne[8], E = m.e;
 #pragma unroll
     for (int n = 0; n < 8; ++n) {
-        const int o = (n & 1) + (n & 2 ? P : 0);
+        const int o = (n & 1) + (n & 2 ? dy : 0);
         const FxHalf p = (n & 4 ? xy1 : xy0)[o], q = (n & 4 ? ze1 : ze0)[o];
         u[n][0] = p.a;
         u[n][1] = p.b;
@@ -498,14 +492,15 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
                 if (ncol[m] >= 0) fx_put(sm.uxy[b], sm.uze[b], tid + m * MPM_THREADS, pl[m]);
         };
         int b0 = 0, b1 = 1, b2 = 2, fb = 0;
-        // nothing above reads what the kernels before this one write: 1.2 us a step against a wait ahead
+        if (tid == 0) fx_mean(sm.m, R.st);
+        // nothing above reads what the kernels before this one write (the mean strain comes from the end of a
+        // Monte Carlo step, which lets no kernel start early): 1.2 us a step against a wait ahead
         // of the range's look-ups
         asm volatile("griddepcontrol.wait;" ::: "memory");
         fetch(k0 - 1);
         store(b0);
         fetch(k0);
         store(b1);
-        if (tid == 0) fx_mean(sm.m, R.st);
         uint4 sp = need ? __ldg(a.spins + col + (long long)plane * wrapi(k0 - 1, nbz)) : make_uint4(0, 0, 0, 0);
         __syncthreads();
 
@@ -565,15 +560,16 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
 
 // The block form (k_mpm.cu): one block per CTA, every cell at once, on SPLIT threads each.  Blocks of
 // at most 96 cells run where there is one to an SM, three warps of whole cells: what bounds them is
-// the length of a cell's code, and halves take 8.6 us a step at 32^3 where whole cells took 11.4.
-// Blocks of 256 cells fill the registers as they are (halves at 128 registers: 24.6 -> 30.3 us at 64^3;
-// the march likewise, 102 -> 133 us at 128^3).
+// the length of a cell's code, and quarters take 7.8 us a step at 32^3 where halves took 8.5 and whole
+// cells 11.4.  Blocks of 256 cells fill the registers as they are (halves at 128 registers: 24.6 ->
+// 30.3 us at 64^3; the march likewise, 102 -> 133 us at 128^3).
 template <int CELLS, int SPLIT, bool SCALED>
 __global__ void __launch_bounds__(CELLS *SPLIT, 1) k_mpm_fixed_block(MpmArgs<double> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FxBlockSmem<CELLS> &sm = *reinterpret_cast<FxBlockSmem<CELLS> *>(smem_raw);
     const int tid = threadIdx.x;
-    const int cell = SPLIT == 2 ? half_cell(tid) : tid, h = SPLIT == 2 ? tid >> 4 & 1 : 0;
+    const int cell = SPLIT == 4 ? (tid >> 5) * 8 + (tid & 7) : tid;
+    const int b = SPLIT == 4 ? tid >> 3 & 1 : 0, c = SPLIT == 4 ? tid >> 4 & 1 : 0;   // this thread's quarter
     const FxUpdate<SCALED> update(a);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     int r = 0;
@@ -588,13 +584,16 @@ __global__ void __launch_bounds__(CELLS *SPLIT, 1) k_mpm_fixed_block(MpmArgs<dou
     };
     const int cells = W * H * B.D;
     const int ci = cell % W, cj = cell / W % H, ck = cell / (W * H);
-    const bool need = cell < cells, some = SPLIT == 2 ? (tid >> 5) * 16 < cells : need;   // (halves: the whole warp)
+    const bool need = cell < cells, some = SPLIT == 4 ? (tid >> 5) * 8 < cells : need;   // (quarters: the whole warp)
     const int lci = tid % W, lcj = tid / W % H, lck = tid / (W * H);   // the first threads own nodes
     const bool own = tid < cells && lci >= 1 && lcj >= 1 && lck >= 1;
     const long long at = own ? block_at(lci, lcj, lck) : 0, cat = need ? block_at(ci, cj, ck) : 0;
-    long long node[2 / SPLIT];
+    constexpr int PER = SPLIT == 4 ? 1 : 2;   // nodes a thread converts: the blocks have at most two a cell
+    long long node[PER];
 #pragma unroll
-    for (int m = 0; m < 2 / SPLIT; ++m) node[m] = B.node(R, tid + m * CELLS);
+    for (int m = 0; m < PER; ++m) node[m] = B.node(R, tid + m * CELLS);
+    // (the mean strain is written only by the end of a Monte Carlo step, which lets no kernel start early)
+    if (tid == 0) fx_mean(sm.m, R.st);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint4 sp = need ? __ldg(a.spins + cat) : make_uint4(0, 0, 0, 0);
     double uold[3] = {0, 0, 0}, vold[3] = {0, 0, 0};
@@ -606,26 +605,25 @@ __global__ void __launch_bounds__(CELLS *SPLIT, 1) k_mpm_fixed_block(MpmArgs<dou
         }
     }
 #pragma unroll
-    for (int m = 0; m < 2 / SPLIT; ++m)
+    for (int m = 0; m < PER; ++m)
         if (node[m] >= 0) {
             const double *p = a.u_in + 3 * node[m];
             const double u[3] = {__ldg(p), __ldg(p + 1), __ldg(p + 2)};
             fx_put(sm.uxy, sm.uze, tid + m * CELLS, u);
         }
-    if (tid == 0) fx_mean(sm.m, R.st);
     __syncthreads();
     if (some) {
         ll u[8][3], eb[6], f[8 / SPLIT][3];
-        const int nd = need ? ci + P * cj + PP * ck : 0, n0 = nd + (h ? PP : 0), n1 = nd + (h ? 0 : PP);
-        const int E = fx_corners(sm.uxy + n0, sm.uze + n0, sm.uxy + n1, sm.uze + n1, P, sm.m, u, eb);
-        if constexpr (SPLIT == 2)
-            fx_half(u, eb, sp, h, a.cfix, f);
+        const int nd = need ? ci + P * cj + PP * ck : 0, n0 = nd + (b ? P : 0) + (c ? PP : 0), dz = c ? -PP : PP;
+        const int E = fx_corners(sm.uxy + n0, sm.uze + n0, sm.uxy + n0 + dz, sm.uze + n0 + dz, b ? -P : P, sm.m, u, eb);
+        if constexpr (SPLIT == 4)
+            fx_quarter(u, eb, sp, b, c, a.cfix, f);
         else
             fx_cell(u, eb, sp, a.cfix, f);
 #pragma unroll
         for (int n = 0; n < 8 / SPLIT; ++n) {
-            sm.fxy[4 * h + n][cell] = FxHalf{f[n][0], f[n][1]};
-            sm.fze[4 * h + n][cell] = FxHalf{f[n][2], (ll)E};
+            sm.fxy[2 * b + 4 * c + n][cell] = FxHalf{f[n][0], f[n][1]};
+            sm.fze[2 * b + 4 * c + n][cell] = FxHalf{f[n][2], (ll)E};
         }
     }
     __syncthreads();
@@ -644,7 +642,7 @@ Form form_of(int variant) {
     if (!mpm_is_block(variant)) return Form{k_mpm_fixed<SCALED>, MPM_THREADS, sizeof(FxMarchSmem)};
     if (variant == MPM_BLOCK)
         return Form{k_mpm_fixed_block<MPM_THREADS, 1, SCALED>, MPM_THREADS, sizeof(FxBlockSmem<MPM_THREADS>)};
-    return Form{k_mpm_fixed_block<MPM_SMALL_BLOCK, 2, SCALED>, 2 * MPM_SMALL_BLOCK,
+    return Form{k_mpm_fixed_block<MPM_SMALL_BLOCK, 4, SCALED>, 4 * MPM_SMALL_BLOCK,
                 sizeof(FxBlockSmem<MPM_SMALL_BLOCK>)};
 }
 
