@@ -1,6 +1,8 @@
 // Stress of every material point (for the sweeps), the end-of-step reductions
 // and loading control, statistics (unlike bonds, orientation volumes, texture
 // bins) and the spin layout conversions.
+#include <cooperative_groups.h>
+
 #include "hmc_device.cuh"
 
 namespace hmc {
@@ -101,6 +103,31 @@ static_assert(BLOCK_THREADS % STRESS_THREADS == 0, "a tile splits evenly over th
 template <typename T>
 constexpr int stress_wide() { return sizeof(T) == 4 ? 304 : 152; }
 
+// A tile's partial sums from the accumulators of its first STRESS_THREADS threads.
+template <typename T>
+__device__ __forceinline__ void tile_sums(Acc7<T> &acc, double (&red)[STRESS_THREADS / 32][7], double *out) {
+    acc.warp_reduce();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0)
+        for (int i = 0; i < 7; ++i) red[warp][i] = acc.get(i);
+    asm volatile("bar.sync 1, %0;" ::"n"(STRESS_THREADS) : "memory");   // the two warps that sum
+    if (threadIdx.x < 7) {
+        double s = 0.0;
+        for (int w = 0; w < STRESS_THREADS / 32; ++w) s += red[w][threadIdx.x];
+        out[threadIdx.x] = s;
+    }
+}
+// ... from the sums of its n <= BLOCK_THREADS blocks, added in the order of the form without them
+template <typename T>
+__device__ __forceinline__ void tile_sums(const T (*cells)[7], int n, double (&red)[STRESS_THREADS / 32][7], double *out) {
+    Acc7<T> acc;
+    acc.zero();
+    for (int t = threadIdx.x; t < n; t += STRESS_THREADS)
+#pragma unroll
+        for (int k = 0; k < 7; ++k) acc.add(k, cells[t][k]);
+    tile_sums<T>(acc, red, out);
+}
+
 template <typename T, bool STORE, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? BLOCK_THREADS : STRESS_THREADS, sizeof(T) == 4 ? (WIDE ? 2 : 8) : 1)
     k_stress(StressArgs<T> a) {
@@ -195,23 +222,111 @@ __global__ void __launch_bounds__(WIDE ? BLOCK_THREADS : STRESS_THREADS, sizeof(
         }
         blk = blk_next;
     }
+    double *out = a.partials + 7ll * blockIdx.x;
     if constexpr (WIDE) {
         __syncthreads();
-        if (threadIdx.x >= STRESS_THREADS) return;
-        for (int t = threadIdx.x; t < BLOCK_THREADS && t0 + t < R.nblk; t += STRESS_THREADS)
+        if (threadIdx.x < STRESS_THREADS) tile_sums<T>(cells, min(BLOCK_THREADS, R.nblk - t0), red, out);
+    } else {
+        tile_sums<T>(acc, red, out);
+    }
+}
+
+// The FP64 pass on small grids: a cluster of SPLIT CTAs to a tile and four threads to a cell, two points
+// each.  An SM retires two FP64 lanes a clock, so what counts is over how many SMs the points are
+// spread: a call at 32^3 took 70 us with its 16 tiles on 16 SMs and takes 45 us (24^3: 70 and 36),
+// although a cell costs 1.5 times the operations (gradients formed once per thread).  16 clusters do not
+// quite fit one CTA to an SM; asking for an SM each did not help.  The line: see launch_stress.
+// The same products and sums in the same order as the other forms (a cell's points are summed in
+// slot order, then tile_sums), so the bits are the same.
+constexpr int SPLIT = 8, SPLIT_CELLS = BLOCK_THREADS / SPLIT;
+template <bool STORE>
+__global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(4 * SPLIT_CELLS) k_stress_split(StressArgs<double> a) {
+    namespace cg = cooperative_groups;
+    __shared__ double red[STRESS_THREADS / 32][7];
+    __shared__ double pts[8][7][SPLIT_CELLS + 1];      // by slot: stress, energy
+    __shared__ double cells[BLOCK_THREADS][7];         // of the tile, in its first CTA
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    cg::cluster_group cl = cg::this_cluster();
+    const int part = blockIdx.x % SPLIT, tile = blockIdx.x / SPLIT;
+    const Replica &R = a.reps[__ldg(a.cta_rep + tile)];
+    const int nblk = R.nblk, tile0 = (tile - R.cta_off) * BLOCK_THREADS, t0 = tile0 + part * SPLIT_CELLS;
+    const int nbx = R.nbx, nby = R.nby, nbz = R.nbz;
+    const double *u = a.u + 3 * R.blk_off;
+    double eb[6];
+    load_ebar<double>(R.st, eb);   // written only by the end of a step, which lets no kernel start early
+    const int tid = threadIdx.x, cell = tid >> 2, b = tid & 1, c = tid >> 1 & 1, blk = t0 + cell;
+    const bool live = blk < nblk;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (live) {
+        const uint4 sp = __ldg(a.spins + R.blk_off + blk);
+        double uc[8][3];
+        const int bx = blk % nbx, rr = blk / nbx, by = rr % nby, bz = rr / nby;
 #pragma unroll
-            for (int k = 0; k < 7; ++k) acc.add(k, cells[t][k]);
+        for (int n = 0; n < 8; ++n) {
+            const int gi = (n & 1) && bx + 1 == nbx ? 0 : bx + (n & 1), gj = (n & 2) && by + 1 == nby ? 0 : by + (n >> 1 & 1);
+            const int gk = (n & 4) && bz + 1 == nbz ? 0 : bz + (n >> 2);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) uc[n][d] = __ldg(u + 3 * (gi + nbx * (gj + nby * gk)) + d);
+        }
+        // interp2's two stages at one point: x d0 + y d1
+        auto mix = [](double x, double d0, double y, double d1) { return rfma(x, d0, rmul(y, d1)); };
+        const double b0 = b ? 0.25 : 0.75, b1 = b ? 0.75 : 0.25;   // first stage, weights in y
+        const double hb0 = b ? 0.125 : 0.375, hb1 = b ? 0.375 : 0.125, hc0 = c ? 0.125 : 0.375, hc1 = c ? 0.375 : 0.125;
+        double gx[3], gy[2][3], gz[2][3];   // [d], [a][d]
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            gx[d] = mix(hc0, mix(b0, uc[1][d] - uc[0][d], b1, uc[3][d] - uc[2][d]), hc1,
+                        mix(b0, uc[5][d] - uc[4][d], b1, uc[7][d] - uc[6][d]));
+            const double y00 = uc[2][d] - uc[0][d], y10 = uc[3][d] - uc[1][d], y01 = uc[6][d] - uc[4][d], y11 = uc[7][d] - uc[5][d];
+            const double z00 = uc[4][d] - uc[0][d], z10 = uc[5][d] - uc[1][d], z01 = uc[6][d] - uc[2][d], z11 = uc[7][d] - uc[3][d];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const double p = i ? 0.25 : 0.75, q = i ? 0.75 : 0.25;
+                gy[i][d] = mix(hc0, mix(p, y00, q, y10), hc1, mix(p, y01, q, y11));
+                gz[i][d] = mix(hb0, mix(p, z00, q, z10), hb1, mix(p, z01, q, z11));
+            }
+        }
+        Row24<double> row;
+        uint32_t qprev = 0xffffffffu;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t q0 = b ? spin_of(sp, local_slot(i + 2)) : spin_of(sp, local_slot(i));
+            const uint32_t q1 = b ? spin_of(sp, local_slot(i + 6)) : spin_of(sp, local_slot(i + 4));
+            const uint32_t q = c ? q1 : q0;
+            if (q != qprev) {
+                row.load(a.ctab + 24ll * q);
+                qprev = q;
+            }
+            const double e[6] = {eb[0] + gx[0], eb[1] + gy[i][1], eb[2] + gz[i][2], eb[3] + (gz[i][1] + gy[i][2]),
+                                 eb[4] + (gz[i][0] + gx[2]), eb[5] + (gy[i][0] + gx[1])};
+            double st[6], w = 0.0;
+            hooke21<double>(row.v, e, st);
+            double(&out)[7][SPLIT_CELLS + 1] = pts[local_slot(i + 2 * b + 4 * c)];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                out[k][cell] = st[k];
+                w = rfma(st[k], e[k], w);
+            }
+            out[6][cell] = 0.5 * w;
+        }
     }
-    acc.warp_reduce();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0)
-        for (int i = 0; i < 7; ++i) red[warp][i] = acc.get(i);
-    asm volatile("bar.sync 1, %0;" ::"n"(STRESS_THREADS) : "memory");   // the two warps that sum
-    if (threadIdx.x < 7) {
+    cl.sync();   // the points are there, and the tile's first CTA runs
+    double(*to)[7] = cl.map_shared_rank(cells, 0) + part * SPLIT_CELLS;
+    for (int i = tid; i < 7 * SPLIT_CELLS; i += 4 * SPLIT_CELLS) {
+        const int k = i / SPLIT_CELLS, n = i % SPLIT_CELLS;
         double s = 0.0;
-        for (int w = 0; w < STRESS_THREADS / 32; ++w) s += red[w][threadIdx.x];
-        a.partials[7ll * blockIdx.x + threadIdx.x] = s;
+#pragma unroll
+        for (int slot = 0; slot < 8; ++slot) s += pts[slot][k][n];
+        if (t0 + n < nblk) to[n][k] = s;
     }
+    if (STORE && live) {
+        double *sig = a.sig + 48ll * R.blk_off + 4ll * t0 + tid;
+#pragma unroll
+        for (int i = 0; i < 12; ++i) __stcs(sig + 4ll * i * nblk, pts[i / 6 * 4 + (tid & 3)][i % 6][cell]);
+    }
+    cl.sync();   // the tile's sums are there
+    if (part == 0 && tid < STRESS_THREADS)
+        tile_sums<double>(cells, min(BLOCK_THREADS, nblk - tile0), red, a.partials + 7ll * tile);
 }
 
 // sum over the lanes of a warp (a butterfly: every lane has it)
@@ -424,8 +539,15 @@ __global__ void k_bins(const unsigned long long *counts, const int32_t *binmap, 
 
 }  // namespace
 
+// FP64 tiles up to which the pass is spread over clusters: three CTAs to an SM (a call at 40^3, 32
+// tiles, takes 46 us against 70; at 48^3, 54 tiles, 69 against 71; at 56^3, 86 tiles, 82 against 71)
+constexpr int STRESS_SPLIT = 57;
+
 template <typename T>
 cudaError_t launch_stress(const StressArgs<T> &a, bool store, cudaStream_t s) {
+    if constexpr (sizeof(T) == 8)
+        if (a.nctas <= STRESS_SPLIT)
+            return launch_pdl(store ? k_stress_split<true> : k_stress_split<false>, a.nctas * SPLIT, 4 * SPLIT_CELLS, 0, s, a);
     if (a.nctas <= stress_wide<T>())
         return launch_pdl(store ? k_stress<T, true, true> : k_stress<T, false, true>, a.nctas, BLOCK_THREADS, 0, s, a);
     return launch_pdl(store ? k_stress<T, true, false> : k_stress<T, false, false>, a.nctas, STRESS_THREADS, 0, s, a);

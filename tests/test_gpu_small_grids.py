@@ -89,3 +89,23 @@ def test_many_steps_equal_single_steps(G, mpm):
     for other in out[1:]:
         for a, b in zip(out[0], other):
             assert np.array_equal(a, b)
+
+
+def test_fp64_stress_forms_on_both_sides_of_the_line(G):
+    # 56, 59 and 61 tiles: alone the first is spread over clusters and the others take one CTA a tile; all
+    # three together (176) take the form of large grids
+    Q, shapes = 9, [(44, 52, 50), (46, 52, 50), (48, 52, 50)]
+    eul = S.euler_uniform_so3(Q, 2)
+    fields = [S.voronoi_spins(s, 60, Q, 3) for s in shapes]
+    common = dict(precision=0, strain=2e-3, mpm_steps_per_mcs=2, **C3)
+    b = G.HMCBatch(shapes, Q, [dict(seed=5)] * 3, **common)
+    b.set_orientations(eul, fields)
+    b.mc_sweeps(2)
+    for r, shape in enumerate(shapes):
+        g = G.HMC(shape, Q, seed=5, **common)
+        g.set_orientations(eul, fields[r])
+        g.mc_sweeps(2)
+        assert np.array_equal(g.strain(), b.strain(r)) and np.array_equal(g.spins(), b.spins(r))
+        assert np.array_equal(g.nodal()[1], b.nodal(r)[1])
+        g.close()
+    b.close()
