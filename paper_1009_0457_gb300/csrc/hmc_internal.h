@@ -228,7 +228,9 @@ inline bool mpm_is_block(int variant) { return variant == MPM_BLOCK || variant =
 
 // A launch with programmatic stream serialisation: the kernel may be scheduled before the one ahead
 // of it in the stream has finished, and executes griddepcontrol.wait before it reads or writes
-// anything that another kernel touches.
+// anything that another kernel touches.  What the kernels before it wrote it reads by ordinary loads:
+// the read-only path (__ldg) is for data that nothing writes while the kernel runs, its own wait
+// included, and its loads may be moved ahead of the wait.
 template <typename... P, typename... A>
 cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
                        const A &...args) {

@@ -71,16 +71,16 @@ struct PlaneLoad {
         }
     }
     // node plane k, -1 <= k <= nbz (periodic in z)
-    __device__ __forceinline__ void fetch(const float *__restrict__ u, long long node0, int k, int nbz, int plane) {
+    __device__ __forceinline__ void fetch(const float *u, long long node0, int k, int nbz, int plane) {
         const int gk = k < 0 ? k + nbz : (k >= nbz ? k - nbz : k);
         const float *base = u + 3 * (node0 + (long long)plane * gk);
 #pragma unroll
         for (int m = 0; m < PER; ++m)
             if (col[m] >= 0) {
                 const float *p = base + 3 * col[m];
-                r[m][0] = __ldg(p);
-                r[m][1] = __ldg(p + 1);
-                r[m][2] = __ldg(p + 2);
+                r[m][0] = p[0];
+                r[m][1] = p[1];
+                r[m][2] = p[2];
             }
     }
     __device__ __forceinline__ void store(Vec4 *us) const {
@@ -347,17 +347,17 @@ __global__ void __launch_bounds__(GT *GROUPS, 512 / (GT * GROUPS)) k_mpm_step(Mp
         PlaneLoad<GT> pl;
         int b0 = 0, b1 = 1, b2 = 2;
         pl.prepare(i0, j0, P, P * (H + 1), nbx, nby);
-        // u, v, the spins and the mean strain come from the kernels before this one; everything above
-        // reads only tables (from the second tile on there is nothing left to wait for).  With the
-        // wait ahead of the range's look-ups, a chain of dependent loads, a step took 1.35 us more
-        // (128^3 19.0 -> 17.65 us); with the two first planes loaded one after the other, 0.25 us more
+        // u, v and the spins come from the kernels before this one; everything above reads only tables
+        // (from the second tile on there is nothing left to wait for).  With the wait ahead of the
+        // range's look-ups, a chain of dependent loads, a step took 1.35 us more (128^3 19.0 -> 17.65
+        // us); with the two first planes loaded one after the other, 0.25 us more
         asm volatile("griddepcontrol.wait;" ::: "memory");
         float eb[6];
         load_ebar<float>(R.st, eb);
         PlaneLoad<GT> pl0 = pl;
         pl0.fetch(a.u_in, node0, k0 - 1, nbz, plane);
         pl.fetch(a.u_in, node0, k0, nbz, plane);
-        uint4 sp = need ? __ldg(a.spins + col + (long long)plane * wrapi(k0 - 1, nbz)) : make_uint4(0, 0, 0, 0);
+        uint4 sp = need ? a.spins[col + (long long)plane * wrapi(k0 - 1, nbz)] : make_uint4(0, 0, 0, 0);
         pl0.store(sm.us[b0]);
         pl.store(sm.us[b1]);
         march_sync<GT, GROUPS>();
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(GT *GROUPS, 512 / (GT * GROUPS)) k_mpm_step(Mp
         for (int kk = k0 - 1; kk < kend; ++kk) {
             // one plane ahead: next plane's spins and u, this plane's owned velocity
             uint4 sp_next = make_uint4(0, 0, 0, 0);
-            if (need && kk + 1 < kend) sp_next = __ldg(spn);
+            if (need && kk + 1 < kend) sp_next = *spn;
             spn += plane;
             float vold[3] = {0.f, 0.f, 0.f};
             if (own && kk >= k0) {
@@ -461,22 +461,22 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_mpm_block(MpmArgs<fl
     long long node[PER];
 #pragma unroll
     for (int m = 0; m < PER; ++m) node[m] = B.node(R, tid + m * THREADS);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     float eb[6], un[3] = {0.f, 0.f, 0.f}, vold[3] = {0.f, 0.f, 0.f};
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     load_ebar<float>(R.st, eb);
-    const uint4 sp = need ? __ldg(a.spins + at) : make_uint4(0, 0, 0, 0);
+    const uint4 sp = need ? a.spins[at] : make_uint4(0, 0, 0, 0);
     if (own) {
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             vold[d] = a.v[3 * at + d];
-            un[d] = __ldg(a.u_in + 3 * at + d);
+            un[d] = a.u_in[3 * at + d];
         }
     }
 #pragma unroll
     for (int m = 0; m < PER; ++m)
         if (node[m] >= 0) {
             const float *p = a.u_in + 3 * node[m];
-            sm.us[tid + m * THREADS] = Vec4{__ldg(p) * 0.03125f, __ldg(p + 1) * 0.03125f, __ldg(p + 2) * 0.03125f, 0.f};
+            sm.us[tid + m * THREADS] = Vec4{p[0] * 0.03125f, p[1] * 0.03125f, p[2] * 0.03125f, 0.f};
         }
     __syncthreads();
     if (need) {

@@ -32,7 +32,7 @@
 // barrier per plane.
 // What bounds it: 244 registers leave eight warps per SM, which issue 36 % of the cycles (the
 // busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
-// 32^3 7.8 (70), 100^3 52 (308), 128^3 102 (420), 256^3 709 (3330).
+// 32^3 8.2 (70), 100^3 52 (308), 128^3 102 (420), 256^3 709 (3330).
 #include "hmc_device.cuh"
 
 namespace hmc {
@@ -484,7 +484,7 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
             for (int m = 0; m < PER; ++m)
                 if (ncol[m] >= 0)
 #pragma unroll
-                    for (int d = 0; d < 3; ++d) pl[m][d] = __ldg(base + 3 * ncol[m] + d);
+                    for (int d = 0; d < 3; ++d) pl[m][d] = base[3 * ncol[m] + d];
         };
         auto store = [&](int b) {
 #pragma unroll
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
         store(b0);
         fetch(k0);
         store(b1);
-        uint4 sp = need ? __ldg(a.spins + col + (long long)plane * wrapi(k0 - 1, nbz)) : make_uint4(0, 0, 0, 0);
+        uint4 sp = need ? a.spins[col + (long long)plane * wrapi(k0 - 1, nbz)] : make_uint4(0, 0, 0, 0);
         __syncthreads();
 
         Fx3 acc = {{0, 0, 0}, 0};
@@ -512,14 +512,14 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
         const long long pstride = 3ll * plane;
         for (int kk = k0 - 1; kk < kend; ++kk) {
             uint4 sp_next = make_uint4(0, 0, 0, 0);
-            if (need && kk + 1 < kend) sp_next = __ldg(spn);
+            if (need && kk + 1 < kend) sp_next = *spn;
             spn += plane;
             double vold[3] = {0, 0, 0}, uold[3] = {0, 0, 0};
             if (own && kk >= k0) {
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
                     vold[d] = vp[d];
-                    uold[d] = __ldg(uip + d);
+                    uold[d] = uip[d];
                 }
             }
             const bool more = kk + 1 < kend;
@@ -560,8 +560,7 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
 
 // The block form (k_mpm.cu): one block per CTA, every cell at once, on SPLIT threads each.  Blocks of
 // at most 96 cells run where there is one to an SM, three warps of whole cells: what bounds them is
-// the length of a cell's code, and quarters take 7.8 us a step at 32^3 where halves took 8.5 and whole
-// cells 11.4.  Blocks of 256 cells fill the registers as they are (halves at 128 registers: 24.6 ->
+// the length of a cell's code, and quarters take 8.2 us a step at 32^3 where whole cells took 11.4.  Blocks of 256 cells fill the registers as they are (halves at 128 registers: 24.6 ->
 // 30.3 us at 64^3; the march likewise, 102 -> 133 us at 128^3).
 template <int CELLS, int SPLIT, bool SCALED>
 __global__ void __launch_bounds__(CELLS *SPLIT, 1) k_mpm_fixed_block(MpmArgs<double> a) {
@@ -592,23 +591,24 @@ __global__ void __launch_bounds__(CELLS *SPLIT, 1) k_mpm_fixed_block(MpmArgs<dou
     long long node[PER];
 #pragma unroll
     for (int m = 0; m < PER; ++m) node[m] = B.node(R, tid + m * CELLS);
-    // (the mean strain is written only by the end of a Monte Carlo step, which lets no kernel start early)
+    // (the mean strain is written only by the end of a Monte Carlo step, which lets no kernel start
+    // early; converted behind the wait 32^3 took 8.55 us instead of 8.2)
     if (tid == 0) fx_mean(sm.m, R.st);
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const uint4 sp = need ? __ldg(a.spins + cat) : make_uint4(0, 0, 0, 0);
+    const uint4 sp = need ? a.spins[cat] : make_uint4(0, 0, 0, 0);
     double uold[3] = {0, 0, 0}, vold[3] = {0, 0, 0};
     if (own) {
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             vold[d] = a.v[3 * at + d];
-            uold[d] = __ldg(a.u_in + 3 * at + d);
+            uold[d] = a.u_in[3 * at + d];
         }
     }
 #pragma unroll
     for (int m = 0; m < PER; ++m)
         if (node[m] >= 0) {
             const double *p = a.u_in + 3 * node[m];
-            const double u[3] = {__ldg(p), __ldg(p + 1), __ldg(p + 2)};
+            const double u[3] = {p[0], p[1], p[2]};
             fx_put(sm.uxy, sm.uze, tid + m * CELLS, u);
         }
     __syncthreads();

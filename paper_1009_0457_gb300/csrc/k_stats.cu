@@ -159,9 +159,9 @@ __global__ void __launch_bounds__(WIDE ? BLOCK_THREADS : STRESS_THREADS, sizeof(
                     const int gk = bz + K == nbz ? 0 : bz + K;
                     const int n = 3 * (gi + nbx * (gj + nby * gk));
 #pragma unroll
-                    for (int d = 0; d < 3; ++d) uc[corner(I, J, K)][d] = __ldg(u + n + d);
+                    for (int d = 0; d < 3; ++d) uc[corner(I, J, K)][d] = u[n + d];
                 }
-        sp = __ldg(a.spins + R.blk_off + blk);
+        sp = a.spins[R.blk_off + blk];
     };
     T un[8][3];
     uint4 spn = make_uint4(0, 0, 0, 0);
@@ -258,7 +258,7 @@ __global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(4 * SPLIT_CELLS)
     const bool live = blk < nblk;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (live) {
-        const uint4 sp = __ldg(a.spins + R.blk_off + blk);
+        const uint4 sp = a.spins[R.blk_off + blk];
         double uc[8][3];
         const int bx = blk % nbx, rr = blk / nbx, by = rr % nby, bz = rr / nby;
 #pragma unroll
@@ -266,7 +266,7 @@ __global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(4 * SPLIT_CELLS)
             const int gi = (n & 1) && bx + 1 == nbx ? 0 : bx + (n & 1), gj = (n & 2) && by + 1 == nby ? 0 : by + (n >> 1 & 1);
             const int gk = (n & 4) && bz + 1 == nbz ? 0 : bz + (n >> 2);
 #pragma unroll
-            for (int d = 0; d < 3; ++d) uc[n][d] = __ldg(u + 3 * (gi + nbx * (gj + nby * gk)) + d);
+            for (int d = 0; d < 3; ++d) uc[n][d] = u[3 * (gi + nbx * (gj + nby * gk)) + d];
         }
         // interp2's two stages at one point: x d0 + y d1
         auto mix = [](double x, double d0, double y, double d1) { return rfma(x, d0, rmul(y, d1)); };

@@ -418,12 +418,12 @@ __global__ void __launch_bounds__(CTA, flat_min_ctas<T, MODE, RECOMP, CTA>())
         const uint2 mine = COL ? make_uint2(own4.z, own4.w) : make_uint2(own4.x, own4.y);
         const uint2 O = oc ? make_uint2(own4.z, own4.w) : make_uint2(own4.x, own4.y);
         uint2 N[6];
-        N[0] = __ldg(q2 + 2 * (blk + (bx == 0 ? nbx - 1 : -1)) + oc);
-        N[1] = __ldg(q2 + 2 * (blk + (bx == nbx - 1 ? 1 - nbx : 1)) + oc);
-        N[2] = __ldg(q2 + 2 * (blk + (by == 0 ? (nby - 1) * sxy : -sxy)) + oc);
-        N[3] = __ldg(q2 + 2 * (blk + (by == nby - 1 ? -(nby - 1) * sxy : sxy)) + oc);
-        N[4] = __ldg(q2 + 2 * (blk + (bz == 0 ? (nbz - 1) * sxz : -sxz)) + oc);
-        N[5] = __ldg(q2 + 2 * (blk + (bz == nbz - 1 ? -(nbz - 1) * sxz : sxz)) + oc);
+        N[0] = q2[2 * (blk + (bx == 0 ? nbx - 1 : -1)) + oc];
+        N[1] = q2[2 * (blk + (bx == nbx - 1 ? 1 - nbx : 1)) + oc];
+        N[2] = q2[2 * (blk + (by == 0 ? (nby - 1) * sxy : -sxy)) + oc];
+        N[3] = q2[2 * (blk + (by == nby - 1 ? -(nby - 1) * sxy : sxy)) + oc];
+        N[4] = q2[2 * (blk + (bz == 0 ? (nbz - 1) * sxz : -sxz)) + oc];
+        N[5] = q2[2 * (blk + (bz == nbz - 1 ? -(nbz - 1) * sxz : sxz)) + oc];
         uint16_t q[4];
         block_trials<COL>(a.trial, a.nq, mine, O, N, rnd, q, qn, dE);
         // recompute mode: the cell's displacement gradients, formed at the first listed trial
@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(CTA, flat_min_ctas<T, MODE, RECOMP, CTA>())
                                 const int gk = bz + K == nbz ? 0 : bz + K;
                                 const int n = 3 * (gi + nbx * (gj + nby * gk));
 #pragma unroll
-                                for (int d = 0; d < 3; ++d) uc[corner(I, J, K)][d] = __ldg(u + n + d);
+                                for (int d = 0; d < 3; ++d) uc[corner(I, J, K)][d] = u[n + d];
                             }
                     cell_gradients<T>(uc, g);
                     load_ebar<T>(R.st, ebv);
