@@ -560,8 +560,9 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
 
 // The block form (k_mpm.cu): one block per CTA, every cell at once, on SPLIT threads each.  Blocks of
 // at most 96 cells run where there is one to an SM, three warps of whole cells: what bounds them is
-// the length of a cell's code, and quarters take 8.2 us a step at 32^3 where whole cells took 11.4.  Blocks of 256 cells fill the registers as they are (halves at 128 registers: 24.6 ->
-// 30.3 us at 64^3; the march likewise, 102 -> 133 us at 128^3).
+// the length of a cell's code, and quarters take 8.2 us a step at 32^3 where whole cells took 11.4.
+// Blocks of 256 cells fill the registers as they are (halves at 128 registers: 24.6 -> 30.3 us at
+// 64^3; the march likewise, 102 -> 133 us at 128^3).
 template <int CELLS, int SPLIT, bool SCALED>
 __global__ void __launch_bounds__(CELLS *SPLIT, 1) k_mpm_fixed_block(MpmArgs<double> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
