@@ -121,7 +121,9 @@ struct hmc_handle {
         int rtab_version = -1;
         void *rtab = nullptr, *lam = nullptr, *ubar = nullptr, *vtmp = nullptr, *seg = nullptr;
         void *ck_u = nullptr, *ck_v = nullptr, *w = nullptr, *g = nullptr, *fcell = nullptr;
-        void *lsum = nullptr, *lerr = nullptr;   // sum of the reverse steps' lambdas (FP32: with its error)
+        // sum of the reverse steps' lambdas (FP32: with its error): two node arrays in the buffer of the
+        // field w (8 values a cell against 6), which is downloaded before a reverse sweep starts
+        void *lsum = nullptr, *lerr = nullptr;
         int seg_held = -1;                       // segment whose states `seg` holds
         double *partials = nullptr, *grad = nullptr;
         hmc::Replica *reps0 = nullptr;   // descriptors whose state has Ebar = 0
@@ -542,7 +544,7 @@ std::string validate_shared(const hmc_params *a, const hmc_params *b) {
 void free_adjoint(hmc_handle *h) {
     void *bufs[] = {h->adj.rtab, h->adj.lam, h->adj.ubar, h->adj.vtmp, h->adj.seg, h->adj.ck_u,
                     h->adj.ck_v, h->adj.w, h->adj.g, h->adj.fcell, h->adj.partials, h->adj.grad, h->adj.reps0,
-                    h->adj.st0, h->adj.lsum, h->adj.lerr};
+                    h->adj.st0};
     for (void *b : bufs)
         if (b) cudaFree(b);
     h->adj.rtab = h->adj.lam = h->adj.ubar = h->adj.vtmp = h->adj.seg = nullptr;
@@ -1217,13 +1219,19 @@ hmc_status hmc_create_batch(const hmc_params *params, int32_t n_replicas, hmc_ha
             {(void **)&h->zone_work, sizeof(uint4) * 4 * (size_t)h->nblk_total, "zone trial list"},
             {(void **)&h->snap, sizeof(uint4) * (size_t)h->nblk_total, "spin copy"},
             {(void **)&h->zone_count, 2 * sizeof(unsigned), "zone trial count"},
-            {(void **)&h->zone_open, well ? sizeof(unsigned) * 4 * (size_t)h->nblk_total : 0, "zone trial list"},
-            {&h->btab, well ? h->tsize * 8 * 48 * (size_t)p->n_orient : 0, "zone bound tables"},
             {&h->ktab, h->tsize * 8 * 320 * (size_t)p->n_orient, "zone element tables"},
             {(void **)&h->zone_sched, sizeof(uint16_t) * zs.size(), "zone schedule"},
         };
         for (auto &a : za)
-            if (a.bytes > 0 && (e = cudaMalloc(a.ptr, a.bytes)) != cudaSuccess) return bail(cuda_fail(h, e, a.what));
+            if ((e = cudaMalloc(a.ptr, a.bytes)) != cudaSuccess) return bail(cuda_fail(h, e, a.what));
+        // the bounds' list and tables; without room for them every trial is decided by the elimination
+        if (well && (cudaMalloc((void **)&h->zone_open, sizeof(unsigned) * 4 * (size_t)h->nblk_total) != cudaSuccess ||
+                     cudaMalloc(&h->btab, h->tsize * 8 * 48 * (size_t)p->n_orient) != cudaSuccess)) {
+            cudaGetLastError();
+            if (h->zone_open) cudaFree(h->zone_open);
+            h->zone_open = nullptr;
+            h->btab = nullptr;
+        }
         if ((e = cudaMemcpy(h->zone_sched, zs.data(), sizeof(uint16_t) * zs.size(), cudaMemcpyHostToDevice)) !=
             cudaSuccess)
             return bail(cuda_fail(h, e, "zone schedule upload"));
@@ -2038,7 +2046,6 @@ hmc_status adj_alloc(hmc_handle *h, int steps, int ck) {
         {&A.fcell, h->tsize * 24 * (size_t)R.nblk, "cell contributions"},
         {(void **)&A.partials, sizeof(double) * 10 * (size_t)A.nctas, "adjoint partials"},
         {(void **)&A.grad, sizeof(double) * 13, "gradient"},
-        {&A.lsum, nb, "sum of lambdas"}, {&A.lerr, h->tsize == 4 ? nb : 0, "sum of lambdas"},
         {(void **)&A.reps0, sizeof(hmc::Replica), "adjoint descriptor"},
         {(void **)&A.st0, sizeof(DevState), "adjoint state"},
     };
@@ -2050,6 +2057,8 @@ hmc_status adj_alloc(hmc_handle *h, int steps, int ck) {
             return cuda_fail(h, e, a.what);
         }
     }
+    A.lsum = A.w;
+    A.lerr = h->tsize == 4 ? seg_ptr(h, A.w, 1) : nullptr;
     A.steps = steps;
     A.ck = ck;
     A.nseg = nseg;
