@@ -462,10 +462,9 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_mpm_block(MpmArgs<fl
 #pragma unroll
     for (int m = 0; m < PER; ++m) node[m] = B.node(R, tid + m * THREADS);
     float eb[6], un[3] = {0.f, 0.f, 0.f}, vold[3] = {0.f, 0.f, 0.f};
-    // (written only by the end of a Monte Carlo step, which lets no kernel start early; read after the
-    // wait, through the replica's pointer, it came last of all loads: 32^3 3.7 -> 3.5 us)
-    load_ebar<float>(R.st, eb);
+    const DevState *st = R.st;   // (looked up behind the wait, the mean strain came last: 32^3 3.7 -> 3.5 us)
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    load_ebar<float>(st, eb);
     const uint4 sp = need ? a.spins[at] : make_uint4(0, 0, 0, 0);
     if (own) {
 #pragma unroll

@@ -342,11 +342,13 @@ __device__ __forceinline__ void fx_put(FxHalf *xy, FxHalf *ze, int t, const doub
     ze[t] = FxHalf{dfix<3>(u[2], E), (ll)E};
 }
 
-__device__ __forceinline__ void fx_mean(FxMean &m, const DevState *st) {   // by one thread
+// By one thread, while the kernel before may still run: from L2, since the SM's L1 may hold an older line
+// (the end of a Monte Carlo step writes the mean strain, fences and lets no kernel start before it is over).
+__device__ __forceinline__ void fx_mean(FxMean &m, const DevState *st) {
     double e[6];
     int E = 0;
     for (int i = 0; i < 6; ++i) {
-        e[i] = st->ebar[i];
+        e[i] = __ldcg(st->ebar + i);
         E = max(E, dexp(e[i]));
     }
     for (int i = 0; i < 3; ++i) m.eb[i] = FxHalf{dfix<8>(e[2 * i], E), dfix<8>(e[2 * i + 1], E)};

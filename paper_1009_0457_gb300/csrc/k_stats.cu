@@ -139,8 +139,7 @@ __global__ void __launch_bounds__(WIDE ? BLOCK_THREADS : STRESS_THREADS, sizeof(
     const int t0 = (blockIdx.x - R.cta_off) * BLOCK_THREADS;
     Acc7<T> acc;
     acc.zero();
-    T eb[6];
-    load_ebar<T>(R.st, eb);   // written only by the end of a step, which lets no kernel start early
+    const DevState *st = R.st;
     const int nbx = R.nbx, nby = R.nby, nbz = R.nbz;
     const T *u = a.u + 3 * R.blk_off;
     T *sig = a.sig + 48ll * R.blk_off;
@@ -167,6 +166,8 @@ __global__ void __launch_bounds__(WIDE ? BLOCK_THREADS : STRESS_THREADS, sizeof(
     uint4 spn = make_uint4(0, 0, 0, 0);
     int blk = t0 + threadIdx.x;
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    T eb[6];
+    load_ebar<T>(st, eb);
     if (blk < R.nblk) load_cell(blk, un, spn);
 #pragma unroll 1
     for (int c8 = 0; c8 < (WIDE ? 1 : STRESS_CELLS); ++c8) {
@@ -252,12 +253,13 @@ __global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(4 * SPLIT_CELLS)
     const int nblk = R.nblk, tile0 = (tile - R.cta_off) * BLOCK_THREADS, t0 = tile0 + part * SPLIT_CELLS;
     const int nbx = R.nbx, nby = R.nby, nbz = R.nbz;
     const double *u = a.u + 3 * R.blk_off;
-    double eb[6];
-    load_ebar<double>(R.st, eb);   // written only by the end of a step, which lets no kernel start early
+    const DevState *st = R.st;
     const int tid = threadIdx.x, cell = tid >> 2, b = tid & 1, c = tid >> 1 & 1, blk = t0 + cell;
     const bool live = blk < nblk;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (live) {
+        double eb[6];
+        load_ebar<double>(st, eb);
         const uint4 sp = a.spins[R.blk_off + blk];
         double uc[8][3];
         const int bx = blk % nbx, rr = blk / nbx, by = rr % nby, bz = rr / nby;
@@ -299,13 +301,13 @@ __global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(4 * SPLIT_CELLS)
             }
             const double e[6] = {eb[0] + gx[0], eb[1] + gy[i][1], eb[2] + gz[i][2], eb[3] + (gz[i][1] + gy[i][2]),
                                  eb[4] + (gz[i][0] + gx[2]), eb[5] + (gy[i][0] + gx[1])};
-            double st[6], w = 0.0;
-            hooke21<double>(row.v, e, st);
+            double sg[6], w = 0.0;
+            hooke21<double>(row.v, e, sg);
             double(&out)[7][SPLIT_CELLS + 1] = pts[local_slot(i + 2 * b + 4 * c)];
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
-                out[k][cell] = st[k];
-                w = rfma(st[k], e[k], w);
+                out[k][cell] = sg[k];
+                w = rfma(sg[k], e[k], w);
             }
             out[6][cell] = 0.5 * w;
         }
@@ -345,7 +347,8 @@ __device__ __forceinline__ double lanes_sum(double x) {
 // 15 us; 4 us).
 // after_sweeps: the kernel before this one is the black half sweep, which lets this one start only
 // when the stress pass has finished: all but the results' stores runs beside it.  This kernel lets
-// none start early, so that the step counter and the mean strain may be read before waiting.
+// none start early and fences its stores, so that the FP64 step may read the mean strain, from L2,
+// before it waits.
 __global__ void __launch_bounds__(224) k_end_mcs(const Replica *reps, int nrep, int gmax, double *partials, int nctas,
                                                   int update_strain, int advance, int after_sweeps) {
     __shared__ double tot[7];
@@ -362,16 +365,16 @@ __global__ void __launch_bounds__(224) k_end_mcs(const Replica *reps, int nrep, 
     // the update's operands, loaded while the sums are formed (lane c: component c)
     const int c = lane < 6 ? lane : 0;
     double sr[6], axN = 0, axNs = 0, axB = 0, axNB = 1, eps0 = 0, sig0 = 0, ebar = 0;
-    if (i == 0) {
+    if (i == 0) {   // (from L2: the SM's L1 may hold a line from before the last end of a step)
 #pragma unroll
-        for (int j = 0; j < 6; ++j) sr[j] = st->sr[6 * c + j];
-        axN = st->axN[c];
-        axNs = st->axNs[c];
-        axB = st->axB[c];
-        axNB = st->axNB;
-        eps0 = st->eps0;
-        sig0 = st->sig0;
-        ebar = st->ebar[c];
+        for (int j = 0; j < 6; ++j) sr[j] = __ldcg(st->sr + 6 * c + j);
+        axN = __ldcg(st->axN + c);
+        axNs = __ldcg(st->axNs + c);
+        axB = __ldcg(st->axB + c);
+        axNB = __ldcg(&st->axNB);
+        eps0 = __ldcg(&st->eps0);
+        sig0 = __ldcg(&st->sig0);
+        ebar = __ldcg(st->ebar + c);
     }
     double s = 0.0;
     for (int p = grp + G * lane; p < R.ncta; p += 32 * G) s += __ldcg(partials + 7ll * (R.cta_off + p) + i);
@@ -434,6 +437,7 @@ __global__ void __launch_bounds__(224) k_end_mcs(const Replica *reps, int nrep, 
         if (advance) st->mcs += 1;
         *arrive = 0u;   // ready for the next launch
     }
+    __threadfence();   // the next kernel may read the mean strain before it waits
 }
 
 // Upload check: flag any orientation index >= Q (8 indices per thread, 16 B loads).

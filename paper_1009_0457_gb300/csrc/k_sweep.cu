@@ -371,14 +371,10 @@ __global__ void __launch_bounds__(CTA, flat_min_ctas<T, MODE, RECOMP, CTA>())
     if (t0 >= R.nblk) return;  // the empty part of a replica's last tile
     const int blk = t0 + tid;  // block within the replica
     const bool live = blk < R.nblk;
-    // What the kernel before this one does not write comes first: the block's place and its random
-    // numbers (the step counter is advanced only by the end of a step, which lets no kernel start early)
+    // the tables' part comes before the wait: the block's place and where its replica's state is
     int bx = 0, by = 0, bz = 0;
-    uint2 rnd[4];
-    if (live) {
-        block_xyz(R, blk, bx, by, bz);
-        block_draws<COL, ONE>(R, a.rkey, a.trial, bx, by, bz, R.st->mcs, rnd);
-    }
+    if (live) block_xyz(R, blk, bx, by, bz);
+    const DevState *st = R.st;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (COL == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (ELASTIC) {
@@ -407,6 +403,7 @@ __global__ void __launch_bounds__(CTA, flat_min_ctas<T, MODE, RECOMP, CTA>())
     uint16_t out[4] = {0, 0, 0, 0}, qn[4] = {0, 0, 0, 0};
     uint32_t pend = 0;   // elastic modes: slots with a listed trial
     T sg[6][4];          // recompute mode: strain of the colour's four sites
+    uint2 rnd[4];
     int dE[4] = {0, 0, 0, 0};
     if (live) {
         const int nbx = R.nbx, nby = R.nby, nbz = R.nbz;
@@ -424,6 +421,7 @@ __global__ void __launch_bounds__(CTA, flat_min_ctas<T, MODE, RECOMP, CTA>())
         N[3] = q2[2 * (blk + (by == nby - 1 ? -(nby - 1) * sxy : sxy)) + oc];
         N[4] = q2[2 * (blk + (bz == 0 ? (nbz - 1) * sxz : -sxz)) + oc];
         N[5] = q2[2 * (blk + (bz == nbz - 1 ? -(nbz - 1) * sxz : sxz)) + oc];
+        block_draws<COL, ONE>(R, a.rkey, a.trial, bx, by, bz, st->mcs, rnd);
         uint16_t q[4];
         block_trials<COL>(a.trial, a.nq, mine, O, N, rnd, q, qn, dE);
         // recompute mode: the cell's displacement gradients, formed at the first listed trial
