@@ -32,7 +32,7 @@
 // barrier per plane.
 // What bounds it: 244 registers leave eight warps per SM, which issue 36 % of the cycles (the
 // busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
-// 32^3 8.2 (70), 100^3 52 (308), 128^3 102 (420), 256^3 709 (3330).
+// 32^3 8.2 (70), 100^3 52 (308), 128^3 102 (420), 256^3 717 (3330).
 #include "hmc_device.cuh"
 
 namespace hmc {
@@ -342,17 +342,28 @@ __device__ __forceinline__ void fx_put(FxHalf *xy, FxHalf *ze, int t, const doub
     ze[t] = FxHalf{dfix<3>(u[2], E), (ll)E};
 }
 
-// By one thread, while the kernel before may still run: from L2, since the SM's L1 may hold an older line
-// (the end of a Monte Carlo step writes the mean strain, fences and lets no kernel start before it is over).
+// Behind the wait: the end of a Monte Carlo step writes the mean strain, and only the wait makes it
+// visible.  By one thread in the march (by a warp there, other code of the loop came out slower: 102 ->
+// 108 us at 128^3) ...
 __device__ __forceinline__ void fx_mean(FxMean &m, const DevState *st) {
     double e[6];
     int E = 0;
     for (int i = 0; i < 6; ++i) {
-        e[i] = __ldcg(st->ebar + i);
+        e[i] = st->ebar[i];
         E = max(E, dexp(e[i]));
     }
     for (int i = 0; i < 3; ++i) m.eb[i] = FxHalf{dfix<8>(e[2 * i], E), dfix<8>(e[2 * i + 1], E)};
     m.e = E;
+}
+// ... and by the first warp, a lane a component, in a block, where it lies in the chain of the
+// step (8.18 us at 32^3, 8.37 by one thread)
+__device__ __forceinline__ void fx_mean_warp(FxMean &m, const DevState *st) {
+    const int lane = threadIdx.x;
+    const double e = lane < 6 ? st->ebar[lane] : 0.0;
+    const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)dexp(e));
+    const ll x = dfix<8>(e, E);
+    if (lane < 6) (lane & 1 ? m.eb[lane >> 1].b : m.eb[lane >> 1].a) = x;
+    if (lane == 0) m.e = E;
 }
 
 // a cell: its corners lie at n0 and n1 (lower and upper plane; for a quarter near and far), dy apart in
@@ -494,11 +505,11 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
                 if (ncol[m] >= 0) fx_put(sm.uxy[b], sm.uze[b], tid + m * MPM_THREADS, pl[m]);
         };
         int b0 = 0, b1 = 1, b2 = 2, fb = 0;
-        if (tid == 0) fx_mean(sm.m, R.st);
-        // nothing above reads what the kernels before this one write (the mean strain comes from the end of a
-        // Monte Carlo step, which lets no kernel start early): 1.2 us a step against a wait ahead
+        const DevState *st = R.st;
+        // nothing above reads what the kernels before this one write: 1.2 us a step against a wait ahead
         // of the range's look-ups
         asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (tid == 0) fx_mean(sm.m, st);
         fetch(k0 - 1);
         store(b0);
         fetch(k0);
@@ -594,10 +605,9 @@ __global__ void __launch_bounds__(CELLS *SPLIT, 1) k_mpm_fixed_block(MpmArgs<dou
     long long node[PER];
 #pragma unroll
     for (int m = 0; m < PER; ++m) node[m] = B.node(R, tid + m * CELLS);
-    // (the mean strain is written only by the end of a Monte Carlo step, which lets no kernel start
-    // early; converted behind the wait 32^3 took 8.55 us instead of 8.2)
-    if (tid == 0) fx_mean(sm.m, R.st);
+    const DevState *st = R.st;
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (tid < 32) fx_mean_warp(sm.m, st);
     const uint4 sp = need ? a.spins[cat] : make_uint4(0, 0, 0, 0);
     double uold[3] = {0, 0, 0}, vold[3] = {0, 0, 0};
     if (own) {

@@ -346,9 +346,9 @@ __device__ __forceinline__ double lanes_sum(double x) {
 // chain: 20 instead of about 150 of them (the 250-thread tree and the update by one thread took
 // 15 us; 4 us).
 // after_sweeps: the kernel before this one is the black half sweep, which lets this one start only
-// when the stress pass has finished: all but the results' stores runs beside it.  This kernel lets
-// none start early and fences its stores, so that the FP64 step may read the mean strain, from L2,
-// before it waits.
+// when the stress pass has finished: all but the results' stores runs beside it.  What it reads ahead of
+// its wait comes from kernels that were over before the black half sweep passed its own: the stress
+// pass and the end of the step before, never the kernel that it overlaps.
 __global__ void __launch_bounds__(224) k_end_mcs(const Replica *reps, int nrep, int gmax, double *partials, int nctas,
                                                   int update_strain, int advance, int after_sweeps) {
     __shared__ double tot[7];
@@ -437,7 +437,6 @@ __global__ void __launch_bounds__(224) k_end_mcs(const Replica *reps, int nrep, 
         if (advance) st->mcs += 1;
         *arrive = 0u;   // ready for the next launch
     }
-    __threadfence();   // the next kernel may read the mean strain before it waits
 }
 
 // Upload check: flag any orientation index >= Q (8 indices per thread, 16 B loads).
