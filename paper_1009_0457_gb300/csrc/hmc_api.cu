@@ -78,7 +78,6 @@ struct hmc_handle {
     void *sig = nullptr, *ctab = nullptr, *wtab = nullptr, *atab = nullptr;
     float *cubw = nullptr;                // FP32 MPM step: Voigt weights of two crystal axes per orientation
     int2 *cfix = nullptr;                 // FP64 MPM step: stiffness rows in fixed point
-    int cexp = 0;
     // 27-point zone (HMC_ELASTIC_ZONE1): trial list, start-of-step spins, element tables, schedule
     uint4 *zone_work = nullptr, *snap = nullptr;
     unsigned *zone_count = nullptr;       // listed trials, trials that the bounds leave open
@@ -227,8 +226,9 @@ std::vector<T> pack_ctab(const std::vector<double> &Cv, int Q) {
 
 // The stiffness rows as 64-bit integers C' 2^cexp with every row's absolute sum below 2^63 (the
 // bound the fixed-point step's accumulators are laid out for), each split into a signed low and a
-// high 32-bit half.
-std::vector<int2> pack_cfix(const std::vector<double> &Cv, int Q, int &cexp) {
+// high 32-bit half.  cexp depends on the orientations, so it is handed to the kernels in the table,
+// behind the first row's entries: captured launches replayed after new orientations use the new one.
+std::vector<int2> pack_cfix(const std::vector<double> &Cv, int Q) {
     double top = 0;
     for (size_t r = 0; r < (size_t)Q * 6; ++r) {
         double s = 0;
@@ -237,7 +237,7 @@ std::vector<int2> pack_cfix(const std::vector<double> &Cv, int Q, int &cexp) {
     }
     int er = 0;
     std::frexp(top * (1.0 + 1e-9), &er);   // top < 2^er
-    cexp = 63 - er;
+    const int cexp = 63 - er;
     std::vector<int2> out((size_t)Q * 24, make_int2(0, 0));
     for (int q = 0; q < Q; ++q) {
         int n = 0;
@@ -248,6 +248,7 @@ std::vector<int2> pack_cfix(const std::vector<double> &Cv, int Q, int &cexp) {
                 out[(size_t)q * 24 + n++] = make_int2(lo, (int)((v - lo) >> 32));
             }
     }
+    out[hmc::CFIX_EXP] = make_int2(cexp, 0);
     return out;
 }
 
@@ -297,7 +298,6 @@ hmc::MpmArgs<T> mpm_args(hmc_handle *h, const void *u_in, void *u_out, void *v) 
     a.v = static_cast<T *>(v);
     a.cubw = h->cubw;               // FP32 step: cubic form of Hooke's law
     a.cfix = h->cfix;               // FP64 step: stiffness in fixed point
-    a.cexp = h->cexp;
     a.cub[0] = (float)h->p.c12;
     a.cub[1] = (float)(2.0 * h->p.c44);
     a.cub[2] = (float)h->p.c44;
@@ -1369,7 +1369,7 @@ hmc_status hmc_set_orientations(hmc_handle *h, const double *euler, const uint16
         auto c = pack_ctab<double>(h->Cv, Q);
         auto w = pack_wtab<double>(h->A, Q);
         auto ax = pack_atab<double>(h->A, Q);
-        auto cf = pack_cfix(h->Cv, Q, h->cexp);
+        auto cf = pack_cfix(h->Cv, Q);
         HMC_CK(h, cudaMemcpy(h->cfix, cf.data(), cf.size() * sizeof(int2), cudaMemcpyHostToDevice), "table upload");
         HMC_CK(h, cudaMemcpy(h->ctab, c.data(), c.size() * sizeof(double), cudaMemcpyHostToDevice), "table upload");
         HMC_CK(h, cudaMemcpy(h->wtab, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice), "table upload");

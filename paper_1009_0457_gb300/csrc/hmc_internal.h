@@ -19,7 +19,7 @@
 //   cubw    float[Q][12]        FP32 MPM step: the Voigt weights (x^2, y^2, z^2, yz,
 //                               xz, xy) of the first two crystal axes a_0, a_1
 //   cfix    int2[Q][24]         FP64 MPM step: C'(q) as 64-bit integers C' 2^cexp, each as
-//                               signed 32-bit halves (x low, y high)
+//                               signed 32-bit halves (x low, y high); cexp behind the first row's 21 entries
 #pragma once
 
 #include <cuda_runtime.h>
@@ -112,13 +112,15 @@ struct MpmArgs {
     const float *cubw;       // FP32 step: Voigt weights of two crystal axes per orientation (12 each)
     float cub[4];            // FP32 step: C12, 2 C44, C44 and C11 - C12 - 2 C44
     const int2 *cfix;        // FP64 step: rotated stiffness in fixed point, 24 entries per orientation (21 used)
-    int cexp;                // ... entry = round(C' 2^cexp), x the signed low half, y the high half
+                             // ... entry = round(C' 2^cexp), x the signed low half, y the high half; cexp
+                             // itself is entry CFIX_EXP
     int nq;                  // orientations (the FP32 step stages cubw in shared memory up to MPM_STAB_MAX)
     T dt, dt_over_m, keep;   // keep = 1 - damping
     T ukeep;                 // u_out = ukeep u + dt v: 1, or 1 - damping in the adjoint's reverse step
     int grid;                // CTAs
 };
 
+constexpr int CFIX_EXP = 21;         // place of cexp (x) in cfix, behind the first orientation's entries
 constexpr int MPM_STAB_MAX = 1024;   // orientations whose FP32 table the MPM step holds in shared memory
 constexpr int MPM_STAB_BLOCK = 256;  // ... in the block form
 

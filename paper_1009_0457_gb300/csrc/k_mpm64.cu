@@ -32,7 +32,7 @@
 // barrier per plane.
 // What bounds it: 244 registers leave eight warps per SM, which issue 36 % of the cycles (the
 // busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
-// 32^3 8.2 (70), 100^3 52 (308), 128^3 102 (420), 256^3 717 (3330).
+// 32^3 8.2 (70), 100^3 52 (308), 128^3 102 (420), 256^3 711 (3330).
 #include "hmc_device.cuh"
 
 namespace hmc {
@@ -428,7 +428,7 @@ struct FxUpdate {
     double fscale, dt, keep, ukeep;   // fscale = -dt / (32 m)
     int cexp, fexp;
     __device__ __forceinline__ explicit FxUpdate(const MpmArgs<double> &a)
-        : fscale(-a.dt_over_m * 0.03125), dt(a.dt), keep(a.keep), ukeep(a.ukeep), cexp(a.cexp) {
+        : fscale(-a.dt_over_m * 0.03125), dt(a.dt), keep(a.keep), ukeep(a.ukeep), cexp(__ldg(&a.cfix[CFIX_EXP].x)) {
         // the force integers of exponent E are 2^(E - cexp - 1013) of the FP32 step's units
         fexp = dexp(fscale) ? dexp(fscale) - cexp - 1013 : -10000;   // (subnormal: the general form)
     }
