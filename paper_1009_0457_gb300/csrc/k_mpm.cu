@@ -539,13 +539,17 @@ Form form_of(int variant, int nq) {
 
 }  // namespace
 
+// The limit of a kernel is the process's, so it is only ever set to the most that the kernel is launched with,
+// each time to the same value: a launch of another thread's handle may come at any moment.
 cudaError_t mpm_prepare() {
-    for (int v = 0; v < mpm_nvariants(true); ++v)
-        for (int nq : {MPM_STAB_BLOCK, MPM_STAB_MAX, MPM_STAB_MAX + 1}) {
+    for (int v = 0; v < mpm_nvariants(true); ++v) {
+        const int most = mpm_is_block(v) ? MPM_STAB_BLOCK : MPM_STAB_MAX;   // orientations staged; beyond: none
+        for (int nq : {most, MPM_STAB_MAX + 1}) {
             const Form f = form_of(v, nq);
             const cudaError_t e = cudaFuncSetAttribute(f.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem);
             if (e != cudaSuccess) return e;
         }
+    }
     return cudaSuccess;
 }
 
