@@ -1659,7 +1659,13 @@ hmc_status hmc_mc_sweeps(hmc_handle *h, int32_t n_mcs, int64_t *accepted) {
                 return cuda_fail(h, e, "capture");
             }
             if (e2 != cudaSuccess) return cuda_fail(h, e2, "end capture");
+            // The graph of several steps may come long after the first call, which a caller makes before a
+            // capture of its own: instantiating is then refused by default, though it touches no captured
+            // stream
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
             e = cudaGraphInstantiate(&gexec, g, 0);
+            cudaThreadExchangeStreamCaptureMode(&mode);
             cudaGraphDestroy(g);
             if (e != cudaSuccess) {
                 gexec = nullptr;
