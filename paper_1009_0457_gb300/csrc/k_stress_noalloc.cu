@@ -54,18 +54,13 @@ struct NoallocArgs {
     long long nblk, n_sites;
 };
 
+// Knuth's TwoSum: hi + x = s + its error exactly, whatever the signs and sizes (Kahan's sum, three additions
+// shorter, loses bits where terms cancel: 1e-9 of them instead of 1e-15).
 __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x) {
     const float s = hi + x;
     const float bb = s - hi;
     lo += (hi - (s - bb)) + (x - bb);
     hi = s;
-}
-
-// Compensated running sum (Kahan 1965): four additions a term against TwoSum's seven.
-__device__ __forceinline__ void kahan_add(float &s, float &c, float x) {
-    const float y = __fsub_rn(x, c), t = __fadd_rn(s, y);
-    c = __fsub_rn(__fsub_rn(t, s), y);
-    s = t;
 }
 
 // a point's full 6x6 stiffness, 16-byte loads where the table allows them
@@ -101,7 +96,7 @@ __device__ __forceinline__ void load_c36(const float *p, float (&c)[36]) {
 //
 // What bounds it: the L1 data pipe (76 % of its wavefronts), most of it the divergent
 // reloads of the 144-byte rows in cells that a grain boundary cuts.  Measured at 256^3, 419
-// voxels a grain: 440 us a call before, 266 us with the coalesced stores, 166 us with four
+// voxels a grain: 440 us a call before, 266 us with the coalesced stores, 165 us with four
 // cells a thread and the Gray-code order (floor of its bytes: 68 us).
 //
 // CELLS: blocks of a CTA's 256 that a thread takes in turn.  Four on large grids: the
@@ -187,9 +182,9 @@ __global__ void __launch_bounds__(NOALLOC_THREADS / CELLS, 2 * CELLS) k_stress_n
                         for (int j = 0; j < 6; ++j) acc += c[6 * i + j] * e[j];
                         out[6 * lx + i] = acc;
                         w += acc * e[i];
-                        kahan_add(hi[i], lo[i], acc);
+                        two_sum_add(hi[i], lo[i], acc);
                     }
-                    kahan_add(hi[6], lo[6], 0.5f * w);
+                    two_sum_add(hi[6], lo[6], 0.5f * w);
                 }
 #pragma unroll
                 for (int j = 0; j < 3; ++j)
@@ -216,8 +211,6 @@ __global__ void __launch_bounds__(NOALLOC_THREADS / CELLS, 2 * CELLS) k_stress_n
             }
         }
     }
-#pragma unroll
-    for (int i = 0; i < 7; ++i) lo[i] = -lo[i];   // Kahan's c is what the sum still owes
 #pragma unroll
     for (int off = 16; off; off >>= 1)
 #pragma unroll
