@@ -34,6 +34,7 @@
 // busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
 // 32^3 8.2 (70), 100^3 52 (308), 128^3 102 (420), 256^3 711 (3330).
 #include "hmc_device.cuh"
+#include "hmc_fixed.h"
 
 namespace hmc {
 
@@ -275,16 +276,6 @@ struct Fx3 {
     ll v[3];
     int e;
 };
-
-// x / 2^n to the nearest, halves away from zero (a shift of 62 or more leaves nothing of |x| < 2^62.3)
-__device__ __forceinline__ ll rshift(ll x, int n) {
-    if (n <= 0) return x;
-    if (n > 61) return 0;
-    return (x + (1ll << (n - 1)) + (x >> 63)) >> n;
-}
-
-// whether a sum of up to eight integers, whose high words / 8 sum to t, stays within 63 bits
-__device__ __forceinline__ bool fits63(int t) { return (unsigned)(t + (1 << 28)) <= (1u << 29) - 8u; }
 
 // The sum of N terms x[i] 2^e[i] per direction.  With one exponent it is exact; otherwise the terms
 // are aligned to the largest exponent, and three bits above it where the sum would leave 63 bits.
