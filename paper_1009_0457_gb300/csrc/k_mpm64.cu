@@ -7,32 +7,37 @@
 // the stiffness per point.  So a cell is computed in integers that share one exponent, and
 // only the node update (v, u) stays in FP64.
 //
-// Numbers.  E = the largest biased exponent among the cell's 24 corner displacements and the
-// mean strain.  A displacement is held as m * 2^3 (m its 53-bit mantissa) aligned to E, so
-// |U| < 2^56 and the largest displacements keep three bits below their own last one.  The
-// gradients (16 x interpolated differences) and the strains (two gradient entries and the mean
-// strain) are exact integer sums below 2^62.6; strains are taken / 8 (< 2^59.6) and split into
-// signed 32-bit halves.  The stiffness is held as integers C 2^cexp with row sums below 2^63,
+// Numbers.  A node's displacement is held as one integer m * 2^3 (m the 53-bit mantissa) and one exponent per
+// component.  A cell aligns each component's eight values to the largest exponent among them and takes
+// the differences against its lowest corner, so that a displacement that all corners share costs nothing;
+// what the alignment drops is below 2^-55 of the component's largest value where its exponents differ, and
+// the differences are then of that size.  The cell's exponent F is the smallest at which all differences of all
+// components stay below 2^56, and at least the mean strain's; each component is shifted to F, up
+// exactly or down to the nearest.  The gradients (16 x interpolated differences) and the strains (two
+// gradient entries and the mean strain) are exact integer sums below 2^62.6; strains are taken / 8 (< 2^59.6)
+// and split into signed 32-bit halves.  The stiffness is held as integers C 2^cexp with row sums below 2^63,
 // split the same way; sigma = round(C e / 2^64) drops only the product of the two low halves
 // (< 2^62, below the rounding) and stays below 2^58.6; the sums behind it stay below 2^63.  The
 // traction sums (< 2^59.6) are exact, their first 3/1 sums (< 2^61.6) are taken / 8, the second
-// (< 2^60.6) and a corner's force (< 2^62.2) are exact again.  Each rounding is far below the
-// 2^-53 that every intermediate of an FP64 evaluation carries, and the corner forces are
+// (< 2^60.6) and a corner's force (< 2^62.2) are exact again.  Each rounding is below the 2^-53 of the
+// cell's largest strain, or stress, that an FP64 evaluation carries for it; a component of strain or
+// stress far below the largest of its cell has that absolute error, not a relative one of its own (FP64
+// keeps one where the stiffness does not couple the components, as in an aligned crystal).  The corner forces are
 // +-X +-Y +-Z of the same integers, so a cell's forces sum to exactly zero whatever was rounded.
 // A node's force is the sum of its eight cells' integers: exact when their exponents agree and
 // the sum cannot leave 63 bits (both are tested), otherwise aligned to the largest exponent with
-// symmetric rounding.  A cell with a non-finite corner gets E = 2047 and its nodes NaN.
+// symmetric rounding.  A cell with a non-finite corner gets F = 2047 and its nodes NaN.
 // A displacement below 2^-1022 (subnormal) counts as zero.
 // Against an 80-bit reference (20x24x28 points, 100 steps) the velocity's relative error is
 // 5.6e-15 and the displacement's 6.8e-16; FP64 arithmetic gave 1.05e-14 and 7.6e-16.
 //
 // Tiling, scheduling and the march in z are those of the FP32 step (k_mpm.cu); nodes and forces
-// are kept in shared memory as two arrays of 16-byte halves, (x, y) and (z, exponent), so that
+// are kept in shared memory as two arrays of 16-byte halves, (x, y) and (z, exponents), so that
 // consecutive lanes read consecutive 16 bytes.  The forces are double-buffered, which leaves one
 // barrier per plane.
-// What bounds it: 244 registers leave eight warps per SM, which issue 36 % of the cycles (the
+// What bounds it: 246 registers leave eight warps per SM, which issue 36 % of the cycles (the
 // busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
-// 32^3 8.2 (70), 100^3 52 (308), 128^3 102 (420), 256^3 711 (3330).
+// 32^3 8.2 (70), 100^3 50 (308), 128^3 98 (420), 256^3 681 (3330).
 #include "hmc_device.cuh"
 #include "hmc_fixed.h"
 
@@ -326,11 +331,11 @@ __device__ __forceinline__ Fx3 fx_sum(const ll (&x)[3][N], const int (&e)[N]) {
     return r;
 }
 
-// a node's displacement into shared memory, its components aligned to the largest of them
+// a node's displacement into shared memory: each component's 2^3 m and their exponents, 16 bits each
 __device__ __forceinline__ void fx_put(FxHalf *xy, FxHalf *ze, int t, const double (&u)[3]) {
-    const int E = max(dexp(u[0]), max(dexp(u[1]), dexp(u[2])));
-    xy[t] = FxHalf{dfix<3>(u[0], E), dfix<3>(u[1], E)};
-    ze[t] = FxHalf{dfix<3>(u[2], E), (ll)E};
+    const int ex = dexp(u[0]), ey = dexp(u[1]), ez = dexp(u[2]);
+    xy[t] = FxHalf{dfix<3>(u[0], ex), dfix<3>(u[1], ey)};
+    ze[t] = FxHalf{dfix<3>(u[2], ez), ((ll)ez << 32) | (unsigned)(ex | ey << 16)};
 }
 
 // Behind the wait: the end of a Monte Carlo step writes the mean strain, and only the wait makes it
@@ -358,10 +363,12 @@ __device__ __forceinline__ void fx_mean_warp(FxMean &m, const DevState *st) {
 }
 
 // a cell: its corners lie at n0 and n1 (lower and upper plane; for a quarter near and far), dy apart in
-// y; returns its exponent
+// y; u becomes their displacements against the cell's lowest corner's (ref: its place among them) at the
+// cell's exponent, which is returned.  (That corner's zeros spare the march more than the differences and
+// the components' own exponents cost: with one exponent and no differences 256^3 took 707 us, now 681.)
 __device__ __forceinline__ int fx_corners(const FxHalf *xy0, const FxHalf *ze0, const FxHalf *xy1, const FxHalf *ze1,
-                                          int dy, const FxMean &m, ll (&u)[8][3], ll (&eb)[6]) {
-    int ne[8], E = m.e;
+                                          int dy, int ref, const FxMean &m, ll (&u)[8][3], ll (&eb)[6]) {
+    unsigned exy[8], ez[8], mxy = 0, mz = 0;
 #pragma unroll
     for (int n = 0; n < 8; ++n) {
         const int o = (n & 1) + (n & 2 ? dy : 0);
@@ -369,23 +376,47 @@ __device__ __forceinline__ int fx_corners(const FxHalf *xy0, const FxHalf *ze0, 
         u[n][0] = p.a;
         u[n][1] = p.b;
         u[n][2] = q.a;
-        ne[n] = (int)q.b;
-        E = max(E, ne[n]);
+        exy[n] = (unsigned)q.b;
+        ez[n] = (unsigned)(q.b >> 32);
+        mxy = __vmaxu2(mxy, exy[n]);
+        mz = max(mz, ez[n]);
     }
 #pragma unroll
     for (int n = 0; n < 8; ++n) {
-        const int s = min(E - ne[n], 63);
-#pragma unroll
-        for (int d = 0; d < 3; ++d) u[n][d] >>= s;
+        const unsigned t = __vminu2(mxy - exy[n], 0x003f003fu);
+        u[n][0] >>= t & 0xffffu;
+        u[n][1] >>= t >> 16;
+        u[n][2] >>= min(mz - ez[n], 63u);
     }
-    const int se = min(E - m.e, 63);
+    const int E[3] = {(int)(mxy & 0xffffu), (int)(mxy >> 16), (int)mz};
+    int F = m.e;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const ll lo = ref & 2 ? u[2][d] : u[0][d], hi = ref & 2 ? u[6][d] : u[4][d], r = ref & 4 ? hi : lo;
+        ll any = 0;
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            u[n][d] -= r;
+            any |= u[n][d] ^ (u[n][d] >> 63);
+        }
+        F = max(F, E[d] + 8 - __clzll(any));
+    }
+    if (max(max(E[0], E[1]), E[2]) == 2047) F = 2047;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const int l = min(max(E[d] - F, 0), 63), r = min(max(F - E[d], 0), 63);
+        const ll half = r > 0 ? 1ll << (r - 1) : 0ll;
+#pragma unroll
+        for (int n = 0; n < 8; ++n) u[n][d] = (ll)(((unsigned long long)u[n][d] << l) + half) >> r;
+    }
+    const int se = min(F - m.e, 63);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const FxHalf t = m.eb[i];
         eb[2 * i] = t.a >> se;
         eb[2 * i + 1] = t.b >> se;
     }
-    return E;
+    return F;
 }
 
 // the four cells (i-1, j-1), (i, j-1), (i-1, j), (i, j) of one plane, W cells a row, on their common
@@ -530,7 +561,7 @@ __global__ void __launch_bounds__(MPM_THREADS, 1) k_mpm_fixed(MpmArgs<double> a)
             if (more) fetch(kk + 2);
             if (need) {
                 ll u[8][3], eb[6], f[8][3];
-                const int E = fx_corners(sm.uxy[b0] + nd, sm.uze[b0] + nd, sm.uxy[b1] + nd, sm.uze[b1] + nd, P, sm.m, u, eb);
+                const int E = fx_corners(sm.uxy[b0] + nd, sm.uze[b0] + nd, sm.uxy[b1] + nd, sm.uze[b1] + nd, P, 0, sm.m, u, eb);
                 fx_cell(u, eb, sp, a.cfix, f);
 #pragma unroll
                 for (int n = 0; n < 8; ++n) {
@@ -619,7 +650,7 @@ __global__ void __launch_bounds__(CELLS *SPLIT, 1) k_mpm_fixed_block(MpmArgs<dou
     if (some) {
         ll u[8][3], eb[6], f[8 / SPLIT][3];
         const int nd = need ? ci + P * cj + PP * ck : 0, n0 = nd + (b ? P : 0) + (c ? PP : 0), dz = c ? -PP : PP;
-        const int E = fx_corners(sm.uxy + n0, sm.uze + n0, sm.uxy + n0 + dz, sm.uze + n0 + dz, b ? -P : P, sm.m, u, eb);
+        const int E = fx_corners(sm.uxy + n0, sm.uze + n0, sm.uxy + n0 + dz, sm.uze + n0 + dz, b ? -P : P, 2 * b + 4 * c, sm.m, u, eb);
         if constexpr (SPLIT == 4)
             fx_quarter(u, eb, sp, b, c, a.cfix, f);
         else
