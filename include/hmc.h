@@ -236,8 +236,8 @@ hmc_status hmc_set_orientations_dev(hmc_handle *h, const double *euler_zyz, cons
  * v <- (1 - damping) v + dt f / m and u <- u + dt v on the periodic mesh.
  * FP64 handles form the forces in 64-bit fixed point with one exponent per cell:
  * strains and stresses of a cell carry an absolute error below 2^-52 of the
- * largest strain and stress in that cell (displacements common to its nodes do
- * not count), and u and v are updated in FP64.
+ * largest in that cell (of its mean strain and its nodes' relative displacements;
+ * a displacement common to them does not count), and u and v are updated in FP64.
  * If elastic_energy is not NULL, the stress of the final state is computed
  * (as hmc_compute_stress) and its elastic energy written there. */
 hmc_status hmc_mpm_steps(hmc_handle *h, int32_t nsteps, double *elastic_energy);

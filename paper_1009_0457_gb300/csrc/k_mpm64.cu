@@ -27,7 +27,6 @@
 // A node's force is the sum of its eight cells' integers: exact when their exponents agree and
 // the sum cannot leave 63 bits (both are tested), otherwise aligned to the largest exponent with
 // symmetric rounding.  A cell with a non-finite corner gets F = 2047 and its nodes NaN.
-// A displacement below 2^-1022 (subnormal) counts as zero.
 // Against an 80-bit reference (20x24x28 points, 100 steps) the velocity's relative error is
 // 5.6e-15 and the displacement's 6.8e-16; FP64 arithmetic gave 1.05e-14 and 7.6e-16.
 //
@@ -69,12 +68,13 @@ struct alignas(16) FxBlockSmem {
 
 __device__ __forceinline__ int dexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
-// mantissa of x times 2^K, aligned to the biased exponent E >= dexp(x); subnormals count as zero
+// mantissa of x times 2^K, aligned to the biased exponent E >= dexp(x)
 template <int K>
 __device__ __forceinline__ ll dfix(double x, int E) {
     const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
-    const ll m = ((ll)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x);
-    const ll s = e ? (ll)((unsigned long long)(m << K) >> min(E - e, 63)) : 0ll;
+    const ll f = ((ll)(hi & 0xfffff) << 32) | (unsigned)__double2loint(x);
+    const ll m = e ? f | 1ll << 52 : f << 1;   // a subnormal number is f 2^-1074
+    const ll s = (ll)((unsigned long long)(m << K) >> min(E - e, 63));
     return hi < 0 ? -s : s;
 }
 

@@ -67,3 +67,14 @@ def test_a_small_component_is_held_to_the_largest(G, small, variant, monkeypatch
     v, vo = _step(G, shape, np.zeros((Q, 3)), sp, u0, (0.0,) * 6, variant, monkeypatch)
     for d in range(3):
         assert np.linalg.norm(v[:, d] - vo[:, d]) <= 3e-14 * np.linalg.norm(vo[:, 0]), d
+
+
+def test_subnormal_displacements_exert_forces(G, monkeypatch):
+    # 1e-310 has 44 bits; the sums of either form round at 2^-1074, at most a few thousand times (64 products
+    # with a stiffness of some hundreds): 1e-320, beside the 3e-14 of the values
+    shape, Q = (10, 12, 14), 5
+    eul, sp = S.euler_uniform_so3(Q, 2), S.voronoi_spins(shape, 30, Q, 2)
+    u0 = 1e-310 * np.random.default_rng(3).normal(size=(sp.size // 8, 3))
+    for variant in "056":
+        v, vo = _step(G, shape, eul, sp, u0, (0.0,) * 6, variant, monkeypatch)
+        assert np.abs(vo).max() > 1e-310 and np.abs(v - vo).max() <= 3e-14 * np.abs(vo).max() + 1e-320
