@@ -759,9 +759,9 @@ std::string tune_signature(const hmc_handle *h) {
 
 // Pick the MPM patch shape and persistent-grid size by timing every candidate
 // on scratch copies of the nodal state (the simulation state is not touched).
-// Every candidate computes bit-identical results: the per-cell arithmetic
-// (explicitly rounded, in one order, paired or not) and the order of each
-// node's force sum do not depend on the variant.
+// Every candidate computes bit-identical results: the per-cell arithmetic (explicitly
+// rounded in one order, or in integers) and the order of each node's force sum do not
+// depend on the variant.
 hmc_status tune_mpm(hmc_handle *h, bool enabled, int &best_limit) {
     hmc_status s = HMC_OK;
     int best_variant = 0;

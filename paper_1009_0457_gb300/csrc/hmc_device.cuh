@@ -227,8 +227,7 @@ __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // Row i of sigma = C e: C_i0 e0, then C_ij e_j added by fused multiply-adds in
-// j order (the order of the paired-FMA variant of the MPM step, which is
-// therefore bit-identical).
+// j order.
 template <typename T>
 __device__ __forceinline__ T hooke_row(T c0, T c1, T c2, T c3, T c4, T c5, const T (&e)[6]) {
     T s = rmul(c0, e[0]);
