@@ -8,12 +8,14 @@
 // only the node update (v, u) stays in FP64.
 //
 // Numbers.  A node's displacement is held as one integer m * 2^3 (m the 53-bit mantissa) and one exponent per
-// component.  A cell aligns each component's eight values to the largest exponent among them and takes
-// the differences against its lowest corner, so that a displacement that all corners share costs nothing;
-// what the alignment drops is below 2^-55 of the component's largest value where its exponents differ, and
-// the differences are then of that size.  The cell's exponent F is the smallest at which all differences of all
-// components stay below 2^56, and at least the mean strain's; each component is shifted to F, up
-// exactly or down to the nearest.  The gradients (16 x interpolated differences) and the strains (two
+// component.  Where no displacement of a cell exceeds the mean strain's exponent (most cells of a loaded
+// body), the cell's exponent F is the mean strain's and the values are shifted to it.  Elsewhere a cell
+// aligns each component's eight values to the largest exponent among them and takes the differences
+// against its lowest corner, so that a displacement that all corners share costs nothing; what the alignment drops
+// is below 2^-55 of the component's largest value where its exponents differ, and the differences are then
+// of that size.  F is the smallest exponent, from the mean strain's on, at which all differences of all components
+// stay below 2^56; a component above it is represented by its differences, shifted up exactly, one below it is
+// shifted down.  The gradients (16 x interpolated differences) and the strains (two
 // gradient entries and the mean strain) are exact integer sums below 2^62.6; strains are taken / 8 (< 2^59.6)
 // and split into signed 32-bit halves.  The stiffness is held as integers C 2^cexp with row sums below 2^63,
 // split the same way; sigma = round(C e / 2^64) drops only the product of the two low halves
@@ -28,15 +30,15 @@
 // the sum cannot leave 63 bits (both are tested), otherwise aligned to the largest exponent with
 // symmetric rounding.  A cell with a non-finite corner gets F = 2047 and its nodes NaN.
 // Against an 80-bit reference (20x24x28 points, 100 steps) the velocity's relative error is
-// 5.6e-15 and the displacement's 6.8e-16; FP64 arithmetic gave 1.05e-14 and 7.6e-16.
+// 5.6e-15 and the displacement's 6.7e-16; FP64 arithmetic gave 1.05e-14 and 7.6e-16.
 //
 // Tiling, scheduling and the march in z are those of the FP32 step (k_mpm.cu); nodes and forces
 // are kept in shared memory as two arrays of 16-byte halves, (x, y) and (z, exponents), so that
 // consecutive lanes read consecutive 16 bytes.  The forces are double-buffered, which leaves one
 // barrier per plane.
-// What bounds it: 246 registers leave eight warps per SM, which issue 36 % of the cycles (the
+// What bounds it: 250 registers leave eight warps per SM, which issue 36 % of the cycles (the
 // busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
-// 32^3 8.2 (70), 100^3 50 (308), 128^3 98 (420), 256^3 681 (3330).
+// 32^3 7.7 (70), 100^3 51 (308), 128^3 99 (420), 256^3 676 (3330).
 #include "hmc_device.cuh"
 #include "hmc_fixed.h"
 
@@ -363,9 +365,11 @@ __device__ __forceinline__ void fx_mean_warp(FxMean &m, const DevState *st) {
 }
 
 // a cell: its corners lie at n0 and n1 (lower and upper plane; for a quarter near and far), dy apart in
-// y; u becomes their displacements against the cell's lowest corner's (ref: its place among them) at the
-// cell's exponent, which is returned.  (That corner's zeros spare the march more than the differences and
-// the components' own exponents cost: with one exponent and no differences 256^3 took 707 us, now 681.)
+// y; u becomes their displacements at the cell's exponent, which is returned, all eight of a component
+// together against the cell's lowest corner's (ref: its place among them) where that keeps bits.  Against one
+// exponent for the displacements of all components, a Monte Carlo run's state takes 2 % longer for it (32^3 7.55 ->
+// 7.7 us, 100^3 47.4 -> 48.4; with the differences formed in every cell 8.3 and 50.3), while states whose displacements pass
+// the mean strain gain, because fewer cells differ in exponent (256^3 707 -> 676).
 __device__ __forceinline__ int fx_corners(const FxHalf *xy0, const FxHalf *ze0, const FxHalf *xy1, const FxHalf *ze1,
                                           int dy, int ref, const FxMean &m, ll (&u)[8][3], ll (&eb)[6]) {
     unsigned exy[8], ez[8], mxy = 0, mz = 0;
@@ -381,33 +385,49 @@ __device__ __forceinline__ int fx_corners(const FxHalf *xy0, const FxHalf *ze0, 
         mxy = __vmaxu2(mxy, exy[n]);
         mz = max(mz, ez[n]);
     }
-#pragma unroll
-    for (int n = 0; n < 8; ++n) {
-        const unsigned t = __vminu2(mxy - exy[n], 0x003f003fu);
-        u[n][0] >>= t & 0xffffu;
-        u[n][1] >>= t >> 16;
-        u[n][2] >>= min(mz - ez[n], 63u);
-    }
-    const int E[3] = {(int)(mxy & 0xffffu), (int)(mxy >> 16), (int)mz};
+    const int E[3] = {(int)(mxy & 0xffffu), (int)(mxy >> 16), (int)mz}, top = max(max(E[0], E[1]), E[2]);
     int F = m.e;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const ll lo = ref & 2 ? u[2][d] : u[0][d], hi = ref & 2 ? u[6][d] : u[4][d], r = ref & 4 ? hi : lo;
-        ll any = 0;
+    if (top <= F) {
+        const unsigned f2 = (unsigned)F | (unsigned)F << 16;
 #pragma unroll
         for (int n = 0; n < 8; ++n) {
-            u[n][d] -= r;
-            any |= u[n][d] ^ (u[n][d] >> 63);
+            const unsigned t = __vminu2(f2 - exy[n], 0x003f003fu);
+            u[n][0] >>= t & 0xffffu;
+            u[n][1] >>= t >> 16;
+            u[n][2] >>= min((unsigned)F - ez[n], 63u);
         }
-        F = max(F, E[d] + 8 - __clzll(any));
-    }
-    if (max(max(E[0], E[1]), E[2]) == 2047) F = 2047;
+    } else {
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const int l = min(max(E[d] - F, 0), 63), r = min(max(F - E[d], 0), 63);
-        const ll half = r > 0 ? 1ll << (r - 1) : 0ll;
+        for (int n = 0; n < 8; ++n) {
+            const unsigned t = __vminu2(mxy - exy[n], 0x003f003fu);
+            u[n][0] >>= t & 0xffffu;
+            u[n][1] >>= t >> 16;
+            u[n][2] >>= min(mz - ez[n], 63u);
+        }
+        ll r[3];   // the lowest corner's
 #pragma unroll
-        for (int n = 0; n < 8; ++n) u[n][d] = (ll)(((unsigned long long)u[n][d] << l) + half) >> r;
+        for (int d = 0; d < 3; ++d) {
+            const ll lo = ref & 2 ? u[2][d] : u[0][d], hi = ref & 2 ? u[6][d] : u[4][d];
+            r[d] = ref & 4 ? hi : lo;
+            ll any = 0;
+#pragma unroll
+            for (int n = 0; n < 8; ++n) {
+                const ll x = u[n][d] - r[d];
+                any |= x ^ (x >> 63);
+            }
+            F = max(F, E[d] + 8 - __clzll(any));
+        }
+        if (top == 2047) F = 2047;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            if (E[d] > F) {
+#pragma unroll
+                for (int n = 0; n < 8; ++n) u[n][d] = (ll)((unsigned long long)(u[n][d] - r[d]) << min(E[d] - F, 63));
+            } else {
+#pragma unroll
+                for (int n = 0; n < 8; ++n) u[n][d] >>= min(F - E[d], 63);
+            }
+        }
     }
     const int se = min(F - m.e, 63);
 #pragma unroll
