@@ -26,9 +26,9 @@
 // stress far below the largest of its cell has that absolute error, not a relative one of its own (FP64
 // keeps one where the stiffness does not couple the components, as in an aligned crystal).  The corner forces are
 // +-X +-Y +-Z of the same integers, so a cell's forces sum to exactly zero whatever was rounded.
-// A node's force is the sum of its eight cells' integers: exact when their exponents agree and
-// the sum cannot leave 63 bits (both are tested), otherwise aligned to the largest exponent with
-// symmetric rounding.  A cell with a non-finite corner gets F = 2047 and its nodes NaN.
+// A node's force is the sum of its eight cells' integers: exact when their exponents agree, or differ by
+// less than the bits that the terms leave free, and the sum cannot leave 63 bits (all tested), otherwise aligned
+// to the largest exponent with symmetric rounding.  A cell with a non-finite corner gets F = 2047 and its nodes NaN.
 // Against an 80-bit reference (20x24x28 points, 100 steps) the velocity's relative error is
 // 5.6e-15 and the displacement's 6.7e-16; FP64 arithmetic gave 1.05e-14 and 7.6e-16.
 //
@@ -38,7 +38,7 @@
 // barrier per plane.
 // What bounds it: 250 registers leave eight warps per SM, which issue 36 % of the cycles (the
 // busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
-// 32^3 7.7 (70), 100^3 51 (308), 128^3 99 (420), 256^3 676 (3330).
+// 32^3 7.7 (70), 100^3 49 (308), 128^3 99 (420), 256^3 675 to 708 (3330).
 #include "hmc_device.cuh"
 #include "hmc_fixed.h"
 
@@ -284,7 +284,9 @@ struct Fx3 {
     int e;
 };
 
-// The sum of N terms x[i] 2^e[i] per direction.  With one exponent it is exact; otherwise the terms
+// The sum of N terms x[i] 2^e[i] per direction.  With one exponent it is exact; with several it is exact at
+// the smallest of them where the terms have the room (they mostly differ by one or two, and rounding
+// every term instead took 256^3 under load along [111] from 708 to 801 us a step).  Otherwise the terms
 // are aligned to the largest exponent, and three bits above it where the sum would leave 63 bits.
 template <int N>
 __device__ __forceinline__ Fx3 fx_sum(const ll (&x)[3][N], const int (&e)[N]) {
@@ -310,6 +312,28 @@ __device__ __forceinline__ Fx3 fx_sum(const ll (&x)[3][N], const int (&e)[N]) {
     }
     if (!plain && r.e < 2047) {
         const int top = r.e;
+        int low = e[0];
+        unsigned any = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            low = min(low, e[i]);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int h = (int)(x[d][i] >> 32);
+                any |= (unsigned)(h ^ (h >> 31));
+            }
+        }
+        if (top - low <= __clz(any) - (N == 4 ? 4 : 3)) {   // then the N terms stay below 2^62 / N
+            r.e = low;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                unsigned long long v = 0;
+#pragma unroll
+                for (int i = 0; i < N; ++i) v += (unsigned long long)x[d][i] << (e[i] - low);
+                r.v[d] = (ll)v;
+            }
+            return r;
+        }
 #pragma unroll 1
         for (int up = 0; up <= 3; up += 3) {
             r.e = top + up;
@@ -367,9 +391,9 @@ __device__ __forceinline__ void fx_mean_warp(FxMean &m, const DevState *st) {
 // a cell: its corners lie at n0 and n1 (lower and upper plane; for a quarter near and far), dy apart in
 // y; u becomes their displacements at the cell's exponent, which is returned, all eight of a component
 // together against the cell's lowest corner's (ref: its place among them) where that keeps bits.  Against one
-// exponent for the displacements of all components, a Monte Carlo run's state takes 2 % longer for it (32^3 7.55 ->
-// 7.7 us, 100^3 47.4 -> 48.4; with the differences formed in every cell 8.3 and 50.3), while states whose displacements pass
-// the mean strain gain, because fewer cells differ in exponent (256^3 707 -> 676).
+// exponent for the displacements of all components this costs a Monte Carlo run's state 2 % (32^3 7.55 ->
+// 7.7 us, 100^3 47.4 -> 48.4; with the differences formed in every cell 8.3 and 50.3); states whose displacements
+// pass the mean strain gain, since fewer cells differ in exponent (256^3 under load along z 696 -> 675).
 __device__ __forceinline__ int fx_corners(const FxHalf *xy0, const FxHalf *ze0, const FxHalf *xy1, const FxHalf *ze1,
                                           int dy, int ref, const FxMean &m, ll (&u)[8][3], ll (&eb)[6]) {
     unsigned exy[8], ez[8], mxy = 0, mz = 0;
