@@ -36,8 +36,8 @@
 // are kept in shared memory as two arrays of 16-byte halves, (x, y) and (z, exponents), so that
 // consecutive lanes read consecutive 16 bytes.  The forces are double-buffered, which leaves one
 // barrier per plane.
-// What bounds it: 250 registers leave eight warps per SM, which issue 36 % of the cycles (the
-// busiest pipe, the multipliers, 41 %).  Measured, us per step against the FP64 form before it:
+// What bounds it: 250 registers leave eight warps per SM, which issue 35 % of the cycles (the
+// busiest pipe, the multipliers, 42 %).  Measured, us per step against the FP64 form before it:
 // 32^3 7.7 (70), 100^3 49 (308), 128^3 99 (420), 256^3 675 to 708 (3330).
 #include "hmc_device.cuh"
 #include "hmc_fixed.h"
